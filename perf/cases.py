@@ -237,7 +237,7 @@ def _stream():
 def _photon_room(case):
     """Photon slots of a job, above what it can emit (a job at full length: up to some hundred per electron)."""
     n, steps = case["n"], case["steps"]
-    if case["family"] == "bunch":
+    if case["family"] in ("bunch", "pic"):
         return 24 * n
     per = {"reflected": 0.08 * steps, "plane": 0.01 * steps, "gauss": 0.02 * steps}[case.get("field", "plane")]
     return int(min(n * max(per, 4.0), 6e7 if n > 30_000 else 4e6))
