@@ -301,6 +301,7 @@ extern "C" pe_status pe_create_tables(const pe_table_params* p, pe_tables** out)
     C.g_last = p->n_E - 1;
     C.s_step = 1.0 / (p->n_s - 1);
     C.ln_k_min = std::log(2.0);
+    C.g_safe = p->gamma_max * (1.0 - 1e-3);
     C.inv_dln_k = p->gamma_max > 2.0 ? (p->n_E - 1) / (std::log(p->gamma_max) - std::log(2.0)) : 0.0;
     const double* cs = &C.eta_min;
     float* cfp = &D.cf.eta_min;
@@ -486,6 +487,10 @@ static void describe_run(const pe_tables* t, const pe_run_params* rp, int64_t n,
     for (int i = 0; i < t->host.p.n_E; ++i) smax = std::max(smax, t->host.sigma[(size_t)iz * t->host.p.n_E + i]);
     d.x_hat = c.K_br * smax;
     c.P_hat = -std::expm1(-d.x_hat);
+    // a passing draw is below floor(P 2^64), so its high word is at most P_hat 2^32 (the margin covers
+    // the step's rounding of P, below 1e-5 relative); 2^32 - 1 rejects nothing
+    const double cap = d.c.P_hat * (1.0 + 1e-4) * 0x1.0p32 + 2.0;
+    d.br_cap = cap < 4294967295.0 ? (uint32_t)cap : 0xFFFFFFFFu;
     d.brems_method = rp->brems_method;
     d.wait = rp->brems_method == PE_BREMS_NULL ? static_cast<uint32_t*>(b->brems_wait) : nullptr;
     d.fk = field_kind(rp->geometry, rp->polarisation, rp->reflect_r > 0);

@@ -34,6 +34,7 @@ struct TabC {
     R eta_last, g_last;                   // n_eta - 1 and n_E - 1 (last row position)
     R s_step;                             // 1 / (n_s - 1)
     R ln_k_min, inv_dln_k;                // Bethe-Heitler rows: k log spaced on [2, gamma_max]
+    R g_safe;                             // gamma below this is below the table's top row whatever log rounds to
 };
 
 // Device view of one table set.  f32 and f64 copies of every table.
@@ -109,6 +110,7 @@ struct RunDevT {
     uint32_t seed_lo, seed_hi;
     int fk;                       // field kind (physics.cuh)
     int brems_method;             // PE_BREMS_DIRECT | PE_BREMS_NULL
+    uint32_t br_cap;              // no brems test of Eq. 4 passes if the draw's high word is above this
     uint32_t* wait;               // null collisions: steps to the next candidate
     double x_hat;                 // null collisions: majorant optical depth per step (both precisions)
     void* grid;                   // 1D PIC: field grid (the run's precision, layout in pe.h)
@@ -137,7 +139,7 @@ inline RunDevT<float> to_float(const RunDevT<double>& d) {
     f.geometry = d.geometry; f.polarisation = d.polarisation;
     f.enable_ncs = d.enable_ncs; f.enable_brems = d.enable_brems; f.box_enable = d.box_enable;
     f.iz = d.iz; f.run_id = d.run_id; f.id0 = d.id0; f.seed_lo = d.seed_lo; f.seed_hi = d.seed_hi;
-    f.fk = d.fk; f.brems_method = d.brems_method; f.wait = d.wait; f.x_hat = d.x_hat;
+    f.fk = d.fk; f.brems_method = d.brems_method; f.br_cap = d.br_cap; f.wait = d.wait; f.x_hat = d.x_hat;
     f.grid = d.grid; f.jacc = d.jacc; f.n_cells = d.n_cells;
     return f;
 }
