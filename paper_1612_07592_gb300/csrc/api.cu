@@ -626,7 +626,7 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
     int block = (cfg && cfg->block > 0) ? cfg->block : 256;
     if (block % 64 || block > 256) return fail(PE_ERR_ARG, "pe_step: block must be 64, 128, 192 or 256");
     int K = (cfg && cfg->steps_per_launch > 0) ? cfg->steps_per_launch : (int)std::min<int64_t>(n_steps, 4096);
-    if (K < 1) K = 1;
+    K = std::min(std::max(K, 1), kMaxLaunchSteps);
     int dev;
     cudaGetDevice(&dev);
     int sms = 0;
@@ -634,6 +634,7 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
     int smem = persistent_smem_bytes(t->dev, prec);
     if (smem > 200 * 1024)
         return fail(PE_ERR_ARG, "pe_step: rate tables (n_eta + n_Z * n_E) too large for shared memory");
+    if (prec == PE_F32) smem = pair_smem_bytes(t->dev);
     for (int fk = 0; fk < kFieldKinds; ++fk) {
         std::vector<int> idx;
         for (int k = 0; k < n_runs; ++k)

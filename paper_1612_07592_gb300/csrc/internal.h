@@ -144,6 +144,9 @@ inline RunDevT<float> to_float(const RunDevT<double>& d) {
     return f;
 }
 
+// Most steps of one launch: the paired kernels count a tile's emissions (two per electron-step at most) in 32 bits.
+constexpr int kMaxLaunchSteps = 1 << 20;
+
 // diagnostics (kernels.cu)
 void launch_electron_spectrum(const RunDev& r, int precision, double e_lo, double e_hi, int n_bins,
                               unsigned long long* out, cudaStream_t s);
@@ -203,7 +206,8 @@ void launch_step_persistent_f32(const TablesDev& t, const BatchDevT<float>& b, i
                                 cudaStream_t s);
 void launch_step_persistent_f64(const TablesDev& t, const BatchDevT<double>& b, int steps, int grid, int block,
                                 cudaStream_t s);
-int persistent_smem_bytes(const TablesDev& t, int precision);
+int persistent_smem_bytes(const TablesDev& t, int precision);   // the FP64 kernels
+int pair_smem_bytes(const TablesDev& t);                          // the paired FP32 kernels
 int default_ctas_per_sm_f32(int fk, int block, int smem, int steps_per_launch);
 // every run of the launch has the paper's setup: NCS on, direct brems, no absorbing box (the FP32
 // kernels then take these flags as compile-time constants)

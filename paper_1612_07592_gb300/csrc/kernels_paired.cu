@@ -14,6 +14,8 @@ namespace pe {
 // of a plane-wave kind use the streaming form of the paired kernel.
 constexpr int kStreamMaxSteps = 4;
 
+int pair_smem_bytes(const TablesDev& t) { return kPairFixedBytes + 4 * (t.n_eta + t.n_Z * t.n_E); }
+
 static bool plane_kind(int fk) { return fk == FK_PLANE_LP || fk == FK_PLANE_CP; }
 static bool use_stream(const BatchDevT<float>& b, int steps, int block) {
     return b.n_runs == 1 && plane_kind(b.runs[0].fk) && steps <= kStreamMaxSteps && block == kStreamTile;
@@ -21,42 +23,46 @@ static bool use_stream(const BatchDevT<float>& b, int steps, int block) {
 // tables, then 16-byte alignment slack and the stage buffers
 static int stream_smem_bytes(int base) { return base + 16 + kStreamStages * kStageBytes; }
 
+// Whether the lanes of a warp wait for one another's emissions: where these are frequent, in the reflected wave (5 %
+// of the particle-steps) and in constant fields when a run's largest bremsstrahlung probability per step
+// reaches 1e-3 (the bunch in Au at dt = T 2.6e-3: 8.2 against 8.7 ms; in Al at dt = T / 10, 1e-5: 0.96 against
+// 0.84 ms); not in the plane wave and the 2D focus (below 1e-3).
+template <int G>
+static bool hold_of(const BatchDevT<float>& b) {
+    if (G == FK_REFL_LP || G == FK_REFL_CP) return true;
+    if (G != FK_CONST) return false;
+    for (int k = 0; k < b.n_runs; ++k)
+        if (!b.runs[k].enable_brems || b.runs[k].c.P_hat < 1e-3f) return false;
+    return true;
+}
+
 // The kernel of a launch, its threads per CTA (block/2: two electrons per thread) and dynamic
 // shared memory: the resident paired kernel, or for the plane wave its streaming form.
+using StepKernel = void (*)(TablesDev, BatchDevT<float>, int);
 template <bool kSingle, int G>
-static const void* kernel_of(const BatchDevT<float>& b, int steps, int block, int base_smem, int& threads, int& smem) {
+static StepKernel kernel_of(const BatchDevT<float>& b, int steps, int block, int base_smem, int& threads, int& smem) {
     smem = base_smem;
     threads = block / 2;
     const bool common = common_flags_f32(b);
     if constexpr (G == FK_PLANE_LP || G == FK_PLANE_CP) {
         if (kSingle && use_stream(b, steps, block)) {
             smem = stream_smem_bytes(base_smem);
-            return common ? (const void*)k_step_pair_stream<G, true> : (const void*)k_step_pair_stream<G, false>;
+            return common ? k_step_pair_stream<G, true> : k_step_pair_stream<G, false>;
         }
     }
-    return common ? (const void*)k_step_pair<kSingle, G, true> : (const void*)k_step_pair<kSingle, G, false>;
+    constexpr bool kMayHold = G == FK_REFL_LP || G == FK_REFL_CP || G == FK_CONST;
+    constexpr bool kMayNot = G != FK_REFL_LP && G != FK_REFL_CP;
+    if (hold_of<G>(b)) return common ? k_step_pair<kSingle, G, true, kMayHold> : k_step_pair<kSingle, G, false, kMayHold>;
+    return common ? k_step_pair<kSingle, G, true, !kMayNot> : k_step_pair<kSingle, G, false, !kMayNot>;
 }
 
 template <bool kSingle, int G>
 static void launch_one(const TablesDev& t, const BatchDevT<float>& b, int steps, int grid, int block, cudaStream_t s,
                        int base_smem) {
     int threads, smem;
-    const void* f = kernel_of<kSingle, G>(b, steps, block, base_smem, threads, smem);
+    const StepKernel f = kernel_of<kSingle, G>(b, steps, block, base_smem, threads, smem);
     if (smem > 48 * 1024) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if constexpr (G == FK_PLANE_LP || G == FK_PLANE_CP) {
-        if (f == (const void*)k_step_pair_stream<G, true>) {
-            k_step_pair_stream<G, true><<<grid, threads, smem, s>>>(t, b, steps);
-            return;
-        }
-        if (f == (const void*)k_step_pair_stream<G, false>) {
-            k_step_pair_stream<G, false><<<grid, threads, smem, s>>>(t, b, steps);
-            return;
-        }
-    }
-    if (f == (const void*)k_step_pair<kSingle, G, true>)
-        k_step_pair<kSingle, G, true><<<grid, threads, smem, s>>>(t, b, steps);
-    else
-        k_step_pair<kSingle, G, false><<<grid, threads, smem, s>>>(t, b, steps);
+    f<<<grid, threads, smem, s>>>(t, b, steps);
 }
 
 template <typename F>
@@ -74,7 +80,7 @@ static void with_paired_kind(int fk, F&& f) {
 
 void launch_step_persistent_f32(const TablesDev& t, const BatchDevT<float>& b, int steps, int grid, int block,
                                 cudaStream_t s) {
-    const int smem = persistent_smem_bytes(t, PE_F32);
+    const int smem = pair_smem_bytes(t);
     with_paired_kind(b.runs[0].fk, [&](auto g) {
         if (b.n_runs == 1) launch_one<true, decltype(g)::value>(t, b, steps, grid, block, s, smem);
         else launch_one<false, decltype(g)::value>(t, b, steps, grid, block, s, smem);
@@ -88,8 +94,8 @@ const void* persistent_kernel_f32(const BatchDevT<float>& b, int steps, int base
     const void* f = nullptr;
     int th = block, smem = base_smem;
     with_paired_kind(b.runs[0].fk, [&](auto g) {
-        f = b.n_runs == 1 ? kernel_of<true, decltype(g)::value>(b, steps, block, base_smem, th, smem)
-                          : kernel_of<false, decltype(g)::value>(b, steps, block, base_smem, th, smem);
+        f = (const void*)(b.n_runs == 1 ? kernel_of<true, decltype(g)::value>(b, steps, block, base_smem, th, smem)
+                                        : kernel_of<false, decltype(g)::value>(b, steps, block, base_smem, th, smem));
     });
     if (smem > 48 * 1024) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     *threads = th;
@@ -110,8 +116,9 @@ int default_ctas_per_sm_f32(int fk, int block, int smem, int steps_per_launch) {
         return e == cudaSuccess && occ > 0 ? occ : 1;
     }
     with_paired_kind(fk, [&](auto g) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step_pair<true, decltype(g)::value, true>, block / 2,
-                                                          smem);
+        constexpr int G = decltype(g)::value;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &occ, k_step_pair<true, G, true, G == FK_REFL_LP || G == FK_REFL_CP>, block / 2, smem);
     });
     return 3 * (e == cudaSuccess && occ > 0 ? occ : 1);
 }

@@ -131,11 +131,11 @@ __device__ __forceinline__ void envelope2(const StepC<float>& c, float2 phi, flo
     dg = make_float2(copysignf(kts.x, side.x), copysignf(kts.y, side.y));
 }
 
-// two electrons; per-electron activity, optical-depth pairs and event fingerprints
+// two electrons; per-electron activity and optical-depth pairs.  The event fingerprints stay in memory: an
+// emission adds to its electron's word there (add_events).
 struct Pair {
     float2 x, x_lo, u0, u1, u2, tau, tau_lo;
     float2 y, y_lo;                     // 2D focus only (zero and unused in 1D)
-    uint32_t ev_cnt[2], ev_hash[2];
     uint32_t wait[2];
     bool act[2];
 };
@@ -146,9 +146,9 @@ __device__ __forceinline__ Particle<float> unpack(const Pair& Q, int k) {
     P.y = comp(Q.y, k); P.y_lo = comp(Q.y_lo, k);
     P.u[0] = comp(Q.u0, k); P.u[1] = comp(Q.u1, k); P.u[2] = comp(Q.u2, k);
     P.tau = comp(Q.tau, k); P.tau_lo = comp(Q.tau_lo, k);
-    // selects, not Q.ev_cnt[k]: an index unknown at compile time (the reflected wave's emission
-    // loop) would move the arrays to local memory
-    P.ev_cnt = k ? Q.ev_cnt[1] : Q.ev_cnt[0]; P.ev_hash = k ? Q.ev_hash[1] : Q.ev_hash[0];
+    P.ev_cnt = P.ev_hash = 0;
+    // a select, not Q.wait[k]: an index unknown at compile time (the emission loops) would move the
+    // array to local memory
     P.wait = k ? Q.wait[1] : Q.wait[0];
     return P;
 }
@@ -157,25 +157,41 @@ __device__ __forceinline__ void repack(Pair& Q, int k, const Particle<float>& P)
     set_comp(Q.y, k, P.y); set_comp(Q.y_lo, k, P.y_lo);
     set_comp(Q.u0, k, P.u[0]); set_comp(Q.u1, k, P.u[1]); set_comp(Q.u2, k, P.u[2]);
     set_comp(Q.tau, k, P.tau); set_comp(Q.tau_lo, k, P.tau_lo);
-    if (k) { Q.ev_cnt[1] = P.ev_cnt; Q.ev_hash[1] = P.ev_hash; Q.wait[1] = P.wait; }
-    else { Q.ev_cnt[0] = P.ev_cnt; Q.ev_hash[0] = P.ev_hash; Q.wait[0] = P.wait; }
+    if (k) Q.wait[1] = P.wait; else Q.wait[0] = P.wait;
+}
+// an emission's fingerprint into electron id's word (its thread alone has the electron)
+__device__ __forceinline__ void add_events(const RunDevT<float>& r, uint32_t id, const Particle<float>& P) {
+    if (!r.events) return;
+    unsigned long long* w = r.events + (uint32_t)(id - r.id0);
+    const unsigned long long e = *w;
+    *w = ((unsigned long long)((uint32_t)(e >> 32) + P.ev_hash) << 32) | ((uint32_t)e + P.ev_cnt);
+}
+// state back to memory without the event word
+__device__ __forceinline__ void store_one(const RunDevT<float>& r, int64_t i, const Particle<float>& P) {
+    store_pos(r, i, P);
+    ((float*)r.ux)[i] = P.u[0];
+    ((float*)r.uy)[i] = P.u[1];
+    ((float*)r.uz)[i] = P.u[2];
+    store_tau(r, i, P);
+    if (r.wait) r.wait[i] = P.wait;
 }
 
-// one step of two electrons (G = FK_PLANE_LP, FK_PLANE_CP: the 1D plane wave; FK_REFL_LP,
-// FK_REFL_CP: the plane wave and its mirror image; FK_GAUSS_LP, FK_GAUSS_CP: the 2D paraxial focus;
-// FK_CONST: constant fields).  An inactive half of the pair (a removed electron, or an
-// empty slot past the end of the run) has x = NaN, so its fields, momenta, eta and optical depth
-// are NaN from its first step on, and the eta count, the optical depth's crossing and the target
-// test are false for it without reading the activity flags.  kCommon: the run has NCS on, direct brems and no
-// absorbing box (the paper's setup), known at compile time, so the step carries no test of the
-// run's flags; otherwise they are read from the run.
+// The first half of a step of two electrons: fields at (x^n, t^n), Boris push, gamma, and with NCS on eta, the
+// rate and the optical depth.  Returns a bit per electron whose optical depth crossed zero (it emits).
+// G = FK_PLANE_LP, FK_PLANE_CP: the 1D plane wave; FK_REFL_LP, FK_REFL_CP: the plane wave and its mirror
+// image; FK_GAUSS_LP, FK_GAUSS_CP: the 2D paraxial focus; FK_CONST: constant fields.  An inactive half of
+// the pair (a removed electron, or an empty slot past the end of the run) has x = NaN, so its fields, momenta,
+// eta and optical depth are NaN from its first step on, and the eta count, the optical depth's crossing and the
+// target test are false for it without reading the activity flags.  kCommon: the run has NCS on, direct brems
+// and no absorbing box (the paper's setup), known at compile time, so the step carries no test of the run's
+// flags; otherwise they are read from the run.
 template <int G, bool kCommon>
-__device__ __forceinline__ void step_pair(const TablesDev& t, const RunDevT<float>& r, const float* h_tab,
-                                          const float* sig_tab, const uint32_t id[2], uint32_t n, float nf, Pair& Q,
-                                          unsigned long long* hist, unsigned long long* tally, float2& n_above) {
+__device__ __forceinline__ unsigned push_pair(const TablesDev& t, const RunDevT<float>& r, const float* h_tab,
+                                              float nf, Pair& Q, float2& gamma, float2& inv_g, float2& eta,
+                                              float2& n_above) {
     const StepC<float>& c = r.c;
     const TabC<float>& tc = t.cf;
-    const float2 dt = P2(c.dt), h = P2(0.5f * c.dt);
+    const float2 h = P2(0.5f * c.dt);
     // fields at (x^n, t^n): phase, envelope, carrier
     const float2 nf2 = P2(nf);
     float2 phi = fma2(nf2, P2(c.dt_lo), sub2(mul2(nf2, P2(c.dt_hi)), Q.x));
@@ -185,7 +201,6 @@ __device__ __forceinline__ void step_pair(const TablesDev& t, const RunDevT<floa
     constexpr bool kPlane = G == FK_PLANE_LP || G == FK_PLANE_CP;
     constexpr bool kRefl = G == FK_REFL_LP || G == FK_REFL_CP;
     constexpr bool kConst = G == FK_CONST;
-    constexpr bool kOneD = kPlane || kRefl || kConst;   // no transverse position
     constexpr bool kCP = G == FK_PLANE_CP || G == FK_GAUSS_CP || G == FK_REFL_CP;
     float2 by = P2(0.0f), bz = P2(0.0f);                // B_y, B_z of the reflected kinds
     const float2 ma0 = P2(-c.a0);
@@ -347,17 +362,14 @@ __device__ __forceinline__ void step_pair(const TablesDev& t, const RunDevT<floa
     // gamma and 1/gamma from one reciprocal square root (1/gamma serves the rate and the
     // position update; emitting lanes refresh it from their new gamma)
     const float2 g2 = fma2(Q.u2, Q.u2, fma2(Q.u1, Q.u1, fma2(Q.u0, Q.u0, P2(1.0f))));
-    float2 inv_g = rsqrt2(g2);
-    float2 gamma = mul2(g2, inv_g);
-    const float2 xn = Q.x, yn = Q.y;
-    float gam[2] = {gamma.x, gamma.y};
-
+    inv_g = rsqrt2(g2);
+    gamma = mul2(g2, inv_g);
+    unsigned crossed = 0;
     if (kCommon || r.enable_ncs) {
         // eta = (gamma - u_x) |E| / E_S for the plane wave; ngm = u_x - gamma, for u_x > 0 as
         // -(1 + u_y^2 + u_z^2) / (gamma + u_x) (no cancellation), its sign taken by the last factor
         float2 up = fma2(Q.u2, Q.u2, fma2(Q.u1, Q.u1, P2(1.0f)));
         float2 ngm = sel2(Q.u0.x > 0.0f, Q.u0.y > 0.0f, mul2(up, nrcp2(add2(gamma, Q.u0))), sub2(Q.u0, gamma));
-        float2 eta;
         if constexpr (kPlane) {
             float2 Emag = (G == FK_PLANE_CP) ? sqrt2(fma2(ez, ez, mul2(ey, ey))) : make_float2(fabsf(ey.x), fabsf(ey.y));
             eta = mul2(mul2(ngm, Emag), P2(-c.inv_ES));
@@ -421,154 +433,162 @@ __device__ __forceinline__ void step_pair(const TablesDev& t, const RunDevT<floa
         Q.tau = s;
         Q.tau_lo = add2(Q.tau_lo, e);
         float2 tsum = add2(Q.tau, Q.tau_lo);
-        if (kRefl && (tsum.x <= 0.0f || tsum.y <= 0.0f)) {
-            // frequent emissions (about 4 % of the particle-steps in the reflected pulse): the crossings
-            // of a lane go one at a time through one inlined branch, so lanes whose crossing is in
-            // different halves of their pairs take it together
-            unsigned m = (unsigned)(tsum.x <= 0.0f) | ((unsigned)(tsum.y <= 0.0f) << 1);
-            while (m) {
-                const int k = (m & 1u) ? 0 : 1;
-                m &= m - 1u;
-                Particle<float> P = unpack(Q, k);
-                float gk = k ? gam[1] : gam[0];
-                bool st;
-                Photon ph;
-                take(ncs_emit_body<float>(t, r, k ? id[1] : id[0], n, P, gk, comp(eta, k), comp(xn, k), 0.0f, hist,
-                                          tally),
-                     P, gk, st, ph);
-                if (st) append_now(r, ph);
-                repack(Q, k, P);
-                set_comp(inv_g, k, __frcp_rn(gk));
-                if (k) gam[1] = gk; else gam[0] = gk;
-            }
-        } else if (tsum.x <= 0.0f || tsum.y <= 0.0f) {  // one test of the pair on the common path
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                if (comp(tsum, k) <= 0.0f) {
-                    Particle<float> P = unpack(Q, k);
-                    bool st;
-                    Photon ph;
-                    take(ncs_emit_body<float>(t, r, id[k], n, P, gam[k], comp(eta, k), comp(xn, k), comp(yn, k), hist,
-                                              tally),
-                         P, gam[k], st, ph);
-                    if (st) append_now(r, ph);
-                    repack(Q, k, P);
-                    // 1/gamma by the correctly rounded reciprocal: with the branch inlined, a plain
-                    // division of its sqrt result is open to per-kernel rewriting (1/sqrt as rsqrt),
-                    // and every paired kernel must round it alike
-                    set_comp(inv_g, k, __frcp_rn(gam[k]));
-                }
-            }
-        }
+        crossed = (unsigned)(tsum.x <= 0.0f) | ((unsigned)(tsum.y <= 0.0f) << 1);
     }
+    return crossed;
+}
 
-    if (kCommon || r.enable_brems) {
-        if (!kCommon && r.brems_method == PE_BREMS_NULL) {
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                if (!Q.act[k]) continue;
-                if (Q.wait[k] == 0u) {
-                    const float x = comp(xn, k);
-                    Particle<float> P = unpack(Q, k);
-                    bool st;
-                    Photon ph;
-                    const bool in_slab = x >= c.x0 && x <= c.x1 && (kOneD || fabsf(comp(yn, k)) <= c.yh);
-                    take(brems_candidate<float>(t, r, sig_tab, id[k], n, P, gam[k], in_slab, x, comp(yn, k), hist,
-                                                tally),
-                         P, gam[k], st, ph);
-                    if (st) append_now(r, ph);
-                    repack(Q, k, P);
-                    set_comp(inv_g, k, __frcp_rn(gam[k]));
-                } else if (Q.wait[k] != PE_WAIT_NEVER) {
-                    --Q.wait[k];
-                }
-            }
-        } else {
-            // Eq. 4.  Almost every test fails, and the draw alone shows it: a passing draw has its high word
-            // at most the run's largest probability (br_cap), so the first thing formed is that one word of
-            // the draw, and the rate, the probability and the rest of the draw only for an electron whose
-            // word is that low (or whose gamma may be above the table, which is counted).  Philox bounds the
-            // test in the target; with the rate and the probability formed for every electron there, 6e6
-            // electrons one step per call took 120 us a step and now take 92, the 1 GeV Au bunch (5e5
-            // electrons, 2000 steps) 10.9 ms and now 9.9 (its emissions are what is left), the 1e6 x 4000
-            // job, in the target for a tenth of its steps, 19.6 and now 19.1 ms.
-            bool in[2];
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const float x = comp(xn, k);
-                in[k] = x >= c.x0 && x <= c.x1 && (kOneD || fabsf(comp(yn, k)) <= c.yh) &&
-                        gam[k] > 1.0f + tc.photon_min;
-            }
-            if (in[0] || in[1]) {
-                const uint32_t hi0 = draw(r, id[0], n, PUR_BREMS).y, hi1 = draw(r, id[1], n, PUR_BREMS).y;
-                in[0] = in[0] && (hi0 <= r.br_cap || gam[0] >= tc.g_safe);
-                in[1] = in[1] && (hi1 <= r.br_cap || gam[1] >= tc.g_safe);
-            }
-            if (in[0] || in[1]) {
-                // x_b = K sigma_Z(gamma) beta on the paired instructions (row position in log gamma from log2 by
-                // one FMA, clamped below the top node as for h(eta); beta = |u| / gamma), then per electron the
-                // whole draw and the integer test
-                const float2 gv = make_float2(gam[0], gam[1]);
-                const float2 tg = fma2(log2v(gv), P2(tc.inv_dln_g * 0.693147180559945309f),
-                                       P2(-tc.ln_g_min * tc.inv_dln_g));
-#pragma unroll
-                for (int k = 0; k < 2; ++k)
-                    if (in[k] && comp(tg, k) >= tc.g_last) atomicAdd(tally + PE_T_N_GAMMA_ABOVE, 1ull);
-                const float2 tgc = clamp2(tg, 0.0f, tc.g_last - 0x1.0p-10f);
-                const float2 tt = add2(sub2(tgc, P2(0.5f)), P2(0x1.8p23f));
-                const int gx = dbg_idx(t.dbg, __float_as_int(tt.x) - 0x4B400000, t.n_E - 1);
-                const int gy = dbg_idx(t.dbg, __float_as_int(tt.y) - 0x4B400000, t.n_E - 1);
-                const float2 w = sub2(tgc, sub2(tt, P2(0x1.8p23f)));
-                const float2 s0 = make_float2(sig_tab[gx], sig_tab[gy]);
-                const float2 s1 = make_float2(sig_tab[gx + 1], sig_tab[gy + 1]);
-                const float2 sig = fma2(w, sub2(s1, s0), s0);
-                const float2 um = sqrt2(fma2(Q.u2, Q.u2, fma2(Q.u1, Q.u1, mul2(Q.u0, Q.u0))));
-                const float2 xb = mul2(mul2(P2(c.K_br), sig), mul2(um, inv_g));
-                // 1 - e^{-x_b} by its Taylor series below 2^-5 (truncation under 2^-26 relative), the
-                // library expm1f above: one_minus_exp_neg_f32 on the paired instructions
-                const float2 ser = brems_series2(xb);
-                float pb_[2] = {ser.x, ser.y};
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    if (!in[k]) continue;
-                    if (!(comp(xb, k) < 0x1.0p-5f)) pb_[k] = -expm1f(-comp(xb, k));
-                    uint32_t idk = id[k];
-                    asm volatile("" : "+r"(idk));       // formed again here, not carried from the test above
-                    const uint4 wd = draw(r, idk, n, PUR_BREMS);
-                    if (brems_event(pb_[k], wd)) {
-                        Particle<float> P = unpack(Q, k);
-                        bool st;
-                        Photon ph;
-                        take(brems_emit_body<float>(t, r, id[k], n, P, gam[k], comp(xn, k), comp(yn, k), wd, hist, tally), P,
-                             gam[k], st, ph);
-                        if (st) append_now(r, ph);
-                        repack(Q, k, P);
-                        set_comp(inv_g, k, __frcp_rn(gam[k]));
-                    }
-                }
-            }
-        }
-    }
-
-    // x^{n+1} = x^n + dt u_x / gamma, compensated
-    float2 d = mul2(mul2(dt, Q.u0), inv_g);
-    float2 s, e;
-    two_sum2(Q.x, d, s, e);
-    Q.x = s;
-    Q.x_lo = add2(Q.x_lo, e);
-    if constexpr (!kOneD) {                             // y^{n+1} = y^n + dt u_y / gamma, compensated
-        two_sum2(Q.y, mul2(mul2(dt, Q.u1), inv_g), s, e);
-        Q.y = s;
-        Q.y_lo = add2(Q.y_lo, e);
-    }
-    if (!kCommon && r.box_enable) {
+// The bremsstrahlung test of Eq. 4 of the pair after its NCS emissions (or the null-collision waits): a bit per
+// electron with a collision to sample (a candidate, for null collisions).
+template <int G, bool kCommon>
+__device__ __forceinline__ unsigned brems_pair(const TablesDev& t, const RunDevT<float>& r, const float* sig_tab,
+                                               const uint32_t id[2], uint32_t n, Pair& Q, float2 gamma, float2 inv_g,
+                                               const SumsCta& acc) {
+    constexpr bool kOneD = G != FK_GAUSS_LP && G != FK_GAUSS_CP;
+    const StepC<float>& c = r.c;
+    const TabC<float>& tc = t.cf;
+    unsigned hit = 0;
+    if (!kCommon && r.brems_method == PE_BREMS_NULL) {
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             if (!Q.act[k]) continue;
-            Particle<float> P = unpack(Q, k);
-            box_check<float>(r, P, n, tally);
-            repack(Q, k, P);
+            if (Q.wait[k] == 0u) hit |= 1u << k;
+            else if (Q.wait[k] != PE_WAIT_NEVER) --Q.wait[k];
         }
+        return hit;
+    }
+    // Almost every test fails, and the draw alone shows it: a passing draw has its high word at most the
+    // run's largest probability (br_cap), so the first thing formed is that one word of the draw, and the
+    // rate, the probability and the rest of the draw only for an electron whose word is that low (or whose
+    // gamma may be above the table, which is counted).  Philox bounds the test in the target; with the rate
+    // and the probability formed for every electron there, 6e6 electrons one step per call took 120 us a
+    // step and then 92, the 1 GeV Au bunch (5e5 electrons, 2000 steps) 10.9 ms and then 9.9, the 1e6 x 4000
+    // job, in the target for a tenth of its steps, 19.6 and then 19.1 ms.
+    bool in[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const float x = comp(Q.x, k);
+        in[k] = x >= c.x0 && x <= c.x1 && (kOneD || fabsf(comp(Q.y, k)) <= c.yh) &&
+                comp(gamma, k) > 1.0f + tc.photon_min;
+    }
+    if (in[0] || in[1]) {
+        const uint32_t hi0 = draw(r, id[0], n, PUR_BREMS).y, hi1 = draw(r, id[1], n, PUR_BREMS).y;
+        in[0] = in[0] && (hi0 <= r.br_cap || gamma.x >= tc.g_safe);
+        in[1] = in[1] && (hi1 <= r.br_cap || gamma.y >= tc.g_safe);
+    }
+    if (in[0] || in[1]) {
+        // x_b = K sigma_Z(gamma) beta on the paired instructions (row position in log gamma from log2 by
+        // one FMA, clamped below the top node as for h(eta); beta = |u| / gamma), then per electron the
+        // whole draw and the integer test
+        const float2 tg = fma2(log2v(gamma), P2(tc.inv_dln_g * 0.693147180559945309f),
+                               P2(-tc.ln_g_min * tc.inv_dln_g));
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (in[k] && comp(tg, k) >= tc.g_last) acc.count(PE_T_N_GAMMA_ABOVE);
+        const float2 tgc = clamp2(tg, 0.0f, tc.g_last - 0x1.0p-10f);
+        const float2 tt = add2(sub2(tgc, P2(0.5f)), P2(0x1.8p23f));
+        const int gx = dbg_idx(t.dbg, __float_as_int(tt.x) - 0x4B400000, t.n_E - 1);
+        const int gy = dbg_idx(t.dbg, __float_as_int(tt.y) - 0x4B400000, t.n_E - 1);
+        const float2 w = sub2(tgc, sub2(tt, P2(0x1.8p23f)));
+        const float2 s0 = make_float2(sig_tab[gx], sig_tab[gy]);
+        const float2 s1 = make_float2(sig_tab[gx + 1], sig_tab[gy + 1]);
+        const float2 sig = fma2(w, sub2(s1, s0), s0);
+        const float2 um = sqrt2(fma2(Q.u2, Q.u2, fma2(Q.u1, Q.u1, mul2(Q.u0, Q.u0))));
+        const float2 xb = mul2(mul2(P2(c.K_br), sig), mul2(um, inv_g));
+        // 1 - e^{-x_b} by its Taylor series below 2^-5 (truncation under 2^-26 relative), the
+        // library expm1f above: one_minus_exp_neg_f32 on the paired instructions
+        const float2 ser = brems_series2(xb);
+        float pb_[2] = {ser.x, ser.y};
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (!in[k]) continue;
+            if (!(comp(xb, k) < 0x1.0p-5f)) pb_[k] = -expm1f(-comp(xb, k));
+            uint32_t idk = id[k];
+            asm volatile("" : "+r"(idk));               // formed again here, not carried from the test above
+            const uint4 wd = draw(r, idk, n, PUR_BREMS);
+            if (brems_event(pb_[k], wd)) hit |= 1u << k;
+        }
+    }
+    return hit;
+}
+
+// A thread's emission state while it waits (see pair_loop), in shared memory: eta and gamma of its step and 1/gamma
+struct Held {
+    float2 *eta, *gamma, *inv_g;
+};
+// its NCS emissions.  One inlined branch that takes the crossings of a lane one at a time, so lanes whose crossing is
+// in different halves of their pairs take it together; or one for each half (kTwoSites), which spares the
+// selects: the single-run kernels of the kinds with rare emissions (2D focus job 16.2 against 16.6 ms; in the
+// batch instances, whose registers spill, 24.9 against 24.5).
+template <int G, bool kTwoSites>
+__device__ __forceinline__ void emit_ncs_pair(const TablesDev& t, const RunDevT<float>& r, const uint32_t id[2],
+                                              uint32_t n, unsigned m, Pair& Q, float2& gamma, float2& inv_g, float2 eta,
+                                              const SumsCta& acc) {
+    auto emit = [&](int k) {
+        Particle<float> P = unpack(Q, k);
+        float gk = comp(gamma, k);
+        const uint32_t idk = k ? id[1] : id[0];
+        bool st;
+        Photon ph;
+        take(ncs_emit_body<float>(t, r, idk, n, P, gk, comp(eta, k), comp(Q.x, k), comp(Q.y, k), acc), P, gk, st, ph);
+        if (st) append_now(r, ph);
+        add_events(r, idk, P);
+        repack(Q, k, P);
+        // 1/gamma by the correctly rounded reciprocal: with the branch inlined, a plain division of its sqrt
+        // result is open to per-kernel rewriting (1/sqrt as rsqrt), and every paired kernel must round it alike
+        set_comp(inv_g, k, __frcp_rn(gk));
+        set_comp(gamma, k, gk);
+    };
+    if constexpr (kTwoSites) {
+        if (m & 1u) emit(0);
+        if (m & 2u) emit(1);
+    } else {
+        while (m) {
+            emit((m & 1u) ? 0 : 1);
+            m &= m - 1u;
+        }
+    }
+}
+// its bremsstrahlung photons, or null-collision candidates
+template <int G, bool kCommon>
+__device__ __forceinline__ void emit_brems_pair(const TablesDev& t, const RunDevT<float>& r, const float* sig_tab,
+                                                const uint32_t id[2], uint32_t n, unsigned m, Pair& Q, float2 gamma,
+                                                float2& inv_g, const SumsCta& acc) {
+    constexpr bool kOneD = G != FK_GAUSS_LP && G != FK_GAUSS_CP;
+    const StepC<float>& c = r.c;
+    while (m) {
+        const int k = (m & 1u) ? 0 : 1;
+        m &= m - 1u;
+        Particle<float> P = unpack(Q, k);
+        float gk = comp(gamma, k);
+        const uint32_t idk = k ? id[1] : id[0];
+        const float x = comp(Q.x, k), y = comp(Q.y, k);
+        bool st;
+        Photon ph;
+        if (!kCommon && r.brems_method == PE_BREMS_NULL) {
+            const bool in_slab = x >= c.x0 && x <= c.x1 && (kOneD || fabsf(y) <= c.yh);
+            take(brems_candidate<float>(t, r, sig_tab, idk, n, P, gk, in_slab, x, y, acc), P, gk, st, ph);
+        } else {
+            take(brems_emit_body<float>(t, r, idk, n, P, gk, x, y, draw(r, idk, n, PUR_BREMS), acc), P, gk, st, ph);
+        }
+        if (st) append_now(r, ph);
+        add_events(r, idk, P);
+        repack(Q, k, P);
+        set_comp(inv_g, k, __frcp_rn(gk));
+    }
+}
+// x^{n+1} = x^n + dt u_x / gamma (and y), compensated
+template <int G>
+__device__ __forceinline__ void move_pair(const StepC<float>& c, Pair& Q, float2 inv_g) {
+    const float2 dt = P2(c.dt);
+    float2 s, e;
+    two_sum2(Q.x, mul2(mul2(dt, Q.u0), inv_g), s, e);
+    Q.x = s;
+    Q.x_lo = add2(Q.x_lo, e);
+    if constexpr (G == FK_GAUSS_LP || G == FK_GAUSS_CP) {
+        two_sum2(Q.y, mul2(mul2(dt, Q.u1), inv_g), s, e);
+        Q.y = s;
+        Q.y_lo = add2(Q.y_lo, e);
     }
 }
 
@@ -580,28 +600,125 @@ __device__ __forceinline__ void load_one(const RunDevT<float>& r, int64_t i, Pai
     repack(Q, k, P);
 }
 
-// K steps of the pair Q (electrons i0 and i1); photons are appended inside the emission branches
-// (append_now), so none is held across the step
-template <int G, bool kCommon>
+// absorbing box (Sec. 3) after a step: a removed electron is stored at once
+__device__ __forceinline__ void box_pair(const RunDevT<float>& r, int64_t i0, int64_t i1, uint32_t n, Pair& Q,
+                                         unsigned long long* s_tally) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        if (!Q.act[k]) continue;
+        Particle<float> P = unpack(Q, k);
+        box_check<float>(r, P, n, s_tally);
+        set_comp(Q.x, k, P.x);
+        if (isnan(P.x)) {
+            Q.act[k] = false;
+            store_one(r, k ? i1 : i0, P);
+        }
+    }
+}
+
+// K steps of the pair Q (electrons i0 and i1), the lanes of a warp in step: an emission is taken where it falls.
+template <int G, bool kCommon, bool kTwoSites>
 __device__ __forceinline__ void pair_loop(const TablesDev& t, const RunDevT<float>& r, const float* s_h,
                                           const float* sig_z, int64_t i0, int64_t i1, Pair& Q, int steps,
-                                          unsigned long long* s_hist, unsigned long long* s_tally) {
+                                          const SumsCta& acc, unsigned long long* s_tally) {
     const uint32_t id[2] = {r.id0 + (uint32_t)i0, r.id0 + (uint32_t)i1};
     const uint32_t n0 = (uint32_t)r.step0;
     float nf = (float)n0;
     float2 n_above = P2(0.0f);                          // particle-steps with eta above the table (exact to 2^24)
     for (int s = 0; s < steps; ++s, nf += 1.0f) {
         if (Q.act[0] || Q.act[1]) {
-            step_pair<G, kCommon>(t, r, s_h, sig_z, id, n0 + (uint32_t)s, nf, Q, s_hist, s_tally, n_above);
-            if (!kCommon && r.box_enable) {
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    if (Q.act[k] && isnan(comp(Q.x, k))) {
-                        Q.act[k] = false;
-                        store_particle<float>(r, k ? i1 : i0, unpack(Q, k));
+            const uint32_t n = n0 + (uint32_t)s;
+            float2 gamma, inv_g, eta;
+            const unsigned crossed = push_pair<G, kCommon>(t, r, s_h, nf, Q, gamma, inv_g, eta, n_above);
+            if (crossed) emit_ncs_pair<G, kTwoSites>(t, r, id, n, crossed, Q, gamma, inv_g, eta, acc);
+            if (kCommon || r.enable_brems) {
+                const unsigned hit = brems_pair<G, kCommon>(t, r, sig_z, id, n, Q, gamma, inv_g, acc);
+                if (hit) emit_brems_pair<G, kCommon>(t, r, sig_z, id, n, hit, Q, gamma, inv_g, acc);
+            }
+            move_pair<G>(r.c, Q, inv_g);
+            if (!kCommon && r.box_enable) box_pair(r, i0, i1, n, Q, s_tally);
+        }
+    }
+    const unsigned int na = __float2uint_rz(n_above.x) + __float2uint_rz(n_above.y);
+    if (na) atomicAdd(s_tally + PE_T_N_ETA_ABOVE, (unsigned long long)na);
+}
+
+// The same with lanes that wait for their emissions.
+//
+// A warp that branches into an emission for one lane issues all of it, several times a step's length, for that lane.
+// The lanes need not be at the same step: electrons are independent and their draws keyed on (electron, step).  So a
+// lane with an emission waits where it is while the others step on, until the lane-steps lost by waiting reach
+// kHoldSteps or no lane can step; then the waiting lanes emit together.  Measured with thresholds of 16, 24, 32
+// and 64 lane-steps against none: the reflected job 16.2, 15.9, 15.9 and 16.2 against 17.7 ms, the bunch 8.32,
+// 8.28, 8.27 and 8.39 against 8.72.  Where emissions are rare a lane waits long for company and in the end the warp
+// waits for that lane: at 48 lane-steps the 1D job took 22.3 against 20.9 ms (hold_of chooses).
+constexpr int kHoldSteps = 32;
+template <int G, bool kCommon>
+__device__ __forceinline__ void pair_loop_hold(const TablesDev& t, const RunDevT<float>& r, const float* s_h,
+                                               const float* sig_z, int64_t i0, int64_t i1, Pair& Q, int steps,
+                                               const SumsCta& acc, const Held& held_at, unsigned long long* s_tally) {
+    const uint32_t id[2] = {r.id0 + (uint32_t)i0, r.id0 + (uint32_t)i1};
+    uint32_t n = (uint32_t)r.step0;                     // this lane's step
+    float nf = (float)n;
+    int left = (Q.act[0] || Q.act[1]) ? steps : 0;      // and its steps to go
+    float2 n_above = P2(0.0f);
+    unsigned held = 0;                                  // emissions waited for: bits 0, 1 NCS, bits 2, 3 brems
+    int lost = 0;
+    while (true) {
+        const bool run = left > 0 && !held;
+        bool test = false, move = false;
+        float2 gamma, inv_g;
+        if (run) {
+            float2 eta;
+            held = push_pair<G, kCommon>(t, r, s_h, nf, Q, gamma, inv_g, eta, n_above);
+            if (held) {
+                *held_at.eta = eta;
+                *held_at.gamma = gamma;
+                *held_at.inv_g = inv_g;
+            }
+            test = !held;
+        }
+        const unsigned waiting = __ballot_sync(0xffffffffu, held != 0);
+        if (waiting) {
+            lost += __popc(waiting);
+            if (lost >= kHoldSteps || !__any_sync(0xffffffffu, test)) {
+                lost = 0;
+                if (held) {
+                    gamma = *held_at.gamma;
+                    inv_g = *held_at.inv_g;
+                    if (held & 3u) {
+                        emit_ncs_pair<G, false>(t, r, id, n, held, Q, gamma, inv_g, *held_at.eta, acc);
+                        test = true;
+                    } else {
+                        emit_brems_pair<G, kCommon>(t, r, sig_z, id, n, held >> 2, Q, gamma, inv_g, acc);
+                        move = true;
                     }
+                    held = 0;
                 }
             }
+        } else if (!__any_sync(0xffffffffu, test)) {
+            break;                                      // no lane waits and none stepped: all are done
+        }
+        if (test) {
+            move = true;
+            if (kCommon || r.enable_brems) {
+                held = brems_pair<G, kCommon>(t, r, sig_z, id, n, Q, gamma, inv_g, acc) << 2;
+                if (held) {
+                    *held_at.gamma = gamma;
+                    *held_at.inv_g = inv_g;
+                    move = false;
+                }
+            }
+        }
+        if (move) {
+            move_pair<G>(r.c, Q, inv_g);
+            if (!kCommon && r.box_enable) {
+                box_pair(r, i0, i1, n, Q, s_tally);
+                if (!Q.act[0] && !Q.act[1]) left = 1;
+            }
+            ++n;
+            nf += 1.0f;
+            --left;
         }
     }
     const unsigned int na = __float2uint_rz(n_above.x) + __float2uint_rz(n_above.y);
@@ -611,25 +728,93 @@ __device__ __forceinline__ void pair_loop(const TablesDev& t, const RunDevT<floa
 __device__ __forceinline__ void pair_clear(Pair& Q) {
     Q.x_lo = Q.y = Q.y_lo = Q.u0 = Q.u1 = Q.u2 = Q.tau_lo = P2(0.0f);
     Q.x = Q.tau = P2(__int_as_float(0x7fc00000));       // an empty slot is NaN, as a removed electron
-    Q.ev_cnt[0] = Q.ev_cnt[1] = Q.ev_hash[0] = Q.ev_hash[1] = 0;
     Q.wait[0] = Q.wait[1] = PE_WAIT_NEVER;
     Q.act[0] = Q.act[1] = false;
 }
 
+// Shared memory of the paired kernels: the CTA's sums, the held lanes' slots, the rate tables (kPairFixedBytes,
+// then h(eta) and sigma_Z(gamma)); a multiple of 16 bytes up to the tables.
+constexpr int kPairFixedBytes = kSumsThreads * (16 * kEnergySums + 3 * 8) + 8 * PE_TALLY_WORDS + 4 * PE_HIST_WORDS +
+                                4 * PE_T_E_NCS_STORED;
+static_assert(kPairFixedBytes % 16 == 0, "tables after a 16-byte boundary");
+struct PairShared {
+    ulonglong2* sums;              // [kEnergySums][kSumsThreads]
+    unsigned long long* tally;     // [PE_TALLY_WORDS]: the counts that are not per emission
+    float2* held;                  // [3][kSumsThreads]
+    uint32_t* hist;                // [PE_HIST_WORDS]
+    uint32_t* cnt;                 // [PE_T_E_NCS_STORED]
+    float *h, *sig;
+    __device__ __forceinline__ explicit PairShared(unsigned char* smem, int n_eta) {
+        sums = reinterpret_cast<ulonglong2*>(smem);
+        tally = reinterpret_cast<unsigned long long*>(sums + kEnergySums * kSumsThreads);
+        held = reinterpret_cast<float2*>(tally + PE_TALLY_WORDS);
+        hist = reinterpret_cast<uint32_t*>(held + 3 * kSumsThreads);
+        cnt = hist + PE_HIST_WORDS;
+        h = reinterpret_cast<float*>(cnt + PE_T_E_NCS_STORED);
+        sig = h + n_eta;
+    }
+    __device__ __forceinline__ void init(const TablesDev& t) const {
+        uint32_t* w = reinterpret_cast<uint32_t*>(sums);
+        for (int k = threadIdx.x; k < kPairFixedBytes / 4; k += blockDim.x) w[k] = 0;
+        for (int k = threadIdx.x; k < t.n_eta; k += blockDim.x) h[k] = t.h32[k];
+        for (int k = threadIdx.x; k < t.n_Z * t.n_E; k += blockDim.x) sig[k] = t.sig32[k];
+        __syncthreads();
+    }
+    __device__ __forceinline__ SumsCta acc() const { return SumsCta{hist, cnt, sums + threadIdx.x}; }
+    __device__ __forceinline__ Held slots() const {
+        float2* s = held + threadIdx.x;
+        return Held{s, s + kSumsThreads, s + 2 * kSumsThreads};
+    }
+    // add everything to the run's words and clear it
+    __device__ __forceinline__ void flush(const RunDevT<float>& r) const {
+        __syncthreads();
+        for (int k = threadIdx.x; k < PE_HIST_WORDS; k += blockDim.x) {
+            const uint32_t v = hist[k];
+            if (v) { atomicAdd(r.hist + k, (unsigned long long)v); hist[k] = 0; }
+        }
+        if (threadIdx.x < PE_T_E_NCS_STORED) {
+            const unsigned long long v = tally[threadIdx.x] + cnt[threadIdx.x];
+            if (v) { atomicAdd(r.tally + threadIdx.x, v); tally[threadIdx.x] = 0; cnt[threadIdx.x] = 0; }
+        }
+        for (int k = 0; k < kEnergySums; ++k) {          // 128-bit sums: over the warp, then one add per warp
+            ulonglong2 v = sums[k * kSumsThreads + threadIdx.x];
+            if (!__any_sync(0xffffffffu, (v.x | v.y) != 0)) continue;
+            sums[k * kSumsThreads + threadIdx.x] = make_ulonglong2(0, 0);
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long lo = __shfl_xor_sync(0xffffffffu, v.x, o);
+                const unsigned long long hi = __shfl_xor_sync(0xffffffffu, v.y, o);
+                v.x += lo;
+                v.y += hi + (v.x < lo ? 1ull : 0ull);
+            }
+            if ((threadIdx.x & 31) == 0) {
+                unsigned long long* w = r.tally + PE_T_E_NCS_STORED + 2 * k;
+                const unsigned long long old = atomicAdd(w, v.x);
+                if (old + v.x < old) v.y += 1;
+                if (v.y) atomicAdd(w + 1, v.y);
+            }
+        }
+        __syncthreads();
+    }
+};
+
 // K steps of the two electrons i0 = base + tid and i1 = base + tid + blockDim
-template <int G, bool kCommon>
+template <int G, bool kCommon, bool kSingle, bool kHold>
 __device__ __forceinline__ void tile_steps_pair(const TablesDev& t, const RunDevT<float>& r, const float* s_h,
                                                 const float* sig_z, int64_t i0, int64_t i1, int steps,
-                                                unsigned long long* s_hist, unsigned long long* s_tally) {
+                                                const SumsCta& acc, const Held& held,
+                                                unsigned long long* s_tally) {
     Pair Q;
     pair_clear(Q);
     if (i0 < r.n) load_one(r, i0, Q, 0, s_tally);
     if (i1 < r.n) load_one(r, i1, Q, 1, s_tally);
     if constexpr (G != FK_GAUSS_LP && G != FK_GAUSS_CP) Q.y = Q.y_lo = P2(0.0f);   // 1D: y is not state
     const bool live0 = i0 < r.n, live1 = i1 < r.n;
-    pair_loop<G, kCommon>(t, r, s_h, sig_z, i0, i1, Q, steps, s_hist, s_tally);
-    if (live0 && Q.act[0]) store_particle<float>(r, i0, unpack(Q, 0));
-    if (live1 && Q.act[1]) store_particle<float>(r, i1, unpack(Q, 1));
+    if constexpr (kHold)
+        pair_loop_hold<G, kCommon>(t, r, s_h, sig_z, i0, i1, Q, steps, acc, held, s_tally);
+    else
+        pair_loop<G, kCommon, kSingle>(t, r, s_h, sig_z, i0, i1, Q, steps, acc, s_tally);
+    if (live0 && Q.act[0]) store_one(r, i0, unpack(Q, 0));
+    if (live1 && Q.act[1]) store_one(r, i1, unpack(Q, 1));
 }
 
 // Resident CTAs of 128 threads per SM the register budget is sized for.  Measured on the headline job
@@ -667,29 +852,27 @@ constexpr int pair_min_ctas() {
                          : (G == FK_REFL_LP || G == FK_REFL_CP) ? PE_PAIR_MIN_CTAS_REFL : PE_PAIR_MIN_CTAS;
     return kCommon || kind < PE_PAIR_MIN_CTAS_GENERAL ? kind : PE_PAIR_MIN_CTAS_GENERAL;
 }
-// Persistent kernel of the paired form: 128 threads cover a tile of 256 electrons.
-template <bool kSingle, int G, bool kCommon>
+// Persistent kernel of the paired form: 128 threads cover a tile of 256 electrons.  kHold: the lanes of a warp wait
+// for one another's emissions (pair_loop_hold).
+template <bool kSingle, int G, bool kCommon, bool kHold>
 __global__ void __launch_bounds__(128, (pair_min_ctas<G, kCommon>())) k_step_pair(TablesDev t, BatchDevT<float> b, int steps) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ RunDevT<float> s_run;
-    unsigned long long* s_hist = reinterpret_cast<unsigned long long*>(smem);
-    unsigned long long* s_tally = s_hist + PE_HIST_WORDS;
-    float* s_h = reinterpret_cast<float*>(s_tally + PE_TALLY_WORDS);
-    float* s_sig = s_h + t.n_eta;
-
-    for (int k = threadIdx.x; k < PE_HIST_WORDS + PE_TALLY_WORDS; k += blockDim.x) s_hist[k] = 0;
-    for (int k = threadIdx.x; k < t.n_eta; k += blockDim.x) s_h[k] = t.h32[k];
-    for (int k = threadIdx.x; k < t.n_Z * t.n_E; k += blockDim.x) s_sig[k] = t.sig32[k];
-    __syncthreads();
+    const PairShared S(smem, t.n_eta);
+    S.init(t);
+    const SumsCta acc = S.acc();
+    const Held held = S.slots();
 
     const int64_t n_tiles = b.tile_start[b.n_runs];
+    const uint32_t per_tile = 2u * (uint32_t)b.tile * (uint32_t)steps;   // most emissions of a tile (kMaxLaunchSteps)
+    uint32_t since = 0;                                                 // and since the last flush
     int cur = -1;
     int run_idx = 0;
     for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         if (!kSingle) {
             while (run_idx + 1 < b.n_runs && b.tile_start[run_idx + 1] <= tile) ++run_idx;
             if (run_idx != cur) {
-                if (cur >= 0) flush_shared<float>(s_hist, s_tally, s_run);
+                if (cur >= 0) { S.flush(s_run); since = 0; }
                 constexpr int kWords = sizeof(RunDevT<float>) / 4;
                 for (int w = threadIdx.x; w < kWords; w += blockDim.x)
                     reinterpret_cast<uint32_t*>(&s_run)[w] = reinterpret_cast<const uint32_t*>(&b.runs[run_idx])[w];
@@ -698,14 +881,16 @@ __global__ void __launch_bounds__(128, (pair_min_ctas<G, kCommon>())) k_step_pai
             }
         }
         const RunDevT<float>& r = kSingle ? b.runs[0] : s_run;
+        if (since > kSumsMax - per_tile) { S.flush(r); since = 0; }
+        since += per_tile;
         const int64_t base = (tile - b.tile_start[run_idx]) * b.tile;
         const int64_t i0 = base + threadIdx.x, i1 = base + threadIdx.x + blockDim.x;
-        tile_steps_pair<G, kCommon>(t, r, s_h, s_sig + (size_t)r.iz * t.n_E, i0, i1, steps, s_hist, s_tally);
+        tile_steps_pair<G, kCommon, kSingle, kHold>(t, r, S.h, S.sig + (size_t)r.iz * t.n_E, i0, i1, steps, acc, held, S.tally);
     }
     if (kSingle) {
-        if (n_tiles > 0) flush_shared<float>(s_hist, s_tally, b.runs[0]);
+        if (n_tiles > 0) S.flush(b.runs[0]);
     } else if (cur >= 0) {
-        flush_shared<float>(s_hist, s_tally, s_run);
+        S.flush(s_run);
     }
 }
 
@@ -795,19 +980,13 @@ __device__ __forceinline__ void stage_take(const RunDevT<float>& r, int64_t j, c
     Q.u0 = *q.pux;
     Q.u1 = *q.puy;
     Q.u2 = *q.puz;
+    Q.y = Q.y_lo = P2(0.0f);
     if (r.wait) {
         const uint2 w = reinterpret_cast<const uint2*>(r.wait)[j];
         Q.wait[0] = w.x;
         Q.wait[1] = w.y;
     } else {
         Q.wait[0] = Q.wait[1] = PE_WAIT_NEVER;
-    }
-    if (r.events) {
-        const ulonglong2 e = reinterpret_cast<const ulonglong2*>(r.events)[j];
-        Q.ev_cnt[0] = (uint32_t)e.x; Q.ev_hash[0] = (uint32_t)(e.x >> 32);
-        Q.ev_cnt[1] = (uint32_t)e.y; Q.ev_hash[1] = (uint32_t)(e.y >> 32);
-    } else {
-        Q.ev_cnt[0] = Q.ev_cnt[1] = Q.ev_hash[0] = Q.ev_hash[1] = 0;
     }
     Q.act[0] = !isnan(Q.x.x);
     Q.act[1] = !isnan(Q.x.y);
@@ -830,13 +1009,9 @@ __device__ __forceinline__ void pair_store(const RunDevT<float>& r, int64_t j, c
         __stcs(reinterpret_cast<float2*>(r.uy) + j, Q.u1);
         __stcs(reinterpret_cast<float2*>(r.uz) + j, Q.u2);
         if (r.wait) reinterpret_cast<uint2*>(r.wait)[j] = make_uint2(Q.wait[0], Q.wait[1]);
-        if (r.events)
-            reinterpret_cast<ulonglong2*>(r.events)[j] =
-                make_ulonglong2(((unsigned long long)Q.ev_hash[0] << 32) | Q.ev_cnt[0],
-                                ((unsigned long long)Q.ev_hash[1] << 32) | Q.ev_cnt[1]);
     } else {
-        if (st0) store_particle<float>(r, 2 * j, unpack(Q, 0));
-        if (st1) store_particle<float>(r, 2 * j + 1, unpack(Q, 1));
+        if (st0) store_one(r, 2 * j, unpack(Q, 0));
+        if (st1) store_one(r, 2 * j + 1, unpack(Q, 1));
     }
 }
 
@@ -844,24 +1019,18 @@ template <int G, bool kCommon>
 __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pair_stream(TablesDev t, BatchDevT<float> b,
                                                                                          int steps) {
     extern __shared__ __align__(16) unsigned char smem[];
-    unsigned long long* s_hist = reinterpret_cast<unsigned long long*>(smem);
-    unsigned long long* s_tally = s_hist + PE_HIST_WORDS;
-    float* s_h = reinterpret_cast<float*>(s_tally + PE_TALLY_WORDS);
-    float* s_sig = s_h + t.n_eta;
+    const PairShared S(smem, t.n_eta);
     // the stages on a 16-byte boundary after the tables
-    const uint32_t table_bytes = 8 * (PE_HIST_WORDS + PE_TALLY_WORDS) + 4 * (t.n_eta + t.n_Z * t.n_E);
+    const uint32_t table_bytes = kPairFixedBytes + 4 * (t.n_eta + t.n_Z * t.n_E);
     unsigned char* stage_buf = smem + ((table_bytes + 15u) & ~15u);
     const RunDevT<float>& r = b.runs[0];
-
-    for (int k = threadIdx.x; k < PE_HIST_WORDS + PE_TALLY_WORDS; k += blockDim.x) s_hist[k] = 0;
-    for (int k = threadIdx.x; k < t.n_eta; k += blockDim.x) s_h[k] = t.h32[k];
-    for (int k = threadIdx.x; k < t.n_Z * t.n_E; k += blockDim.x) s_sig[k] = t.sig32[k];
-    __syncthreads();
+    S.init(t);
+    const SumsCta acc = S.acc();                        // at most 2^31 / grid electrons, 4 steps: far below kSumsMax
 
     const int64_t n_tiles = b.tile_start[1];
     const int64_t n_pairs = r.n >> 1;                   // j < n_pairs: electrons 2j and 2j + 1 both present
     const int64_t stride = (int64_t)gridDim.x * kStreamThreads;
-    const float* sig_z = s_sig + (size_t)r.iz * t.n_E;
+    const float* sig_z = S.sig + (size_t)r.iz * t.n_E;
     // tile k of this CTA (k = 0, 1, ...) is tile blockIdx.x + k gridDim.x, staged in stage k mod S;
     // the copies of tiles k + 1 .. k + S - 1 are in flight while tile k is stepped
     const int64_t j0 = (int64_t)blockIdx.x * kStreamThreads + threadIdx.x;
@@ -881,18 +1050,18 @@ __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pai
         Pair Q;
         const bool full = j < n_pairs;
         if (full) {
-            stage_take(r, j, stage_slots(stage_buf + stage * kStageBytes, threadIdx.x), Q, s_tally);
+            stage_take(r, j, stage_slots(stage_buf + stage * kStageBytes, threadIdx.x), Q, S.tally);
         } else {
             pair_clear(Q);
-            if (2 * j < r.n) load_one(r, 2 * j, Q, 0, s_tally);   // the odd last electron
+            if (2 * j < r.n) load_one(r, 2 * j, Q, 0, S.tally);   // the odd last electron
         }
         const bool live0 = 2 * j < r.n, live1 = full;
-        pair_loop<G, kCommon>(t, r, s_h, sig_z, 2 * j, 2 * j + 1, Q, steps, s_hist, s_tally);
+        pair_loop<G, kCommon, false>(t, r, S.h, sig_z, 2 * j, 2 * j + 1, Q, steps, acc, S.tally);
         pair_store(r, j, Q, live0 && Q.act[0], live1 && Q.act[1]);
         stage = stage + 1 == kStreamStages ? 0 : stage + 1;
     }
     cp_async_wait<0>();
-    if (n_tiles > 0) flush_shared<float>(s_hist, s_tally, r);
+    if (n_tiles > 0) S.flush(r);
 }
 
 }  // namespace pe

@@ -162,19 +162,24 @@ __device__ __forceinline__ float tau_draw_f32(uint32_t wlo, uint32_t whi) {
     return -logf(u.hi) - u.lo / u.hi;
 }
 
-// 128-bit fixed-point add of a float v >= 0 (m c^2) with integer operations only:
-// v 2^64 = m 2^(e - 86) for the 24-bit significand m and biased exponent e
-__device__ __forceinline__ void fx_add_f32(unsigned long long* w, float v) {
-    if (!(v > 0.0f)) return;
+// 128-bit fixed-point value of a float v (m c^2) with integer operations only: v 2^64 = m 2^(e - 86) for
+// the 24-bit significand m and biased exponent e; false (nothing to add) unless v > 0
+__device__ __forceinline__ bool fx_of_f32(float v, unsigned long long& lo, unsigned long long& hi) {
+    if (!(v > 0.0f)) return false;
     uint32_t b = __float_as_uint(v);
     int e = (int)(b >> 23);
     unsigned long long m = (b & 0x7FFFFFu) | (e ? 0x800000u : 0u);
     if (e == 0) e = 1;
     int s = e - 86;
-    unsigned long long lo, hi;
     if (s >= 64) { lo = 0; hi = m << (s - 64); }
     else if (s > 0) { lo = m << s; hi = (s > 40) ? (m >> (64 - s)) : 0ull; }
     else { lo = (s > -64) ? (m >> (-s)) : 0ull; hi = 0; }
+    return true;
+}
+// 128-bit fixed-point add of a float v >= 0 (m c^2) into (lo, hi)
+__device__ __forceinline__ void fx_add_f32(unsigned long long* w, float v) {
+    unsigned long long lo, hi;
+    if (!fx_of_f32(v, lo, hi)) return;
     unsigned long long old = atomicAdd(w, lo);
     if (old + lo < old) hi += 1;
     if (hi) atomicAdd(w + 1, hi);
