@@ -43,6 +43,28 @@ __device__ __forceinline__ void fx_add(unsigned long long* w, double v) {
     if (hi) atomicAdd(w + 1, hi);
 }
 
+// the same value as (lo, hi), zero unless v > 0; sums of such pairs; a pair added to (lo, hi) in memory
+__device__ __forceinline__ ulonglong2 fx_of(double v) {
+    if (!(v > 0.0)) return make_ulonglong2(0, 0);
+    const double ip = floor(v);
+    return make_ulonglong2(__double2ull_rz((v - ip) * 0x1.0p64), (unsigned long long)ip);
+}
+__device__ __forceinline__ void fx_acc(ulonglong2& a, ulonglong2 b) {
+    a.x += b.x;
+    a.y += b.y + (a.x < b.x ? 1ull : 0ull);
+}
+__device__ __forceinline__ ulonglong2 warp_sum(ulonglong2 v) {        // over all 32 lanes
+    for (int o = 16; o > 0; o >>= 1)
+        fx_acc(v, make_ulonglong2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o)));
+    return v;
+}
+__device__ __forceinline__ void fx_add_words(unsigned long long* w, ulonglong2 v) {
+    if (!(v.x | v.y)) return;
+    const unsigned long long old = atomicAdd(w, v.x);
+    if (old + v.x < old) v.y += 1;
+    if (v.y) atomicAdd(w + 1, v.y);
+}
+
 struct Photon {
     float x, y, e, kx, ky, kz;
     uint32_t step, id_mech;

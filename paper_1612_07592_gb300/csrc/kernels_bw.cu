@@ -11,7 +11,8 @@
 // One thread per photon, with the step loop flattened: every pass of the loop takes one
 // step of each lane's current photon, and a lane whose photon is done (converted, at
 // step_end, or out of reach of every pulse for good) takes its next photon, so the lanes of
-// a warp stay busy whatever the spread of path lengths.  A pulse is out of reach of a photon
+// a warp stay busy whatever the spread of path lengths.  The steps before the first pulse reaches a photon are
+// counted in one go.  A pulse is out of reach of a photon
 // when it is behind it -- its fields vanish identically once its phase t - x (for the
 // reflected wave t + x - 2 x_m) is past the pulse's end, and both phases only grow along a
 // photon's path -- or when it can never give chi above the table: a plane wave gives
@@ -126,28 +127,101 @@ __device__ __forceinline__ float bw_pos(const StepC<float>& c, float d, float e,
     return fmaf(d, sf * c.dt, e);
 }
 
+// Resident CTAs of 256 threads per SM the registers are sized for (FP32 reflected kind, 4e5 / 3e6 photons of 2000
+// steps, two thirds converted): 2 CTAs 2.6 / 14.3 ms, 3 2.57 / 13.2, 4 2.66 / 14.0, 5 3.05, 6 3.42
 #ifndef PE_BW_MIN_CTAS
-#define PE_BW_MIN_CTAS 4
+#define PE_BW_MIN_CTAS 3
 #endif
 
+constexpr int kBwThreads = 256;
+// conversions of a warp that wait for their sampling: photon, step, chi and position (fewer than 32 left by the last
+// pass and at most 32 more)
+template <typename R>
+struct Conversions {
+    uint32_t j[64], m[64];
+    R chi[64], x[64], y[64];
+    ulonglong2 e_pairs, e_pos;          // the warp's energy sums, its lane 0's
+};
+
+// steps a photon can be advanced at once before a pulse whose phase is `phi` at its present step and grows by `rate`
+// a step: the fields vanish identically while the phase is <= 0 (0.05 of margin covers the rounding of the FP32 phase),
+// so chi and T are 0 there
+template <typename R>
+__device__ __forceinline__ R free_steps(R phi, R rate) {
+    const R d = ((R)-0.05 - phi) / rate - (R)1;
+    return rate > (R)1e-6 && d > (R)0 ? m_floor(d) : (R)0;
+}
+
+// One warp-wide loop: each pass, the lanes without a photon take their next one from the CTA's share (a counter in
+// shared memory: lanes whose photons end early take more of them), and every lane with one takes a step of it.  The
+// votes hold the lanes of a warp together; without them the lanes that had left one another in the search for a
+// photon never met again, and each pass ran for 10 of 32 lanes.  A conversion's sampling is FP64, on GB300's narrow
+// pipe, and was done by the one lane that had it: 35 of 35 M FP64 warp instructions, half of the time; queued and done
+// 32 at a time it is 2.4 M.  Measured, 4e5 photons x 2000 steps in the reflected a0 = 400 pulse, two thirds of them
+// converted: 5.5 ms; 4.0 with the votes and the steps ahead of the pulse counted in one go; 2.57 with the queue.
+// What is left is issue (0.8 a cycle), a third of it for lanes that wait for the last photons of a CTA's share.
 template <typename R, int G>
-__global__ void __launch_bounds__(256, PE_BW_MIN_CTAS) k_bw_transport(BwDev bw, RunDevT<R> r, const Photon* ph,
-                                                                     int64_t n_ph, int64_t step_end, PairRec* out,
-                                                                     int64_t cap, unsigned long long* tally) {
+__global__ void __launch_bounds__(kBwThreads, PE_BW_MIN_CTAS) k_bw_transport(BwDev bw, RunDevT<R> r, const Photon* ph,
+                                                                     int64_t n_ph, int64_t step_end, int64_t share,
+                                                                     PairRec* out, int64_t cap,
+                                                                     unsigned long long* tally) {
     const StepC<R>& c = r.c;
     const bool two_d = r.geometry == PE_GAUSS_2D;
-    constexpr bool kLeave = G != FK_CONST;                 // a prescribed pulse: fields vanish behind it
+    constexpr bool kLeave = G != FK_CONST;                 // a prescribed pulse: fields vanish before and behind it
     constexpr bool kRefl = G == FK_REFL_LP || G == FK_REFL_CP;
     constexpr bool kPlane = G == FK_PLANE_LP || G == FK_PLANE_CP || kRefl;   // chi bounded as for a plane wave
     // 2 E_max / E_S of the incident pulse: twice the bound on chi / (k - k_x)
     const R reach = (R)2 * c.a0 * m_sqrt((R)1 + c.k_env * c.k_env) * c.inv_ES;
     const R chi_min = sizeof(R) == 8 ? (R)bw.chi_min : (R)bw.fchi_min;
     const R L_end = (R)2 * c.phi_r + c.phi_f + (sizeof(R) == 8 ? (R)1e-6 : (R)1e-3);   // pulse end + margin
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
+    __shared__ unsigned int s_taken;                       // photons of the CTA's share handed out
+    __shared__ Conversions<R> s_conv[kBwThreads / 32];
+    if (threadIdx.x == 0) s_taken = 0;
+    __syncthreads();
+    Conversions<R>& Q = s_conv[threadIdx.x >> 5];
+    int queued = 0;                                        // conversions in Q (the same on every lane)
+    if (lane == 0) Q.e_pairs = Q.e_pos = make_ulonglong2(0, 0);
+    // the last `count` queued conversions, one to a lane: the positron's share of k, the pair record and the sums
+    auto sample = [&](int count) {
+        const bool on = lane < count;
+        PairRec q;
+        double kd = 0.0, ep = 0.0;
+        if (on) {
+            const int at = queued - count + lane;
+            const uint32_t jq = Q.j[at], mq = Q.m[at];
+            const Photon p = ph[jq];
+            const uint4 w = philox4x32_10(make_uint4(p.id_mech, r.run_id, mq, kPurBWX + p.step), r.seed_lo, r.seed_hi);
+            kd = (double)p.e;
+            const double x = bw_sample_x(bw, (double)Q.chi[at], uni53(w64(w.x, w.y)));
+            ep = x * kd;
+            q.x = (float)Q.x[at];
+            q.y = (float)(two_d ? Q.y[at] : (R)0);
+            q.e_minus = (float)(kd - ep);
+            q.e_plus = (float)ep;
+            q.kx = p.kx; q.ky = p.ky; q.kz = p.kz;
+            q.step = mq;
+            q.photon = jq;
+            q.id_mech = p.id_mech;
+        }
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(tally + PE_PT_N_PAIRS, (unsigned long long)count);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (on && base + lane < (unsigned long long)cap) out[base + lane] = q;
+        const ulonglong2 a = warp_sum(fx_of(kd)), b = warp_sum(fx_of(ep));
+        if (lane == 0) {
+            fx_acc(Q.e_pairs, a);
+            fx_acc(Q.e_pos, b);
+        }
+        queued -= count;
+        __syncwarp();
+    };
+    const int64_t j_first = (int64_t)blockIdx.x * share;
+    const int64_t j_left = n_ph - j_first;
+    const unsigned int mine = (unsigned int)(j_left < share ? (j_left > 0 ? j_left : 0) : share);
     unsigned long long n_followed = 0, n_tests = 0, n_above = 0;
-    int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - stride;
-    bool have = false;
+    int64_t j = 0;
+    bool have = false, more = true;                // a photon in hand; the share may hold another
     Photon p{};
     R k = 0, kv[3] = {0, 0, 0}, gm = 0, kx = 0, ky = 0, xe = 0, ye = 0, kdt = 0;
     int64_t ne = 0, m = 0;
@@ -156,111 +230,138 @@ __global__ void __launch_bounds__(256, PE_BW_MIN_CTAS) k_bw_transport(BwDev bw, 
     Depth<R> tau;
     tau.set(1.0);
     while (true) {
-        if (!have) {
-            // this lane's next photon to step: k > 2 m c^2, a step left before step_end, and a pulse
-            // that can raise its chi into the table; the others are only counted (no draw)
-            while (true) {
-                j += stride;
-                if (j >= n_ph) break;
-                p = ph[j];
-                if (!(p.e > 2.0f)) continue;               // the same decision as (double) k > 2
-                ++n_followed;
-                ne = (int64_t)p.step;
-                m = ne + 1;
-                k = (R)p.e;
-                kx = (R)p.kx; ky = (R)p.ky; xe = (R)p.x; ye = (R)p.y;
-                kv[0] = k * kx; kv[1] = k * ky; kv[2] = k * (R)p.kz;
-                const R kk = m_sqrt(kv[0] * kv[0] + kv[1] * kv[1] + kv[2] * kv[2]);
-                gm = (kv[0] > (R)0) ? (kv[1] * kv[1] + kv[2] * kv[2]) / (kk + kv[0]) : kk - kv[0];
-                if (kPlane) {
-                    // k - k_x is gm (formed without cancellation); k + k_x likewise for backward photons
-                    const R gp = (kv[0] < (R)0) ? (kv[1] * kv[1] + kv[2] * kv[2]) / (kk - kv[0]) : kk + kv[0];
-                    inc_never = gm * reach < chi_min;
-                    ref_never = !kRefl || gp * c.refl_r * reach < chi_min;
-                    if (inc_never && ref_never) {        // no pulse can convert it: every step counted, none taken
-                        n_tests += (unsigned long long)(step_end > m ? step_end - m : 0);
-                        continue;
+        const unsigned need = __ballot_sync(0xffffffffu, !have && more);
+        if (need) {
+            unsigned int first = 0;
+            if (lane == __ffs(need) - 1) first = atomicAdd(&s_taken, (unsigned int)__popc(need));
+            first = __shfl_sync(0xffffffffu, first, __ffs(need) - 1);
+            if (!have && more) {
+                // a photon to step has k > 2 m c^2, a step left before step_end, and a pulse that can raise its
+                // chi into the table; the others are only counted (no draw)
+                const unsigned int q = first + __popc(need & ((1u << lane) - 1u));
+                more = q < mine;
+                if (more) {
+                    j = j_first + q;
+                    p = ph[j];
+                }
+                if (more && p.e > 2.0f) {                  // the same decision as (double) k > 2
+                    ++n_followed;
+                    ne = (int64_t)p.step;
+                    m = ne + 1;
+                    k = (R)p.e;
+                    kx = (R)p.kx; ky = (R)p.ky; xe = (R)p.x; ye = (R)p.y;
+                    kv[0] = k * kx; kv[1] = k * ky; kv[2] = k * (R)p.kz;
+                    const R kk = m_sqrt(kv[0] * kv[0] + kv[1] * kv[1] + kv[2] * kv[2]);
+                    gm = (kv[0] > (R)0) ? (kv[1] * kv[1] + kv[2] * kv[2]) / (kk + kv[0]) : kk - kv[0];
+                    if (kPlane) {
+                        // k - k_x is gm (formed without cancellation); k + k_x likewise for backward photons
+                        const R gp = (kv[0] < (R)0) ? (kv[1] * kv[1] + kv[2] * kv[2]) / (kk - kv[0]) : kk + kv[0];
+                        inc_never = gm * reach < chi_min;
+                        ref_never = !kRefl || gp * c.refl_r * reach < chi_min;
+                    }
+                    have = m < step_end;
+                    if (kPlane && inc_never && ref_never) {  // no pulse can convert it: every step counted, none taken
+                        n_tests += (unsigned long long)(have ? step_end - m : 0);
+                        have = false;
                     }
                 }
-                if (m >= step_end) continue;
-                const uint4 w = philox4x32_10(make_uint4(p.id_mech, r.run_id, (uint32_t)ne, kPurBWTau + p.step),
-                                              r.seed_lo, r.seed_hi);
-                kdt = c.bw_coef / k;
-                sf = (R)1;
-                if constexpr (sizeof(R) == 8) {
-                    tau.set(-log(uni53(w64(w.x, w.y))));
-                    mf = (R)m;
-                } else {
-                    // -ln U from the same 53 bits in float-pair arithmetic, and the step as a float
-                    // without a conversion instruction (m < 8192): no FP64-pipe work per photon
-                    tau.set(tau_draw_f32(w.x, w.y));
-                    mf = int_to_float_small((int)m);
+                if (have) {
+                    const uint4 w = philox4x32_10(make_uint4(p.id_mech, r.run_id, (uint32_t)ne, kPurBWTau + p.step),
+                                                  r.seed_lo, r.seed_hi);
+                    kdt = c.bw_coef / k;
+                    sf = (R)1;
+                    if constexpr (sizeof(R) == 8) {
+                        tau.set(-log(uni53(w64(w.x, w.y))));
+                        mf = (R)m;
+                    } else {
+                        // -ln U from the same 53 bits in float-pair arithmetic, and the step as a float
+                        // without a conversion instruction (m < 8192): no FP64-pipe work per photon
+                        tau.set(tau_draw_f32(w.x, w.y));
+                        mf = int_to_float_small((int)m);
+                    }
+                    if constexpr (kLeave) {
+                        // the steps before the first pulse that matters reaches it are counted, not taken
+                        const R px = bw_pos(c, kx, xe, sf);
+                        R skip = inc_never && kPlane ? (R)(step_end - m)
+                                                     : free_steps<R>(phase(c, mf, px, (R)0), c.dt * ((R)1 - kx));
+                        if (kRefl && !ref_never) {
+                            const R s2 = free_steps<R>(phase_refl(c, mf, px, (R)0), c.dt * ((R)1 + kx));
+                            skip = s2 < skip ? s2 : skip;
+                        }
+                        if (skip >= (R)(step_end - m)) {
+                            n_tests += (unsigned long long)(step_end - m);
+                            have = false;
+                        } else {
+                            n_tests += (unsigned long long)skip;
+                            m += (int64_t)skip;
+                            sf += skip;
+                            mf += skip;
+                        }
+                    }
                 }
-                have = true;
-                break;
             }
-            if (!have) break;                          // no photon left for this lane
         }
-        // step m of the lane's photon
-        const R px = bw_pos(c, kx, xe, sf);
-        const R py = bw_pos(c, ky, ye, sf);
-        R E[3], B[3];
-        fields<R, G>(r, px, (R)0, py, mf, E, B);
-        const R chi = chi_photon<R>(kv, gm, E, B, c.inv_ES);
-        int fl;
-        const R T = bw_T(bw, chi, fl);
-        ++n_tests;
-        n_above += fl == 1;
-        if constexpr (sizeof(R) == 8) tau.sub(c.bw_coef * T / k);    // (alpha E_S dt) T / k, the oracle's order
-        else tau.sub(kdt * T);
+        if (!__any_sync(0xffffffffu, have)) {
+            if (!__any_sync(0xffffffffu, more)) break;
+            continue;
+        }
         bool conv = false;
-        PairRec q;
-        if (tau.crossed()) {
-            const uint4 w = philox4x32_10(make_uint4(p.id_mech, r.run_id, (uint32_t)m, kPurBWX + p.step),
-                                          r.seed_lo, r.seed_hi);
-            const double kd = (double)p.e;
-            const double x = bw_sample_x(bw, (double)chi, uni53(w64(w.x, w.y)));
-            const double ep = x * kd;
-            q.x = (float)px;
-            q.y = (float)(two_d ? py : (R)0);
-            q.e_minus = (float)(kd - ep);
-            q.e_plus = (float)ep;
-            q.kx = p.kx; q.ky = p.ky; q.kz = p.kz;
-            q.step = (uint32_t)m;
-            q.photon = (uint32_t)j;
-            q.id_mech = p.id_mech;
-            fx_add(tally + PE_PT_E_PAIRS, kd);
-            fx_add(tally + PE_PT_E_POSITRONS, ep);
-            conv = true;
-            have = false;
-        } else {
-            ++m;
-            if (m >= step_end) {
+        R chi = 0, px = 0, py = 0;
+        if (have) {
+            // step m of the lane's photon
+            px = bw_pos(c, kx, xe, sf);
+            py = bw_pos(c, ky, ye, sf);
+            R E[3], B[3];
+            fields<R, G>(r, px, (R)0, py, mf, E, B);
+            chi = chi_photon<R>(kv, gm, E, B, c.inv_ES);
+            int fl;
+            const R T = bw_T(bw, chi, fl);
+            ++n_tests;
+            n_above += fl == 1;
+            if constexpr (sizeof(R) == 8) tau.sub(c.bw_coef * T / k);    // (alpha E_S dt) T / k, the oracle's order
+            else tau.sub(kdt * T);
+            if (tau.crossed()) {
+                conv = true;
                 have = false;
-            } else if (kLeave) {
-                // every pulse behind the photon for good, or never strong enough for it: the
-                // remaining steps see chi below the table
-                bool gone = inc_never || phase(c, mf, px, (R)0) > L_end;
-                if (kRefl) gone = gone && (ref_never || phase_refl(c, mf, px, (R)0) > L_end);
-                if (gone) {
-                    n_tests += (unsigned long long)(step_end - m);
+            } else {
+                ++m;
+                if (m >= step_end) {
                     have = false;
+                } else if (kLeave) {
+                    // every pulse behind the photon for good, or never strong enough for it: the
+                    // remaining steps see chi below the table
+                    bool gone = inc_never || phase(c, mf, px, (R)0) > L_end;
+                    if (kRefl) gone = gone && (ref_never || phase_refl(c, mf, px, (R)0) > L_end);
+                    if (gone) {
+                        n_tests += (unsigned long long)(step_end - m);
+                        have = false;
+                    }
                 }
+                sf += (R)1;
+                mf += (R)1;
             }
-            sf += (R)1;
-            mf += (R)1;
         }
-        // conversions of this pass, one counter atomic per converging group of lanes
-        const unsigned act = __activemask();
-        const unsigned mask = __ballot_sync(act, conv);
-        if (conv) {
-            const int leader = __ffs(mask) - 1;
-            unsigned long long base = 0;
-            if (lane == leader) base = atomicAdd(tally + PE_PT_N_PAIRS, (unsigned long long)__popc(mask));
-            base = __shfl_sync(mask, base, leader);
-            const unsigned long long idx = base + __popc(mask & ((1u << lane) - 1u));
-            if (idx < (unsigned long long)cap) out[idx] = q;
+        // A conversion ends its photon, so nothing of this pass waits for it: its sampling (FP64, a binary search)
+        // is queued and done 32 at a time, on full warps
+        const unsigned mask = __ballot_sync(0xffffffffu, conv);
+        if (mask) {
+            if (conv) {
+                const int at = queued + __popc(mask & ((1u << lane) - 1u));
+                Q.j[at] = (uint32_t)j;
+                Q.m[at] = (uint32_t)m;
+                Q.chi[at] = chi;
+                Q.x[at] = px;
+                Q.y[at] = py;
+            }
+            queued += __popc(mask);
+            __syncwarp();
+            if (queued >= 32) sample(32);
         }
+    }
+    if (queued) sample(queued);
+    if (lane == 0) {
+        fx_add_words(tally + PE_PT_E_PAIRS, Q.e_pairs);
+        fx_add_words(tally + PE_PT_E_POSITRONS, Q.e_pos);
     }
     // counters: one warp sum each
     for (int o = 16; o > 0; o >>= 1) {
@@ -281,11 +382,14 @@ void launch_kind(const BwDev& b, const RunDevT<R>& r, const void* photons, int64
     int dev = 0, sms = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_bw_transport<R, G>, 256, 0) != cudaSuccess || occ < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_bw_transport<R, G>, kBwThreads, 0) != cudaSuccess || occ < 1)
         occ = 1;
-    const int64_t blocks = (n + 255) / 256;
-    const int grid = (int)(blocks < (int64_t)sms * occ ? (blocks > 0 ? blocks : 1) : (int64_t)sms * occ);
-    k_bw_transport<R, G><<<grid, 256, 0, s>>>(b, r, static_cast<const Photon*>(photons), n, step_end,
+    // equal shares for the resident CTAs; a few photons are spread a warp's worth to a CTA
+    const int64_t blocks = (n + 31) / 32;
+    const int64_t most = blocks < (int64_t)sms * occ ? (blocks > 0 ? blocks : 1) : (int64_t)sms * occ;
+    const int64_t share = (n + most - 1) / most;
+    const int grid = (int)((n + share - 1) / share);
+    k_bw_transport<R, G><<<grid, kBwThreads, 0, s>>>(b, r, static_cast<const Photon*>(photons), n, step_end, share,
                                               static_cast<PairRec*>(pairs), cap, tally);
 }
 

@@ -29,11 +29,13 @@ static int stream_smem_bytes(int base) { return base + 16 + kStreamStages * kSta
 // 0.84 ms); not in the plane wave and the 2D focus (below 1e-3).
 template <int G>
 static bool hold_of(const BatchDevT<float>& b) {
-    if (G == FK_REFL_LP || G == FK_REFL_CP) return true;
-    if (G != FK_CONST) return false;
-    for (int k = 0; k < b.n_runs; ++k)
-        if (!b.runs[k].enable_brems || b.runs[k].c.P_hat < 1e-3f) return false;
-    return true;
+    if constexpr (G == FK_CONST) {
+        for (int k = 0; k < b.n_runs; ++k)
+            if (!b.runs[k].enable_brems || b.runs[k].c.P_hat < 1e-3f) return false;
+        return true;
+    } else {
+        return G == FK_REFL_LP || G == FK_REFL_CP;
+    }
 }
 
 // The kernel of a launch, its threads per CTA (block/2: two electrons per thread) and dynamic

@@ -780,18 +780,8 @@ struct PairShared {
             ulonglong2 v = sums[k * kSumsThreads + threadIdx.x];
             if (!__any_sync(0xffffffffu, (v.x | v.y) != 0)) continue;
             sums[k * kSumsThreads + threadIdx.x] = make_ulonglong2(0, 0);
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long lo = __shfl_xor_sync(0xffffffffu, v.x, o);
-                const unsigned long long hi = __shfl_xor_sync(0xffffffffu, v.y, o);
-                v.x += lo;
-                v.y += hi + (v.x < lo ? 1ull : 0ull);
-            }
-            if ((threadIdx.x & 31) == 0) {
-                unsigned long long* w = r.tally + PE_T_E_NCS_STORED + 2 * k;
-                const unsigned long long old = atomicAdd(w, v.x);
-                if (old + v.x < old) v.y += 1;
-                if (v.y) atomicAdd(w + 1, v.y);
-            }
+            v = warp_sum(v);
+            if ((threadIdx.x & 31) == 0) fx_add_words(r.tally + PE_T_E_NCS_STORED + 2 * k, v);
         }
         __syncthreads();
     }
