@@ -10,7 +10,7 @@ kernel, state in registers across the steps of a launch).
 Lines printed (rank 0): one JSON object with the contract keys plus
   roofline      the dominant kernel (k_step_persistent<float>) against the FP32 pipe
   roofline_hbm  the one-step-per-launch form on a state larger than L2 against HBM
-  fp64_plain    the plain FP64 path (one launch per step) on the same job
+  fp64_plain    the FP64 path on the same job
   cpu_baseline  the FP64 oracle on the host cores on a bounded sample
   e2e           the same metric through the public API with host buffers
 `--impl reference` times the oracle alone on the same workload and metric.
@@ -456,7 +456,7 @@ def fma_peaks(pe, stream, sms):
 
 
 def fp64_plain(pe, tables, cfg, stream, flush, reps=3):
-    """The plain FP64 path (one launch per step, tables in global memory) on the same job: one
+    """The FP64 path (k_step_persistent) on the same job: one
     warm-up job, then the mean of `reps` timed jobs from the same initial state, L2 flushed."""
     import torch
     run = dict(cfg["run"], run_id=0)
@@ -468,7 +468,7 @@ def fp64_plain(pe, tables, cfg, stream, flush, reps=3):
     out = r.tally_out()
     r.close()
     return {"value": out.live_particle_steps / (ms * 1e-3), "unit": UNIT, "ms_per_job": ms,
-            "kernel": "k_step_plain (fp64, one launch per step)", "timed_jobs": reps, "warmup_jobs": 1}
+            "kernel": "k_step_persistent (fp64, up to 4096 steps per launch)", "timed_jobs": reps, "warmup_jobs": 1}
 
 
 def batch64(pe, stream, flush):

@@ -208,7 +208,8 @@ typedef struct {
  * tile with block/2 threads, two electrons each, the FP64 kernel with block
  * threads; ctas_per_sm: CTAs per SM in the grid; steps_per_launch: steps done
  * per launch with the state held in registers (1 = state round-trips memory
- * every step).  Zeros pick defaults: 256 electrons per tile; three times the
+ * every step; at most 2^20).  Zeros pick defaults: 256 electrons per tile (32 for FP64
+ * runs of up to 512 electrons per SM); three times the
  * CTAs that fit on an SM for the FP32 kernel (once for the one-step form of a
  * single plane-wave run, launches of at most 4 steps), twice for the FP64
  * kernel; min(steps, 4096) steps per launch.                                   */
@@ -272,8 +273,7 @@ pe_status pe_init_particles(const pe_tables* tables, const pe_run_params* params
 pe_status pe_resume_particles(const pe_tables* tables, const pe_run_params* params, int64_t n,
                               const pe_buffers* buffers, int64_t step0, void* cuda_stream, pe_run** out);
 
-/* Advance runs by n_steps.  n_runs == 1: PE_F64 runs use the plain kernel
- * (one launch per step); PE_F32 runs use the persistent kernel.  n_runs > 1
+/* Advance runs by n_steps in launches of at most steps_per_launch steps.  n_runs > 1
  * (<= PE_MAX_BATCH): all runs must be PE_F32 and share the first run's
  * stream; they advance together, one persistent launch per field kind present
  * per steps_per_launch steps.  Asynchronous.  cfg may be NULL.

@@ -18,7 +18,7 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", 
 # arithmetic is unaffected); the stated FP32 error budget includes this
 KERNEL_FLAGS = ["-prec-div=false", "-prec-sqrt=false"]
 # Every rounding as written where kernels must agree bit for bit: the FP64 step kernels (no
-# multiply-add contraction: the plain and the persistent FP64 kernels round every operation
+# multiply-add contraction: every FP64 kernel instance rounds every operation
 # alike, and the oracle builds the same way), and the paired FP32 kernels, whose single-run, batch
 # and streaming instances inline the same emission branches (no contraction, IEEE division and
 # square root: approximate forms lowered per instance made them differ in the last bit).

@@ -619,11 +619,12 @@ static void set_step0(PlanLaunch& L, pe_run* const* runs, int64_t base_extra) {
 }
 
 // persistent launches (grouped by field kind, chunked by steps_per_launch)
+// (any_tables: FP64 rate tables that do not fit shared memory stay in global memory; otherwise they are refused)
 static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, const pe_launch_config* cfg,
-                            Plan& plan) {
+                            bool any_tables, Plan& plan) {
     const pe_tables* t = runs[0]->tables;
     int prec = runs[0]->params.precision;
-    int block = (cfg && cfg->block > 0) ? cfg->block : 256;
+    int block = (cfg && cfg->block > 0) ? cfg->block : 256;          // electrons per tile
     if (block % 64 || block > 256) return fail(PE_ERR_ARG, "pe_step: block must be 64, 128, 192 or 256");
     int K = (cfg && cfg->steps_per_launch > 0) ? cfg->steps_per_launch : (int)std::min<int64_t>(n_steps, 4096);
     K = std::min(std::max(K, 1), kMaxLaunchSteps);
@@ -631,8 +632,16 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
     cudaGetDevice(&dev);
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (prec == PE_F64 && !(cfg && cfg->block > 0)) {
+        int64_t n_all = 0;
+        for (int k = 0; k < n_runs; ++k) n_all += runs[k]->dev.n;
+        block = default_tile_f64(n_all, sms);
+    }
     int smem = persistent_smem_bytes(t->dev, prec);
-    if (smem > 200 * 1024)
+    const bool staged = smem <= 200 * 1024;
+    if (!staged && any_tables)
+        smem = kSumsBytesF64;
+    else if (!staged)
         return fail(PE_ERR_ARG, "pe_step: rate tables (n_eta + n_Z * n_E) too large for shared memory");
     if (prec == PE_F32) smem = pair_smem_bytes(t->dev);
     for (int fk = 0; fk < kFieldKinds; ++fk) {
@@ -666,6 +675,7 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
                 L.bf.reset(new BatchDevT<float>());
                 std::memset(L.bf.get(), 0, sizeof(BatchDevT<float>));
                 L.bf->n_runs = m;
+                L.bf->staged = staged;
                 L.bf->tile = block;
                 for (int k = 0; k <= m; ++k) L.bf->tile_start[k] = tile_start[k];
                 for (int k = 0; k < m; ++k) L.bf->runs[k] = to_float(runs[idx[k]]->dev);
@@ -673,6 +683,7 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
                 L.bd.reset(new BatchDevT<double>());
                 std::memset(L.bd.get(), 0, sizeof(BatchDevT<double>));
                 L.bd->n_runs = m;
+                L.bd->staged = staged;
                 L.bd->tile = block;
                 for (int k = 0; k <= m; ++k) L.bd->tile_start[k] = tile_start[k];
                 for (int k = 0; k < m; ++k) L.bd->runs[k] = runs[idx[k]]->dev;
@@ -730,30 +741,17 @@ extern "C" pe_status pe_step_ex(pe_run* const* runs, int n_runs, int64_t n_steps
         r->steps_done += n_steps;
         return PE_OK;
     }
-    if (n_runs == 1 && prec == PE_F64 && !(cfg && cfg->steps_per_launch > 0)) {
-        pe_run* r = runs[0];
-        RunDev d = r->dev;
-        for (int64_t k = 0; k < n_steps; ++k) {
-            d.step0 = r->steps_done + k;
-            launch_step_plain_f64(t->dev, d, s);
-            g_launches++;
-        }
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return cuda_fail(e, "pe_step: k_step_plain");
-        r->steps_done += n_steps;
-        return PE_OK;
-    }
-
+    // one FP64 run without a number of steps per launch takes any table set and the default launch shape
+    const bool lone_f64 = n_runs == 1 && prec == PE_F64 && !(cfg && cfg->steps_per_launch > 0);
     Plan plan;
-    pe_status st = build_plan(runs, n_runs, n_steps, cfg, plan);
-    (void)prec;
+    pe_status st = build_plan(runs, n_runs, n_steps, lone_f64 ? nullptr : cfg, lone_f64, plan);
     if (st != PE_OK) return st;
     for (PlanLaunch& L : plan.launches) {
         set_step0(L, runs, 0);
         if (L.prec == PE_F32)
             launch_step_persistent_f32(t->dev, *L.bf, L.steps, L.grid, L.block, s);
         else
-            launch_step_persistent_f64(t->dev, *L.bd, L.steps, L.grid, L.block, s);
+            launch_step_persistent_f64(t->dev, *L.bd, L.steps, L.grid, L.block, L.smem, s);
         g_launches++;
     }
     cudaError_t e = cudaGetLastError();
@@ -966,7 +964,7 @@ extern "C" pe_status pe_graph_create(pe_run* const* runs, int n_runs, int64_t st
     g->runs.assign(runs, runs + n_runs);
     g->steps = steps_per_replay;
     g->stream = runs[0]->stream;
-    st = build_plan(runs, n_runs, steps_per_replay, cfg, g->plan);
+    st = build_plan(runs, n_runs, steps_per_replay, cfg, false, g->plan);
     if (st != PE_OK) { delete g; return st; }
     const pe_tables* t = runs[0]->tables;
     cudaError_t e = cudaGraphCreate(&g->graph, 0);

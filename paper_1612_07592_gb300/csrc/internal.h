@@ -124,6 +124,7 @@ template <typename R>
 struct BatchDevT {
     int n_runs;
     int tile;                           // particles per tile
+    int staged;                         // FP64: the rate tables are copied to shared memory
     int64_t tile_start[PE_MAX_BATCH + 1];
     RunDevT<R> runs[PE_MAX_BATCH];
 };
@@ -201,11 +202,11 @@ int fma_chains();
 
 // kernels.cu
 void launch_init(const RunDev& r, int precision, int init_dist, double theta, double beam_u, cudaStream_t s);
-void launch_step_plain_f64(const TablesDev& t, const RunDev& r, cudaStream_t s);
 void launch_step_persistent_f32(const TablesDev& t, const BatchDevT<float>& b, int steps, int grid, int block,
                                 cudaStream_t s);
 void launch_step_persistent_f64(const TablesDev& t, const BatchDevT<double>& b, int steps, int grid, int block,
-                                cudaStream_t s);
+                                int smem, cudaStream_t s);
+constexpr int kSumsBytesF64 = 8 * (PE_HIST_WORDS + PE_TALLY_WORDS);
 int persistent_smem_bytes(const TablesDev& t, int precision);   // the FP64 kernels
 int pair_smem_bytes(const TablesDev& t);                          // the paired FP32 kernels
 int default_ctas_per_sm_f32(int fk, int block, int smem, int steps_per_launch);
@@ -222,5 +223,6 @@ const void* persistent_kernel_f32(const BatchDevT<float>& b, int steps, int smem
                                   int* smem_out);
 const void* persistent_kernel_f64(const BatchDevT<double>& b, int smem, int block, int* threads);
 int persistent_occupancy_f64(int block, int smem);
+int default_tile_f64(int64_t n, int sms);
 
 }  // namespace pe

@@ -81,7 +81,7 @@ void launch_init(const RunDev& r, int precision, int init_dist, double theta, do
 
 int persistent_smem_bytes(const TablesDev& t, int precision) {
     size_t rs = precision == PE_F32 ? 4 : 8;
-    return (int)(8 * (PE_HIST_WORDS + PE_TALLY_WORDS) + rs * (t.n_eta + (size_t)t.n_Z * t.n_E));
+    return (int)(kSumsBytesF64 + rs * (t.n_eta + (size_t)t.n_Z * t.n_E));
 }
 
 }  // namespace pe

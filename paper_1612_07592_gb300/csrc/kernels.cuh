@@ -2,16 +2,13 @@
 //
 //  k_init            one thread per particle: initial position, momentum and
 //                    optical depth from the particle's Philox stream.
-//  k_step_plain      FP64, one thread per particle, one step per launch,
-//                    tables read from global memory, histograms and tallies
-//                    by global atomics (the plain per-run path).
-//  k_step_persistent grid-stride over tiles of one or many runs, K steps per
+//  k_step_persistent FP64: grid-stride over tiles of one or many runs, K steps per
 //                    launch with the particle state in registers, the rate
 //                    tables (h(eta), sigma_Z(gamma)) staged in shared memory,
 //                    photons appended inside the emission branch (one atomic per
 //                    group of lanes there together), histograms and tallies
 //                    accumulated in shared memory and flushed once per run per
-//                    CTA.  Instantiated for double; the FP32 step runs on the
+//                    CTA.  The FP32 step runs on the
 //                    paired kernels (pair_f32.cuh), and the FP32 PIC kernel
 //                    uses step_one below.
 //
@@ -354,8 +351,11 @@ template <typename R, typename A>
 __device__ __forceinline__ void brems_collide(const TablesDev& t, const RunDevT<R>& r, const R* sig_tab,
                                               uint32_t id, uint32_t n, Particle<R>& P, R& gamma, R xn, R yn,
                                               bool& stored, Photon& ph, const A& acc) {
-    R Pbr = brems_prob<R>(t, r, sig_tab, P, gamma, acc);
+    // the draw's high word first: above the run's largest probability no test passes, and neither the rate nor the
+    // probability is needed (gamma below the table's top row, so not counted either)
     uint4 w = draw(r, id, n, PUR_BREMS);
+    if (w.y > r.br_cap && gamma < tabc<R>(t).g_safe) return;
+    R Pbr = brems_prob<R>(t, r, sig_tab, P, gamma, acc);
     if (brems_event(Pbr, w)) take(brems_emit<R>(t, r, id, n, P, gamma, xn, yn, w, acc), P, gamma, stored, ph);
 }
 
@@ -415,7 +415,18 @@ __device__ __forceinline__ void step_one(const TablesDev& t, const RunDevT<R>& r
     const R dt = c.dt;
     R E[3], B[3];
     fields<R, G>(r, P.x, P.x_lo, P.y, nf, E, B);
-    boris<R>(P.u, E, B, dt);
+    // ahead of and behind a pulse the fields are exactly zero: the push is the identity, eta is 0 and the optical
+    // depth stays (FP64 only; the test on the words' bits, off the FP64 pipe)
+    bool field = true;
+    if constexpr (sizeof(R) == 8 && G != FK_PIC) {
+        int bits = 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            bits |= (__double2hiint(E[k]) & 0x7FFFFFFF) | __double2loint(E[k]) | (__double2hiint(B[k]) & 0x7FFFFFFF) |
+                    __double2loint(B[k]);
+        field = bits != 0;
+    }
+    if (field) boris<R>(P.u, E, B, dt);
     // gamma; in FP32 also 1/gamma from one reciprocal square root (v / gamma below becomes
     // v * (1/gamma); an emission refreshes it)
     R gamma, inv_g = 0;
@@ -435,7 +446,7 @@ __device__ __forceinline__ void step_one(const TablesDev& t, const RunDevT<R>& r
     };
     const R xn = P.x, yn = P.y;
 
-    if (kCommon || r.enable_ncs) {
+    if ((kCommon || r.enable_ncs) && (field || !(P.tau > (R)0))) {
         R eta = eta_of<R, G>(P.u, gamma, E, B, c.inv_ES);
         int fl;
         R h = h_of_eta<R>(t, h_tab, eta, fl);
@@ -575,17 +586,12 @@ __device__ void flush_shared(unsigned long long* s_hist, unsigned long long* s_t
         unsigned long long v = s_hist[k];
         if (v) { atomicAdd(r.hist + k, v); s_hist[k] = 0; }
     }
-    if (threadIdx.x < PE_T_E_NCS_STORED) {
-        unsigned long long v = s_tally[threadIdx.x];
-        if (v) { atomicAdd(r.tally + threadIdx.x, v); s_tally[threadIdx.x] = 0; }
-    } else if (threadIdx.x < PE_TALLY_WORDS && ((threadIdx.x - PE_T_E_NCS_STORED) & 1) == 0 &&
-               threadIdx.x <= PE_T_E_RECOIL_BR) {
-        int k = threadIdx.x;
-        unsigned long long lo = s_tally[k], hi = s_tally[k + 1];
-        if (lo || hi) {
-            unsigned long long old = atomicAdd(r.tally + k, lo);
-            if (old + lo < old) hi += 1;
-            if (hi) atomicAdd(r.tally + k + 1, hi);
+    for (int k = threadIdx.x; k <= PE_T_E_RECOIL_BR; k += blockDim.x) {
+        if (k < PE_T_E_NCS_STORED) {
+            const unsigned long long v = s_tally[k];
+            if (v) { atomicAdd(r.tally + k, v); s_tally[k] = 0; }
+        } else if (((k - PE_T_E_NCS_STORED) & 1) == 0) {
+            fx_add_words(r.tally + k, make_ulonglong2(s_tally[k], s_tally[k + 1]));
             s_tally[k] = 0;
             s_tally[k + 1] = 0;
         }
@@ -613,10 +619,10 @@ __device__ __forceinline__ void tile_steps(const TablesDev& t, const RunDevT<R>&
 // straight from the kernel parameters (constant-bank operands); otherwise the
 // current run's descriptor is copied to shared memory once per tile, so no step
 // reads an indexed kernel parameter.
-// Resident CTAs of 256 threads per SM the register budget is sized for (64 registers; the FP64
-// persistent kernels)
+// Resident CTAs of 256 threads per SM the register budget is sized for (128 registers, no spills; the FP64 persistent
+// kernels, which a few warps per scheduler bring to the FP64 pipe's rate)
 #ifndef PE_MIN_CTAS
-#define PE_MIN_CTAS 4
+#define PE_MIN_CTAS 2
 #endif
 template <typename R, bool kSingle, int G, bool kCommon = false>
 __global__ void __launch_bounds__(256, PE_MIN_CTAS) k_step_persistent(TablesDev t, BatchDevT<R> b, int steps) {
@@ -630,9 +636,13 @@ __global__ void __launch_bounds__(256, PE_MIN_CTAS) k_step_persistent(TablesDev 
     const R* g_sig = (sizeof(R) == 4) ? (const R*)t.sig32 : (const R*)t.sig64;
 
     for (int k = threadIdx.x; k < PE_HIST_WORDS + PE_TALLY_WORDS; k += blockDim.x) s_hist[k] = 0;
-    for (int k = threadIdx.x; k < t.n_eta; k += blockDim.x) s_h[k] = g_h[k];
-    for (int k = threadIdx.x; k < t.n_Z * t.n_E; k += blockDim.x) s_sig[k] = g_sig[k];
+    if (b.staged) {
+        for (int k = threadIdx.x; k < t.n_eta; k += blockDim.x) s_h[k] = g_h[k];
+        for (int k = threadIdx.x; k < t.n_Z * t.n_E; k += blockDim.x) s_sig[k] = g_sig[k];
+    }
     __syncthreads();
+    const R* h_tab = b.staged ? s_h : g_h;                     // tables too large for shared memory are read where they are
+    const R* sig_tab = b.staged ? s_sig : g_sig;
 
     const int64_t n_tiles = b.tile_start[b.n_runs];
     int cur = -1;
@@ -643,10 +653,8 @@ __global__ void __launch_bounds__(256, PE_MIN_CTAS) k_step_persistent(TablesDev 
             if (run_idx != cur) {
                 if (cur >= 0) flush_shared<R>(s_hist, s_tally, s_run);
                 constexpr int kWords = sizeof(RunDevT<R>) / 4;
-                static_assert(kWords <= 256, "run descriptor larger than one word per thread");
-                if (threadIdx.x < kWords)
-                    reinterpret_cast<uint32_t*>(&s_run)[threadIdx.x] =
-                        reinterpret_cast<const uint32_t*>(&b.runs[run_idx])[threadIdx.x];
+                for (int w = threadIdx.x; w < kWords; w += blockDim.x)
+                    reinterpret_cast<uint32_t*>(&s_run)[w] = reinterpret_cast<const uint32_t*>(&b.runs[run_idx])[w];
                 __syncthreads();
                 cur = run_idx;
             }
@@ -659,8 +667,8 @@ __global__ void __launch_bounds__(256, PE_MIN_CTAS) k_step_persistent(TablesDev 
             load_particle<R>(r, i, P);
             active = live_or_kill<R>(r, i, P, (uint32_t)r.step0, s_tally);
         }
-        const R* sig_z = s_sig + (size_t)r.iz * t.n_E;
-        tile_steps<R, G, kCommon>(t, r, s_h, sig_z, i, active, P, steps, s_hist, s_tally);
+        const R* sig_z = sig_tab + (size_t)r.iz * t.n_E;
+        tile_steps<R, G, kCommon>(t, r, h_tab, sig_z, i, active, P, steps, s_hist, s_tally);
         cur = kSingle ? 0 : cur;
     }
     if (kSingle) {
