@@ -54,3 +54,65 @@ def test_f64_tables_beyond_shared_memory():
     np.testing.assert_allclose(a[:, 5], b[:, 5], rtol=1e-3)     # the rates differ by the interpolation of 512 rows
     with pytest.raises(pe.PeError):
         pe.pe_step_ex([r.handle], 10, steps_per_launch=5)
+
+
+# ------------------------------------------------------------------- binning of the diagnostics ----
+MEC2 = 0.51099895
+
+
+def near_edges(rng, edges, n):
+    """Values at the edges of a log grid, off by relative amounts of 1e-8 .. 1e-3 (and well inside the bins)."""
+    d = 10.0 ** rng.uniform(-8, -3, n) * rng.choice([-1.0, 1.0], n)
+    d[::7] = rng.uniform(0.01, 0.9, len(d[::7])) * (edges[1] / edges[0] - 1.0)
+    return rng.choice(edges, n) * (1.0 + d)
+
+
+@pytest.mark.parametrize("precision", [pe.PE_F32, pe.PE_F64])
+@pytest.mark.parametrize("n,bins,lo,hi", [(1, 1, 0.01, 1e4), (4099, 200, 0.01, 1e4), (20_001, 4096, 1.0, 50.0),
+                                          (4098, 64, 1e-9, 1e-3)])
+def test_spectrum_bins_at_the_edges(precision, n, bins, lo, hi):
+    """Electrons whose energies lie at the bin edges are counted as the FP64 formula counts them (values so near an
+    edge that another logarithm could place them differently are left out)."""
+    import torch
+    rng = np.random.default_rng(n)
+    lt = small_tables()
+    r = pe.Run(lt, pe.run_params(precision=precision, **W.base_run()), n)
+    e = near_edges(rng, np.exp(np.linspace(np.log(lo), np.log(hi), bins + 1)), n) / MEC2
+    u = np.sqrt(e * (e + 2.0))
+    u = u.astype(np.float32 if precision == pe.PE_F32 else np.float64)
+    ek = (np.sqrt(1.0 + u.astype(np.float64) ** 2) - 1.0) * MEC2
+    with np.errstate(divide="ignore"):
+        pos = (np.log(ek) - np.log(lo)) * (bins / (np.log(hi) - np.log(lo)))
+    u[np.abs(pos - np.round(pos)) < 1e-9 * bins] = 0.0        # at rest: counted nowhere
+    pos[u == 0.0] = -1.0
+    r.ux.copy_(torch.from_numpy(u))
+    r.uy.zero_()
+    r.uz.zero_()
+    inside = pos[(pos >= 0) & (pos < bins)]
+    want = np.bincount(np.floor(inside).astype(int), minlength=bins)
+    np.testing.assert_array_equal(r.electron_spectrum(bins, lo, hi).astype(np.int64), want)
+
+
+@pytest.mark.parametrize("n,nx,ne", [(1, 1, 1), (5003, 40, 32), (3001, 200_000, 4)])
+def test_photon_map_bins_at_the_edges(n, nx, ne):
+    """The same for the photon map: positions and energies at the bin edges."""
+    import torch
+    rng = np.random.default_rng(nx)
+    lt = small_tables()
+    r = pe.Run(lt, pe.run_params(precision=pe.PE_F32, **W.base_run()), 4, capacity=n)
+    kl = 2.0 * np.pi / W.LAMBDA
+    x_lo, x_hi, lo, hi = -1.5e-6, 8e-6, 0.511, 1e4
+    x = (x_lo + (x_hi - x_lo) * (rng.integers(0, nx + 1, n) / nx + 10.0 ** rng.uniform(-9, -2, n) / nx)) * kl
+    p = np.zeros((n, 8), dtype=np.float32)
+    p[:, 0] = x
+    p[:, 2] = near_edges(rng, np.exp(np.linspace(np.log(lo), np.log(hi), ne + 1)), n) / MEC2
+    px = (p[:, 0].astype(np.float64) - x_lo * kl) * (nx / ((x_hi - x_lo) * kl))
+    pe_ = (np.log(p[:, 2].astype(np.float64) * MEC2) - np.log(lo)) * (ne / (np.log(hi) - np.log(lo)))
+    unsure = (np.abs(px - np.round(px)) < 1e-9 * nx) | (np.abs(pe_ - np.round(pe_)) < 1e-9 * ne)
+    p[unsure, 2] = 0.0
+    r.photons.copy_(torch.from_numpy(p.view(np.int32).reshape(-1)))
+    r.tally[pe.T["N_PHOTONS"]] = n
+    ok = ~unsure & (px >= 0) & (px < nx) & (pe_ >= 0) & (pe_ < ne)
+    want = np.bincount(np.floor(px[ok]).astype(int) * ne + np.floor(pe_[ok]).astype(int), minlength=nx * ne)
+    got = r.photon_map(nx, x_lo, x_hi, ne, lo, hi).astype(np.int64).reshape(-1)
+    np.testing.assert_array_equal(got, want)
