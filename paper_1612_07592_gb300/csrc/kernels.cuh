@@ -204,6 +204,53 @@ struct SumsCta {
     }
 };
 
+// SumsDigits: the PIC kernel's, for launches in which an electron adds to a word at most once between two flushes.  Every
+// energy is a 128-bit sum in eight 16-bit digits, one 32-bit word each: native atomics, and 2^16 adds fit before a
+// word can fill.
+struct SumsDigits {
+    uint32_t* hist;                                  // [PE_HIST_WORDS]
+    uint32_t* cnt;                                   // [PE_T_E_NCS_STORED]
+    uint32_t* digits;                                // [kEnergySums][8]
+    __device__ __forceinline__ void count(int w) const { atomicAdd(cnt + w, 1u); }
+    __device__ __forceinline__ void bin(int k) const { atomicAdd(hist + k, 1u); }
+    template <typename R>
+    __device__ __forceinline__ void energy(int w, R v) const {
+        ulonglong2 q = make_ulonglong2(0, 0);
+        if constexpr (sizeof(R) == 4) {
+            if (!fx_of_f32(v, q.x, q.y)) return;
+        } else {
+            q = fx_of(v);
+        }
+        uint32_t* d = digits + (w - PE_T_E_NCS_STORED) / 2 * 8;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t x = (uint32_t)((k < 4 ? q.x : q.y) >> (16 * (k & 3))) & 0xFFFFu;
+            if (x) atomicAdd(d + k, x);
+        }
+    }
+    // the energies into the run's words, by one thread per sum, and cleared
+    __device__ __forceinline__ void flush_energies(unsigned long long* tally) const {
+        if (threadIdx.x >= kEnergySums) return;
+        uint32_t* d = digits + threadIdx.x * 8;
+        ulonglong2 a = make_ulonglong2(0, 0);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const unsigned long long x = d[k];
+            const int sh = 16 * (k & 3);
+            if (k < 4) fx_acc(a, make_ulonglong2(x << sh, sh ? x >> (64 - sh) : 0ull));
+            else a.y += x << sh;
+            d[k] = 0;
+        }
+        fx_add_words(tally + PE_T_E_NCS_STORED + 2 * threadIdx.x, a);
+    }
+    __device__ __forceinline__ void flush_counts(unsigned long long* h, unsigned long long* tally) const {
+        for (int k = threadIdx.x; k < PE_HIST_WORDS; k += blockDim.x)
+            if (hist[k]) atomicAdd(h + k, (unsigned long long)hist[k]);
+        if (threadIdx.x < PE_T_E_NCS_STORED && cnt[threadIdx.x])
+            atomicAdd(tally + threadIdx.x, (unsigned long long)cnt[threadIdx.x]);
+    }
+};
+
 template <typename R, typename A>
 __device__ __forceinline__ void hist_add(const A& acc, int mech, R e, R kx, R ky, R inv_log_emax,
                                          unsigned long long* dbg) {
@@ -353,8 +400,9 @@ __device__ __forceinline__ void brems_collide(const TablesDev& t, const RunDevT<
                                               bool& stored, Photon& ph, const A& acc) {
     // the draw's high word first: above the run's largest probability no test passes, and neither the rate nor the
     // probability is needed (gamma below the table's top row, so not counted either)
+    if (draw(r, id, n, PUR_BREMS).y > r.br_cap && gamma < tabc<R>(t).g_safe) return;
+    asm volatile("" : "+r"(id));                        // the whole draw is formed here, not carried from above
     uint4 w = draw(r, id, n, PUR_BREMS);
-    if (w.y > r.br_cap && gamma < tabc<R>(t).g_safe) return;
     R Pbr = brems_prob<R>(t, r, sig_tab, P, gamma, acc);
     if (brems_event(Pbr, w)) take(brems_emit<R>(t, r, id, n, P, gamma, xn, yn, w, acc), P, gamma, stored, ph);
 }
@@ -401,18 +449,24 @@ __device__ __forceinline__ void box_check(const RunDevT<R>& r, Particle<R>& P, u
     }
 }
 
-// kCommon: the run has NCS on, direct brems and no absorbing box (the paper's setup), known at
-// compile time, so the step carries no test of the run's flags; otherwise they are read from the run.
-template <typename R, int G, bool kCommon = false>
-__device__ __forceinline__ void step_one(const TablesDev& t, const RunDevT<R>& r, const R* h_tab, const R* sig_tab,
-                                         uint32_t id, uint32_t n, R nf, Particle<R>& P,
-                                         unsigned long long* hist, unsigned long long* tally) {
-    const Sums64 acc{hist, tally};
-    bool st;           // an emission branch stored a photon, appended at once (append_now)
-    Photon ph;
+// The step of one particle in two halves: push_one up to the optical depth (true: it crossed zero, the particle
+// emits), rest_one from the bremsstrahlung test on.  kCommon: the run has NCS on, direct brems and no absorbing box (the
+// paper's setup), known at compile time, so the step carries no test of the run's flags; otherwise they are read from
+// the run.  FP32 keeps 1/gamma from one reciprocal square root (v / gamma becomes v * (1/gamma); an emission
+// refreshes it).
+template <typename R>
+__device__ __forceinline__ R over_gamma(R v, R gamma, R inv_g) {
+    if constexpr (sizeof(R) == 4) return v * inv_g;
+    else return v / gamma;
+}
+template <typename R>
+__device__ __forceinline__ void refresh(R gamma, R& inv_g) {
+    if constexpr (sizeof(R) == 4) inv_g = 1.0f / gamma;
+}
+template <typename R, int G, bool kCommon, typename A>
+__device__ __forceinline__ bool push_one(const TablesDev& t, const RunDevT<R>& r, const R* h_tab, R nf, Particle<R>& P,
+                                         R& gamma, R& inv_g, R& eta, const A& acc) {
     const StepC<R>& c = r.c;
-    const R photon_min = tabc<R>(t).photon_min;
-    const R dt = c.dt;
     R E[3], B[3];
     fields<R, G>(r, P.x, P.x_lo, P.y, nf, E, B);
     // ahead of and behind a pulse the fields are exactly zero: the push is the identity, eta is 0 and the optical
@@ -426,10 +480,8 @@ __device__ __forceinline__ void step_one(const TablesDev& t, const RunDevT<R>& r
                     __double2loint(B[k]);
         field = bits != 0;
     }
-    if (field) boris<R>(P.u, E, B, dt);
-    // gamma; in FP32 also 1/gamma from one reciprocal square root (v / gamma below becomes
-    // v * (1/gamma); an emission refreshes it)
-    R gamma, inv_g = 0;
+    if (field) boris<R>(P.u, E, B, c.dt);
+    inv_g = 0;
     if constexpr (sizeof(R) == 4) {
         const float g2 = 1.0f + P.u[0] * P.u[0] + P.u[1] * P.u[1] + P.u[2] * P.u[2];
         inv_g = rsqrtf(g2);
@@ -437,29 +489,32 @@ __device__ __forceinline__ void step_one(const TablesDev& t, const RunDevT<R>& r
     } else {
         gamma = m_sqrt((R)1 + P.u[0] * P.u[0] + P.u[1] * P.u[1] + P.u[2] * P.u[2]);
     }
-    auto over_gamma = [&](R v) -> R {
-        if constexpr (sizeof(R) == 4) return v * inv_g;
-        else return v / gamma;
-    };
-    auto refresh = [&]() {
-        if constexpr (sizeof(R) == 4) inv_g = 1.0f / gamma;
-    };
+    if (!(kCommon || r.enable_ncs) || !(field || !(P.tau > (R)0))) return false;
+    eta = eta_of<R, G>(P.u, gamma, E, B, c.inv_ES);
+    int fl;
+    R h = h_of_eta<R>(t, h_tab, eta, fl);
+    if (fl == 1) acc.count(PE_T_N_ETA_ABOVE);
+    // dN/dt dt = sqrt(3) alpha/(2 pi) (m c^2/hbar) (eta/gamma) h(eta) dt
+    tau_sub(P, c.ncs_coef * over_gamma(eta, gamma, inv_g) * h);
+    return tau_crossed(P);
+}
+// the emission at a crossing: photon, recoil, new optical depth
+template <typename R, typename A>
+__device__ __forceinline__ void emit_one(const TablesDev& t, const RunDevT<R>& r, uint32_t id, uint32_t n,
+                                         Particle<R>& P, R& gamma, R& inv_g, R eta, const A& acc) {
+    bool st;           // the branch stored a photon, appended at once (append_now)
+    Photon ph;
+    take(ncs_emit<R>(t, r, id, n, P, gamma, eta, P.x, P.y, acc), P, gamma, st, ph);
+    if (st) append_now(r, ph);
+    refresh(gamma, inv_g);
+}
+template <typename R, int G, bool kCommon, typename A>
+__device__ __forceinline__ void rest_one(const TablesDev& t, const RunDevT<R>& r, const R* sig_tab, uint32_t id,
+                                         uint32_t n, Particle<R>& P, R& gamma, R& inv_g, const A& acc) {
+    const StepC<R>& c = r.c;
+    bool st;
+    Photon ph;
     const R xn = P.x, yn = P.y;
-
-    if ((kCommon || r.enable_ncs) && (field || !(P.tau > (R)0))) {
-        R eta = eta_of<R, G>(P.u, gamma, E, B, c.inv_ES);
-        int fl;
-        R h = h_of_eta<R>(t, h_tab, eta, fl);
-        if (fl == 1) atomicAdd(tally + PE_T_N_ETA_ABOVE, 1ull);
-        // dN/dt dt = sqrt(3) alpha/(2 pi) (m c^2/hbar) (eta/gamma) h(eta) dt
-        tau_sub(P, c.ncs_coef * over_gamma(eta) * h);
-        if (tau_crossed(P)) {
-            take(ncs_emit<R>(t, r, id, n, P, gamma, eta, xn, yn, acc), P, gamma, st, ph);
-            if (st) append_now(r, ph);
-            refresh();
-        }
-    }
-
     if (kCommon || r.enable_brems) {
         bool in_slab = (xn >= c.x0 && xn <= c.x1);
         if ((G == FK_GAUSS_LP || G == FK_GAUSS_CP) && fabs(yn) > c.yh) in_slab = false;
@@ -468,21 +523,29 @@ __device__ __forceinline__ void step_one(const TablesDev& t, const RunDevT<R>& r
                 const R g_before = gamma;
                 take(brems_candidate<R>(t, r, sig_tab, id, n, P, gamma, in_slab, xn, yn, acc), P, gamma, st, ph);
                 if (st) append_now(r, ph);
-                if (gamma != g_before) refresh();
+                if (gamma != g_before) refresh(gamma, inv_g);
             } else if (P.wait != PE_WAIT_NEVER) {
                 --P.wait;
             }
-        } else if (in_slab && gamma > (R)1 + photon_min) {
+        } else if (in_slab && gamma > (R)1 + tabc<R>(t).photon_min) {
             const R g_before = gamma;
             st = false;
             brems_collide<R>(t, r, sig_tab, id, n, P, gamma, xn, yn, st, ph, acc);
             if (st) append_now(r, ph);
-            if (gamma != g_before) refresh();
+            if (gamma != g_before) refresh(gamma, inv_g);
         }
     }
-
-    advance(P.x, P.x_lo, over_gamma(dt * P.u[0]));
-    if (G == FK_GAUSS_LP || G == FK_GAUSS_CP) advance(P.y, P.y_lo, over_gamma(dt * P.u[1]));
+    advance(P.x, P.x_lo, over_gamma(c.dt * P.u[0], gamma, inv_g));
+    if (G == FK_GAUSS_LP || G == FK_GAUSS_CP) advance(P.y, P.y_lo, over_gamma(c.dt * P.u[1], gamma, inv_g));
+}
+template <typename R, int G, bool kCommon = false>
+__device__ __forceinline__ void step_one(const TablesDev& t, const RunDevT<R>& r, const R* h_tab, const R* sig_tab,
+                                         uint32_t id, uint32_t n, R nf, Particle<R>& P,
+                                         unsigned long long* hist, unsigned long long* tally) {
+    const Sums64 acc{hist, tally};
+    R gamma, inv_g, eta;
+    if (push_one<R, G, kCommon>(t, r, h_tab, nf, P, gamma, inv_g, eta, acc)) emit_one<R>(t, r, id, n, P, gamma, inv_g, eta, acc);
+    rest_one<R, G, kCommon>(t, r, sig_tab, id, n, P, gamma, inv_g, acc);
     if (!kCommon) box_check<R>(r, P, n, tally);
 }
 

@@ -37,26 +37,38 @@ __device__ __forceinline__ void acc_add(unsigned long long* a, long long v) {
     if (v) atomicAdd(a, (unsigned long long)v);
 }
 
-// Shared-memory current sums as two 32-bit words per grid word (32-bit shared atomics
-// run about four times faster than 64-bit ones on GB300): a contribution v (|v| <= 2^36)
-// adds v >> 16 (|.| <= 2^20) to the high word and v & 0xffff to the low word, so
-// v = hi 2^16 + lo exactly.  Up to kFlushTiles tiles of 256 electrons (each adds at
-// most once per word per electron) the high sums stay below 2^31 in magnitude and the
-// low sums below 2^32; the CTA then moves them into the run's 64-bit sums.
+// Shared-memory current sums as two 32-bit words per grid word (32-bit shared atomics are native, 64-bit ones a
+// compare-and-swap loop): a contribution V = rn(v 2^36) (|v| <= 1) adds h = rint(v 2^20) to the high word and
+// l = V - 2^16 h, |l| <= 2^15, to the low word, both signed.  In FP32 h and l come from two magic-number roundings:
+// t = v 2^20 and its remainder r = t - h are exact, and since 2^16 h is even, rn(r 2^16) rounds as V does.  A
+// float-to-64-bit conversion runs on the FP64 pipe (64 clocks of a scheduler for a warp, eight of them an
+// electron: a fifth of the step).  Up to kFlushTiles tiles of 256 electrons (each adds at most once per word per
+// electron) both sums stay below 2^31 in magnitude; the CTA then moves them into the run's 64-bit sums.
 constexpr int kFlushTiles = 7;
 struct SplitSums {
-    unsigned int* hi;   // [3 n_cells], two's complement
-    unsigned int* lo;   // [3 n_cells]
+    int* hi;   // [3 n_cells]
+    int* lo;   // [3 n_cells]
 };
-__device__ __forceinline__ void acc_add(const SplitSums& a, int k, long long v) {
-    if (v) {
-        atomicAdd(a.hi + k, (unsigned int)(int)(v >> 16));
-        atomicAdd(a.lo + k, (unsigned int)(v & 0xffff));
+__device__ __forceinline__ void acc_add(const SplitSums& a, int k, float v) {
+    const float t = v * 0x1.0p20f;
+    const float hb = t + 0x1.8p23f;
+    const float lb = (t - (hb - 0x1.8p23f)) * 0x1.0p16f + 0x1.8p23f;
+    const int h = __float_as_int(hb) - 0x4B400000, l = __float_as_int(lb) - 0x4B400000;
+    if ((h | l) && fabsf(v) < 2.0f) {                   // nothing for a NaN (an electron removed at the next step)
+        atomicAdd(a.hi + k, h);
+        atomicAdd(a.lo + k, l);
+    }
+}
+__device__ __forceinline__ void acc_add(const SplitSums& a, int k, double v) {
+    const long long q = fxq(v);
+    if (q) {
+        atomicAdd(a.hi + k, (int)(q >> 16));
+        atomicAdd(a.lo + k, (int)(q & 0xffff));
     }
 }
 __device__ __forceinline__ void flush_split(const SplitSums& a, int nj, unsigned long long* acc) {
     for (int k = threadIdx.x; k < nj; k += blockDim.x) {
-        const long long v = (long long)(int)a.hi[k] * 65536 + (long long)a.lo[k];
+        const long long v = (long long)a.hi[k] * 65536 + (long long)a.lo[k];
         if (v) atomicAdd(acc + k, (unsigned long long)v);
         a.hi[k] = 0;
         a.lo[k] = 0;
@@ -76,24 +88,25 @@ __device__ __forceinline__ void pic_deposit(R dx, int n, R x_old, R x_new, R vy,
 #pragma unroll
     for (int k = ia; k <= ia + 1; ++k) {
         cum += lin_w<R>(sn, k, (R)0) - lin_w<R>(so, k, (R)0);
-        if (k >= 0 && k < n) acc_add(sj, k, fxq(cum));
+        if (k >= 0 && k < n) acc_add(sj, k, cum);
     }
 #pragma unroll
     for (int k = ia - 1; k <= ia + 1; ++k) {
         const R sbar = (R)0.5 * (lin_w<R>(so, k, (R)0.5) + lin_w<R>(sn, k, (R)0.5));
         if (sbar > (R)0 && k >= 0 && k < n) {
-            acc_add(sj, n + k, fxq(vy * sbar));
-            acc_add(sj, 2 * n + k, fxq(vz * sbar));
+            acc_add(sj, n + k, vy * sbar);
+            acc_add(sj, 2 * n + k, vz * sbar);
         }
     }
 }
 
 // The field update of one step by one CTA of any size: E_x -= dt J_x at the half nodes;
 // F+ and G+ carried one cell along +x, F- and G- along -x, each with the current at the
-// midpoint of its path; the laser enters at x = 0; the current sums are cleared.  Each
-// thread updates one contiguous run of nodes in place (descending for the +x variants,
-// ascending for the -x ones) after keeping the one value it needs from the neighbouring
-// run.  The sums are read at L2 (they were built there by atomics).
+// midpoint of its path; the laser enters at x = 0; the current sums are cleared.  In place, by blocks of kNodes
+// nodes a thread: a block's values are formed in registers, all its loads in flight together, and stored after
+// a barrier; the +x variants go through the blocks from the right and the -x ones from the left, so no block reads
+// what another has written.  The update is the serial end of a step, bound by the latency of its loads (with one
+// node after the other a thread, 1000 cells took some 4 us).  The sums are read at L2 (they were built there by atomics).
 template <typename R, bool kCP>
 __device__ void pic_fields_block(const RunDevT<R>& r) {
     const int n = r.n_cells;
@@ -109,30 +122,33 @@ __device__ void pic_fields_block(const RunDevT<R>& r) {
     const R dt = c.dt;
     const R kx = c.pic_kx, kyz = c.pic_kyz;   // J_x = kx sum, J_y,z = kyz sum (charge sign included)
     auto J = [](const unsigned long long* a, int i) { return (R)(long long)__ldcg(a + i); };
-    const int chunk = (n + 1 + blockDim.x - 1) / blockDim.x;
-    const int i0 = threadIdx.x * chunk, i1 = min(i0 + chunk, n + 1) - 1;   // this thread's nodes [i0, i1]
-    R fp_in = 0, gp_in = 0, fm_in = 0, gm_in = 0;
-    if (i0 <= i1) {
-        if (i0 >= 1) { fp_in = fp[i0 - 1]; gp_in = gp[i0 - 1]; }
-        if (i1 < n) { fm_in = fm[i1 + 1]; gm_in = gm[i1 + 1]; }
-    }
-    __syncthreads();
-    if (i0 <= i1) {
-        for (int i = i1; i >= i0; --i) {            // along +x from node i - 1 through half node i - 1
-            const R f = i == i0 ? fp_in : fp[i - 1];
-            const R g = i == i0 ? gp_in : gp[i - 1];
-            fp[i] = i > 0 ? f - dt * kyz * J(jy, i - 1) : (R)0;
-            gp[i] = i > 0 ? g - dt * kyz * J(jz, i - 1) : (R)0;
+    constexpr int kNodes = sizeof(R) == 4 ? 4 : 2;
+    const int block = kNodes * blockDim.x;
+    const int blocks = (n + block) / block;                            // of the n + 1 nodes
+    for (int b = 0; b < blocks; ++b) {
+        const int right = (blocks - 1 - b) * block + threadIdx.x;      // this thread's nodes: every blockDim-th
+        const int left = b * block + threadIdx.x;
+        R vp[kNodes], wp[kNodes], vm[kNodes], wm[kNodes], e[kNodes];
+#pragma unroll
+        for (int k = 0; k < kNodes; ++k) {
+            const int i = right + k * blockDim.x, m = left + k * blockDim.x;
+            const bool in = i > 0 && i <= n, im = m < n;
+            vp[k] = in ? fp[i - 1] - dt * kyz * J(jy, i - 1) : (R)0;   // along +x through half node i - 1
+            wp[k] = in ? gp[i - 1] - dt * kyz * J(jz, i - 1) : (R)0;
+            vm[k] = im ? fm[m + 1] - dt * kyz * J(jy, m) : (R)0;       // along -x through half node m
+            wm[k] = im ? gm[m + 1] - dt * kyz * J(jz, m) : (R)0;
+            e[k] = im ? ex[m] - dt * kx * J(jx, m) : (R)0;
         }
-        for (int i = i0; i <= i1; ++i) {            // along -x from node i + 1 through half node i
-            const R f = i == i1 ? fm_in : fm[i + 1];
-            const R g = i == i1 ? gm_in : gm[i + 1];
-            fm[i] = i < n ? f - dt * kyz * J(jy, i) : (R)0;
-            gm[i] = i < n ? g - dt * kyz * J(jz, i) : (R)0;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kNodes; ++k) {
+            const int i = right + k * blockDim.x, m = left + k * blockDim.x;
+            if (i <= n) { fp[i] = vp[k]; gp[i] = wp[k]; }
+            if (m <= n) { fm[m] = vm[k]; gm[m] = wm[k]; }
+            if (m < n) ex[m] = e[k];
         }
-        for (int i = i0; i <= i1 && i < n; ++i) ex[i] -= dt * kx * J(jx, i);
+        __syncthreads();
     }
-    __syncthreads();
     for (int i = threadIdx.x; i < 3 * n; i += blockDim.x) jx[i] = 0;
     if (threadIdx.x == 0) {
         // the laser enters at x = 0: F+ = 2 g_y, G+ = 2 g_z at t^{n+1}
@@ -144,60 +160,131 @@ __device__ void pic_fields_block(const RunDevT<R>& r) {
     }
 }
 
-// kCommon: NCS on and direct brems (a PIC run has no absorbing box), known at compile time
+#ifndef PE_PIC_MIN_CTAS
+#define PE_PIC_MIN_CTAS 4
+#endif
+constexpr int kPicThreads = 256;
+// emissions of a warp that wait (fewer than 32 left by the last round and at most 32 more): electron, eta, gamma
+template <typename R>
+struct PicQueue {
+    uint32_t i[64];
+    R eta[64], gamma[64];
+};
+
+// kCommon: NCS on and direct brems (a PIC run has no absorbing box), known at compile time.  The rate tables are read
+// from shared memory if `staged`.
+//
+// An emission is several times as long as the rest of the step and falls to a few per cent of the electrons, so more
+// than half of the warps would issue all of it for one or two lanes.  An electron whose optical depth crosses is
+// stored as it is after the push and queued by its warp; the warp takes the queue 32 emissions at a time, or what there
+// is when its electrons of the round are done, and goes through the rest of the step with them.  1e6 electrons, 1000
+// cells, steps 0 to 500 (us per step): 59 with the emissions where they fell, 64-bit shared sums and a kernel that waits
+// for the one before; 58.6 with the currents' 64-bit conversions off the FP64 pipe; 49 with the queue, native sums and
+// overlapped launches; 48 with the test of Eq. 4 from the draw's high word; 45 with the field update below.  5000
+// electrons: 19, now 14, the length of the chain from one step's loads to the next's.  What is left is issue (0.6 a
+// cycle, some 900 instructions for 32 electrons, a quarter of them the deposit).
 template <typename R, bool kCommon>
-__global__ void __launch_bounds__(256, 4) k_pic_particles(TablesDev t, RunDevT<R> r) {
+__global__ void __launch_bounds__(kPicThreads, PE_PIC_MIN_CTAS) k_pic_particles(TablesDev t, RunDevT<R> r, int staged) {
     extern __shared__ __align__(16) unsigned char smem[];
-    unsigned long long* s_hist = reinterpret_cast<unsigned long long*>(smem);
-    unsigned long long* s_tally = s_hist + PE_HIST_WORDS;
-    unsigned long long* s_j = s_tally + PE_TALLY_WORDS;             // 3 n_cells current sums (split)
-    const SplitSums sj{reinterpret_cast<unsigned int*>(s_j), reinterpret_cast<unsigned int*>(s_j) + 3 * r.n_cells};
-    R* s_h = reinterpret_cast<R*>(s_j + 3 * r.n_cells);
+    PicQueue<R>* s_queue = reinterpret_cast<PicQueue<R>*>(smem);
+    int* s_j = reinterpret_cast<int*>(s_queue + kPicThreads / 32);              // 3 n_cells current sums (split)
+    const int nj = 3 * r.n_cells;
+    uint32_t* s_hist = reinterpret_cast<uint32_t*>(s_j + 2 * nj);
+    R* s_h = reinterpret_cast<R*>(s_hist + PE_HIST_WORDS + PE_T_E_NCS_STORED + 8 * kEnergySums);
     R* s_sig = s_h + t.n_eta;
+    const SplitSums sj{s_j, s_j + nj};
+    const SumsDigits acc{s_hist, s_hist + PE_HIST_WORDS, s_hist + PE_HIST_WORDS + PE_T_E_NCS_STORED};
     const R* g_h = (sizeof(R) == 4) ? (const R*)t.h32 : (const R*)t.h64;
     const R* g_sig = (sizeof(R) == 4) ? (const R*)t.sig32 : (const R*)t.sig64;
-    const int nj = 3 * r.n_cells;
-    for (int k = threadIdx.x; k < PE_HIST_WORDS + PE_TALLY_WORDS + nj; k += blockDim.x) s_hist[k] = 0;
-    for (int k = threadIdx.x; k < t.n_eta; k += blockDim.x) s_h[k] = g_h[k];
-    for (int k = threadIdx.x; k < t.n_Z * t.n_E; k += blockDim.x) s_sig[k] = g_sig[k];
+    constexpr int kWords = PE_HIST_WORDS + PE_T_E_NCS_STORED + 8 * kEnergySums;
+    static_assert(kWords % 2 == 0, "cleared in 8-byte words");
+    for (int k = threadIdx.x; k < nj + kWords / 2; k += blockDim.x) reinterpret_cast<int2*>(s_j)[k] = make_int2(0, 0);
+    if (staged) {
+        for (int k = threadIdx.x; k < t.n_eta; k += blockDim.x) s_h[k] = g_h[k];
+        for (int k = threadIdx.x; k < t.n_Z * t.n_E; k += blockDim.x) s_sig[k] = g_sig[k];
+    }
+    // what follows reads what the previous step wrote: the launch of this kernel may overlap its end
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __syncthreads();
 
-    const R* sig_z = s_sig + (size_t)r.iz * t.n_E;
+    const R* h_tab = staged ? s_h : g_h;
+    const R* sig_z = (staged ? s_sig : g_sig) + (size_t)r.iz * t.n_E;
     const uint32_t step = (uint32_t)r.step0;
     const R nf = (R)step;
-    int tiles = 0;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < r.n; base += (int64_t)gridDim.x * blockDim.x) {
-        if (tiles == kFlushTiles) {                     // keep the split sums in range
-            __syncthreads();
-            flush_split(sj, nj, r.jacc);
-            __syncthreads();
-            tiles = 0;
-        }
-        ++tiles;
-        const int64_t i = base + threadIdx.x;
-        bool active = i < r.n;
-        Particle<R> P;
-        if (active) {
-            load_particle<R>(r, i, P);
-            active = live_or_kill<R>(r, i, P, step, s_tally);
-        }
-        if (active) {
-            const R x_old = P.x + P.x_lo;
-            step_one<R, FK_PIC, kCommon>(t, r, s_h, sig_z, r.id0 + (uint32_t)i, step, nf, P, s_hist, s_tally);
-            const R gamma = m_sqrt((R)1 + P.u[0] * P.u[0] + P.u[1] * P.u[1] + P.u[2] * P.u[2]);
-            const R x_new = P.x + P.x_lo;
-            pic_deposit<R>(r.c.dt, r.n_cells, x_old, x_new, P.u[1] / gamma, P.u[2] / gamma, sj);
-            if (x_new < (R)0 || x_new > r.c.box1) {   // it left through a boundary face, carrying its charge out
-                P.x = (R)NAN;
-                atomicAdd(s_tally + PE_T_N_KILLED, 1ull);
-                atomicAdd(s_tally + PE_T_KILLED_STEPS, (unsigned long long)step + 1ull);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    PicQueue<R>& Q = s_queue[warp];
+    // groups of kFlushTiles tiles: the split sums and the digits stay in range
+    for (int64_t group = (int64_t)blockIdx.x * blockDim.x; group < r.n; group += kFlushTiles * stride) {
+        int64_t base = group + 32 * warp;
+        int tiles = 0, queued = 0;
+        while (true) {
+            const bool more = tiles < kFlushTiles && base < r.n;
+            const int emitting = queued >= 32 ? 32 : (more ? 0 : queued);     // of the warp, this round
+            if (!more && !emitting) break;
+            int64_t i = 0;
+            bool on = false;
+            Particle<R> P;
+            R gamma, inv_g, x_old;
+            if (emitting) {
+                if (lane < emitting) {
+                    const int at = queued - emitting + lane;
+                    i = Q.i[at];
+                    gamma = Q.gamma[at];
+                    load_particle<R>(r, i, P);
+                    x_old = P.x + P.x_lo;
+                    emit_one<R>(t, r, r.id0 + (uint32_t)i, step, P, gamma, inv_g, Q.eta[at], acc);
+                    on = true;
+                }
+                queued -= emitting;
+            } else {
+                i = base + lane;
+                bool active = i < r.n;
+                if (active) {
+                    load_particle<R>(r, i, P);
+                    active = live_or_kill<R>(r, i, P, step, r.tally);
+                }
+                bool crossed = false;
+                R eta;
+                if (active) {
+                    x_old = P.x + P.x_lo;
+                    crossed = push_one<R, FK_PIC, kCommon>(t, r, h_tab, nf, P, gamma, inv_g, eta, acc);
+                }
+                const unsigned mask = __ballot_sync(0xffffffffu, crossed);
+                if (crossed) {
+                    const int at = queued + __popc(mask & ((1u << lane) - 1u));
+                    Q.i[at] = (uint32_t)i;
+                    Q.eta[at] = eta;
+                    Q.gamma[at] = gamma;
+                    store_particle<R>(r, i, P);
+                }
+                queued += __popc(mask);
+                on = active && !crossed;
+                base += stride;
+                ++tiles;
             }
-            store_particle<R>(r, i, P);
+            __syncwarp();
+            if (on) {
+                rest_one<R, FK_PIC, kCommon>(t, r, sig_z, r.id0 + (uint32_t)i, step, P, gamma, inv_g, acc);
+                const R g = m_sqrt((R)1 + P.u[0] * P.u[0] + P.u[1] * P.u[1] + P.u[2] * P.u[2]);
+                const R x_new = P.x + P.x_lo;
+                pic_deposit<R>(r.c.dt, r.n_cells, x_old, x_new, P.u[1] / g, P.u[2] / g, sj);
+                if (x_new < (R)0 || x_new > r.c.box1) {   // it left through a boundary face, carrying its charge out
+                    P.x = (R)NAN;
+                    atomicAdd(r.tally + PE_T_N_KILLED, 1ull);
+                    atomicAdd(r.tally + PE_T_KILLED_STEPS, (unsigned long long)step + 1ull);
+                }
+                store_particle<R>(r, i, P);
+            }
+            __syncwarp();
         }
+        __syncthreads();
+        flush_split(sj, nj, r.jacc);
+        acc.flush_energies(r.tally);
+        __syncthreads();
     }
-    __syncthreads();
-    flush_split(sj, nj, r.jacc);
-    flush_shared<R>(s_hist, s_tally, r);
+    acc.flush_counts(r.hist, r.tally);
     // the last CTA to finish (its sums and every other CTA's are in the run's sums) advances
     // the fields; the count word after the sums goes back to zero for the next step
     __shared__ bool s_last;
@@ -242,23 +329,44 @@ __global__ void __launch_bounds__(kFieldThreads) k_pic_rho_store(RunDevT<R> r) {
 
 }  // namespace
 
-static int pic_smem_bytes(const TablesDev& t, int n_cells, int precision) {
+// Dynamic shared memory of the particle kernel and whether the rate tables are in it.  Tables that leave no room for the
+// queues are read in global memory; a grid and tables beyond kPicSharedMost together are refused (the launch
+// fails), as they are without the queues.
+constexpr size_t kPicSharedMost = 232448 - 16;
+static size_t pic_smem_bytes(const TablesDev& t, int n_cells, int precision, int& staged) {
     const size_t rs = precision == PE_F32 ? 4 : 8;
-    return (int)(8 * (PE_HIST_WORDS + PE_TALLY_WORDS + 3 * (size_t)n_cells) + rs * (t.n_eta + (size_t)t.n_Z * t.n_E));
+    const size_t queues = kPicThreads / 32 * (precision == PE_F32 ? sizeof(PicQueue<float>) : sizeof(PicQueue<double>));
+    const size_t sums = 4 * (6 * (size_t)n_cells + PE_HIST_WORDS + PE_T_E_NCS_STORED + 8 * kEnergySums);
+    const size_t tables = rs * (t.n_eta + (size_t)t.n_Z * t.n_E);
+    const size_t grid_and_tables = 8 * (PE_HIST_WORDS + PE_TALLY_WORDS) + 24 * (size_t)n_cells + tables;
+    staged = queues + sums + tables <= kPicSharedMost;
+    if (grid_and_tables > kPicSharedMost) return grid_and_tables;
+    return queues + sums + (staged ? tables : 0);
 }
 
 template <typename R>
 static void pic_step(const TablesDev& t, const RunDevT<R>& r, int sms, cudaStream_t s) {
-    const int smem = pic_smem_bytes(t, r.n_cells, sizeof(R) == 4 ? PE_F32 : PE_F64);
+    int staged = 1;
+    const size_t smem = pic_smem_bytes(t, r.n_cells, sizeof(R) == 4 ? PE_F32 : PE_F64, staged);
     const bool common = r.enable_ncs && r.enable_brems && r.brems_method == PE_BREMS_DIRECT;
-    const void* f = common ? (const void*)k_pic_particles<R, true> : (const void*)k_pic_particles<R, false>;
-    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    // four resident CTAs of 256 threads per SM (64 registers): measured 90 us per step on 1e6
-    // electrons against 112 us at two (each CTA adds one flush of its current sums)
-    const int64_t blocks = (r.n + 255) / 256;
-    const int grid = (int)(blocks < 4 * (int64_t)sms ? (blocks > 0 ? blocks : 1) : 4 * (int64_t)sms);
-    if (common) k_pic_particles<R, true><<<grid, 256, smem, s>>>(t, r);
-    else k_pic_particles<R, false><<<grid, 256, smem, s>>>(t, r);
+    auto* f = common ? k_pic_particles<R, true> : k_pic_particles<R, false>;
+    cudaFuncSetAttribute((const void*)f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // four resident CTAs of 256 threads per SM (64 registers): on 1e6 electrons, 500 steps, 24.6 ms against 26.8 at
+    // two, 26.3 at three and 27.6 at five (each CTA adds one flush of its current sums)
+    const int64_t blocks = (r.n + kPicThreads - 1) / kPicThreads;
+    const int grid = (int)(blocks < PE_PIC_MIN_CTAS * (int64_t)sms ? (blocks > 0 ? blocks : 1) : PE_PIC_MIN_CTAS * (int64_t)sms);
+    // the next step's CTAs start as this step's leave, clear their sums and wait there for its last (griddepcontrol)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kPicThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, f, t, r, staged);
 }
 
 void launch_pic_step(const TablesDev& t, const RunDev& r, int precision, int sms, cudaStream_t s) {

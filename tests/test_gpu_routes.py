@@ -116,3 +116,59 @@ def test_photon_map_bins_at_the_edges(n, nx, ne):
     want = np.bincount(np.floor(px[ok]).astype(int) * ne + np.floor(pe_[ok]).astype(int), minlength=nx * ne)
     got = r.photon_map(nx, x_lo, x_hi, ne, lo, hi).astype(np.int64).reshape(-1)
     np.testing.assert_array_equal(got, want)
+
+
+# ------------------------------------------------------------------------------------- the 1D PIC ----
+@pytest.mark.parametrize("precision", [pe.PE_F32, pe.PE_F64])
+@pytest.mark.parametrize("n_cells", [4, 255, 256, 511, 512, 1023, 1024, 1500, 4096])
+def test_pic_fields_advect_by_one_cell_per_step(precision, n_cells):
+    """Without charge the wave variants move one cell a step along +-x whatever the blocks of the update: a random
+    grid, shifted, with the laser in front."""
+    import torch
+    lt = small_tables()
+    L = n_cells * 0.01e-6
+    run = W.base_run(a0=5.0, polarisation=1, geometry=pe.PE_PIC_1D, n_cells=n_cells, ne_over_nc=0.0,
+                     slab_x0_m=0.3 * L, slab_thick_m=0.3 * L, **W.AL | dict(charge_state=11.0))
+    r = pe.Run(lt, pe.run_params(precision=precision, **run), 3)
+    rng = np.random.default_rng(n_cells)
+    g = torch.from_numpy(rng.uniform(-1.0, 1.0, 6 * n_cells + 5)).to(r.grid.dtype)
+    r.grid.copy_(g)
+    steps = 3
+    pe.pe_step([r.handle], steps)
+    a, b = g.numpy(), r.grid.cpu().numpy()
+    n = n_cells
+    np.testing.assert_array_equal(a[:n], b[:n])                     # E_x: no current
+    for v in range(4):
+        old, new = a[n + v * (n + 1): n + (v + 1) * (n + 1)], b[n + v * (n + 1): n + (v + 1) * (n + 1)]
+        if v in (0, 2):                                             # F+, G+
+            np.testing.assert_array_equal(new[steps:], old[:-steps])
+        else:
+            np.testing.assert_array_equal(new[:-steps], old[steps:])
+            np.testing.assert_array_equal(new[-steps:], 0.0)
+
+
+@pytest.mark.parametrize("precision", [pe.PE_F32, pe.PE_F64])
+@pytest.mark.parametrize("n,n_cells", [(1, 300), (33, 300), (5_001, 300), (700_001, 400)])
+def test_pic_queue_splits(precision, n, n_cells):
+    """Steps in one call and in calls of one step agree bit for bit (each step launches by itself and may start under the
+    end of the one before), and a run of several tiles a warp counts every emission once: photons, counts and
+    energies of the sums agree with the photon records."""
+    if precision == pe.PE_F64 and n > 10_000:
+        n = 20_001
+    lt = small_tables()
+    run = W.base_run(a0=300.0, init_dist=1, seed=n, geometry=pe.PE_PIC_1D, n_cells=n_cells, slab_x0_m=0.3e-6, **W.AU)
+    outs = []
+    for calls in ((160,), (1,) * 20 + (70, 70)):
+        r = pe.Run(lt, pe.run_params(precision=precision, **run), n, capacity=1 << 22, events=n < 10_000)
+        for k in calls:
+            pe.pe_step([r.handle], k)
+        t = r.tally_out()
+        ph = r.photon_records()
+        outs.append((r.state(), r.grid.cpu().numpy(), bytes(t.tally), bytes(t.hist),
+                     ph[np.lexsort((ph["step"], ph["id_mech"]))].tobytes()))
+        assert len(ph) == t.tally[pe.T["N_NCS_STORED"]] + t.tally[pe.T["N_BR_STORED"]]
+        np.testing.assert_allclose(ph["energy"].astype(np.float64).sum(), t.e_ncs_stored + t.e_br_stored, rtol=1e-6)
+        assert sum(t.hist[:2 * pe.HIST_E_BINS]) == len(ph)
+    np.testing.assert_array_equal(outs[0][0], outs[1][0])
+    np.testing.assert_array_equal(outs[0][1], outs[1][1])
+    assert outs[0][2:] == outs[1][2:]
