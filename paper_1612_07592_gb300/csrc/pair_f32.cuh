@@ -30,11 +30,20 @@ __device__ __forceinline__ float2 neg2(float2 a) { return __fmul2_rn(a, P2(-1.0f
 // paired kernels rounds its own divisions and square roots as IEEE operations)
 __device__ __forceinline__ float2 sqrt2(float2 a) {
     float2 r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r.x) : "f"(a.x));
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r.y) : "f"(a.y));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(a.x));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(a.y));
     return r;
 }
-__device__ __forceinline__ float2 rsqrt2(float2 a) { return make_float2(rsqrtf(a.x), rsqrtf(a.y)); }
+// Reciprocal square root of a >= 1 (every use: 1 + u^2, 1 + a^2), square root (above) and base-2 logarithm in their
+// flush-to-zero forms: the same results for normal operands without the scaling that subnormal ones need, some three
+// instructions each (an eta, or its square, below 2^-126 counts as 0).  1D job 19.5 -> 18.4 ms, 2D focus 16.3 -> 15.4,
+// bunch 8.2 -> 7.7; same bits.
+__device__ __forceinline__ float2 rsqrt2(float2 a) {
+    float2 r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(a.x));
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(a.y));
+    return r;
+}
 // -1/d for d >= 1 (both uses below): the hardware reciprocal estimate of -d refined by one
 // Newton-Raphson step, r' = r + r (1 + d r), which squares its relative error (about 1 ulp after
 // it); it replaces an IEEE division, whose special-case check and branch cost more than the
@@ -48,7 +57,12 @@ __device__ __forceinline__ float2 nrcp2(float2 d) {
     const float2 e = fma2(d, r, P2(1.0f));
     return fma2(r, e, r);
 }
-__device__ __forceinline__ float2 log2v(float2 a) { return make_float2(__log2f(a.x), __log2f(a.y)); }
+__device__ __forceinline__ float2 log2v(float2 a) {
+    float2 r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(a.x));
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(a.y));
+    return r;
+}
 __device__ __forceinline__ float2 sel2(bool cx, bool cy, float2 a, float2 b) {
     return make_float2(cx ? a.x : b.x, cy ? a.y : b.y);
 }
