@@ -494,6 +494,11 @@ static void describe_run(const pe_tables* t, const pe_run_params* rp, int64_t n,
     d.brems_method = rp->brems_method;
     d.wait = rp->brems_method == PE_BREMS_NULL ? static_cast<uint32_t*>(b->brems_wait) : nullptr;
     d.fk = field_kind(rp->geometry, rp->polarisation, rp->reflect_r > 0);
+    if (rp->geometry == PE_CONST) {
+        d.no_field = 1;                       // as the FP32 step sees them
+        for (int k = 0; k < 3; ++k)
+            if ((float)rp->E_const[k] != 0.0f || (float)rp->B_const[k] != 0.0f) d.no_field = 0;
+    }
     d.geometry = rp->geometry;
     d.polarisation = rp->polarisation;
     d.enable_ncs = rp->enable_ncs;

@@ -109,6 +109,7 @@ struct RunDevT {
     uint32_t id0;                 // global id of particle 0 (Philox counter word 0 = id0 + index)
     uint32_t seed_lo, seed_hi;
     int fk;                       // field kind (physics.cuh)
+    int no_field;                 // PE_CONST with all six components zero (the bunch: fields off)
     int brems_method;             // PE_BREMS_DIRECT | PE_BREMS_NULL
     uint32_t br_cap;              // no brems test of Eq. 4 passes if the draw's high word is above this
     uint32_t* wait;               // null collisions: steps to the next candidate
@@ -140,7 +141,7 @@ inline RunDevT<float> to_float(const RunDevT<double>& d) {
     f.geometry = d.geometry; f.polarisation = d.polarisation;
     f.enable_ncs = d.enable_ncs; f.enable_brems = d.enable_brems; f.box_enable = d.box_enable;
     f.iz = d.iz; f.run_id = d.run_id; f.id0 = d.id0; f.seed_lo = d.seed_lo; f.seed_hi = d.seed_hi;
-    f.fk = d.fk; f.brems_method = d.brems_method; f.br_cap = d.br_cap; f.wait = d.wait; f.x_hat = d.x_hat;
+    f.fk = d.fk; f.no_field = d.no_field; f.brems_method = d.brems_method; f.br_cap = d.br_cap; f.wait = d.wait; f.x_hat = d.x_hat;
     f.grid = d.grid; f.jacc = d.jacc; f.n_cells = d.n_cells;
     return f;
 }
@@ -210,15 +211,6 @@ constexpr int kSumsBytesF64 = 8 * (PE_HIST_WORDS + PE_TALLY_WORDS);
 int persistent_smem_bytes(const TablesDev& t, int precision);   // the FP64 kernels
 int pair_smem_bytes(const TablesDev& t);                          // the paired FP32 kernels
 int default_ctas_per_sm_f32(int fk, int block, int smem, int steps_per_launch);
-// every run of the launch has the paper's setup: NCS on, direct brems, no absorbing box (the FP32
-// kernels then take these flags as compile-time constants)
-inline bool common_flags_f32(const BatchDevT<float>& b) {
-    for (int k = 0; k < b.n_runs; ++k) {
-        const RunDevT<float>& r = b.runs[k];
-        if (!r.enable_ncs || !r.enable_brems || r.brems_method != PE_BREMS_DIRECT || r.box_enable) return false;
-    }
-    return true;
-}
 const void* persistent_kernel_f32(const BatchDevT<float>& b, int steps, int smem, int block, int* threads,
                                   int* smem_out);
 const void* persistent_kernel_f64(const BatchDevT<double>& b, int smem, int block, int* threads);

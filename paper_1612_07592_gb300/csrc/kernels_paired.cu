@@ -38,6 +38,18 @@ static bool hold_of(const BatchDevT<float>& b) {
     }
 }
 
+// the flags that every run of a launch has (pair_f32.cuh)
+static int flags_of(const BatchDevT<float>& b) {
+    bool paper = true, brems = true;
+    for (int k = 0; k < b.n_runs; ++k) {
+        const RunDevT<float>& r = b.runs[k];
+        const bool direct = r.enable_brems && r.brems_method == PE_BREMS_DIRECT && !r.box_enable;
+        paper = paper && direct && r.enable_ncs;
+        brems = brems && direct && !r.enable_ncs;
+    }
+    return paper ? kFlagsPaper : brems ? kFlagsBrems : kFlagsRun;
+}
+
 // The kernel of a launch, its threads per CTA (block/2: two electrons per thread) and dynamic
 // shared memory: the resident paired kernel, or for the plane wave its streaming form.
 using StepKernel = void (*)(TablesDev, BatchDevT<float>, int);
@@ -45,17 +57,22 @@ template <bool kSingle, int G>
 static StepKernel kernel_of(const BatchDevT<float>& b, int steps, int block, int base_smem, int& threads, int& smem) {
     smem = base_smem;
     threads = block / 2;
-    const bool common = common_flags_f32(b);
+    const int flags = flags_of(b);
     if constexpr (G == FK_PLANE_LP || G == FK_PLANE_CP) {
         if (kSingle && use_stream(b, steps, block)) {
             smem = stream_smem_bytes(base_smem);
-            return common ? k_step_pair_stream<G, true> : k_step_pair_stream<G, false>;
+            return flags == kFlagsPaper ? k_step_pair_stream<G, kFlagsPaper> : k_step_pair_stream<G, kFlagsRun>;
         }
     }
     constexpr bool kMayHold = G == FK_REFL_LP || G == FK_REFL_CP || G == FK_CONST;
     constexpr bool kMayNot = G != FK_REFL_LP && G != FK_REFL_CP;
-    if (hold_of<G>(b)) return common ? k_step_pair<kSingle, G, true, kMayHold> : k_step_pair<kSingle, G, false, kMayHold>;
-    return common ? k_step_pair<kSingle, G, true, !kMayNot> : k_step_pair<kSingle, G, false, !kMayNot>;
+    const bool hold = hold_of<G>(b);
+    if constexpr (G == FK_CONST)
+        if (flags == kFlagsBrems)
+            return hold ? k_step_pair<kSingle, G, kFlagsBrems, true> : k_step_pair<kSingle, G, kFlagsBrems, false>;
+    if (flags == kFlagsPaper)
+        return hold ? k_step_pair<kSingle, G, kFlagsPaper, kMayHold> : k_step_pair<kSingle, G, kFlagsPaper, !kMayNot>;
+    return hold ? k_step_pair<kSingle, G, kFlagsRun, kMayHold> : k_step_pair<kSingle, G, kFlagsRun, !kMayNot>;
 }
 
 template <bool kSingle, int G>
@@ -113,14 +130,14 @@ int default_ctas_per_sm_f32(int fk, int block, int smem, int steps_per_launch) {
     int occ = 0;
     cudaError_t e;
     if (plane_kind(fk) && steps_per_launch <= kStreamMaxSteps && block == kStreamTile) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step_pair_stream<FK_PLANE_LP, true>, block / 2,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step_pair_stream<FK_PLANE_LP, kFlagsPaper>, block / 2,
                                                           stream_smem_bytes(smem));
         return e == cudaSuccess && occ > 0 ? occ : 1;
     }
     with_paired_kind(fk, [&](auto g) {
         constexpr int G = decltype(g)::value;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &occ, k_step_pair<true, G, true, G == FK_REFL_LP || G == FK_REFL_CP>, block / 2, smem);
+            &occ, k_step_pair<true, G, kFlagsPaper, G == FK_REFL_LP || G == FK_REFL_CP>, block / 2, smem);
     });
     return 3 * (e == cudaSuccess && occ > 0 ? occ : 1);
 }

@@ -132,11 +132,14 @@ __device__ __forceinline__ void gouy2(float2 a, float2& Rn, float2& In, float2& 
 // envelope g = sin^2(k psi) of a pulse at phase phi, psi the phase distance to the nearer end of
 // the pulse, k psi clamped to [0, pi/2] (0 outside the pulse, pi/2 on the flat top); dg/dphi =
 // +-k sin(2 k psi), + before the middle of the pulse and - after it (it vanishes on the flat top
-// and outside)
-__device__ __forceinline__ void envelope2(const StepC<float>& c, float2 phi, float2& g, float2& dg) {
-    const float2 rem = sub2(P2(2.0f * c.phi_r + c.phi_f), phi);
+// and outside).  envelope_arg2: k psi and the distance to the pulse's end.
+__device__ __forceinline__ float2 envelope_arg2(const StepC<float>& c, float2 phi, float2& rem) {
+    rem = sub2(P2(2.0f * c.phi_r + c.phi_f), phi);
     const float2 psi = make_float2(fminf(phi.x, rem.x), fminf(phi.y, rem.y));
-    const float2 arg = clamp2(mul2(P2(c.k_env), psi), 0.0f, 1.57079632679489662f);
+    return clamp2(mul2(P2(c.k_env), psi), 0.0f, 1.57079632679489662f);
+}
+__device__ __forceinline__ void envelope2(const StepC<float>& c, float2 phi, float2 arg, float2 rem, float2& g,
+                                          float2& dg) {
     float2 rs, rc;
     ramp_sincos2(arg, rs, rc);
     g = mul2(rs, rs);
@@ -144,6 +147,24 @@ __device__ __forceinline__ void envelope2(const StepC<float>& c, float2 phi, flo
     const float2 side = sub2(rem, phi);
     dg = make_float2(copysignf(kts.x, side.x), copysignf(kts.y, side.y));
 }
+
+// What the run's flags are at compile time: nothing (read from the run), the paper's setup (NCS on, direct brems, no
+// absorbing box), or brems alone (direct, no NCS, no box: the Sec. 2.2 bunch), so that the step carries no test of them
+// and no code of a process that is off (the bunch, 5e5 electrons x 2000 steps: 7.7 ms with the flags read in each step
+// and the push of zero fields, 5.7 without either).
+enum { kFlagsRun = 0, kFlagsPaper = 1, kFlagsBrems = 2 };
+template <int F>
+__device__ __forceinline__ bool ncs_on(const RunDevT<float>& r) {
+    return F == kFlagsPaper ? true : F == kFlagsBrems ? false : r.enable_ncs != 0;
+}
+template <int F>
+__device__ __forceinline__ bool brems_on(const RunDevT<float>& r) { return F != kFlagsRun || r.enable_brems; }
+template <int F>
+__device__ __forceinline__ bool null_on(const RunDevT<float>& r) {
+    return F == kFlagsRun && r.brems_method == PE_BREMS_NULL;
+}
+template <int F>
+__device__ __forceinline__ bool box_on(const RunDevT<float>& r) { return F == kFlagsRun && r.box_enable; }
 
 // two electrons; per-electron activity and optical-depth pairs.  The event fingerprints stay in memory: an
 // emission adds to its electron's word there (add_events).
@@ -190,16 +211,38 @@ __device__ __forceinline__ void store_one(const RunDevT<float>& r, int64_t i, co
     if (r.wait) r.wait[i] = P.wait;
 }
 
+// phase t^n - x of the pulse and t^n + x - 2 x_m of its mirror image at the pair's positions
+__device__ __forceinline__ float2 phase2(const StepC<float>& c, float2 nf2, const Pair& Q) {
+    return sub2(fma2(nf2, P2(c.dt_lo), sub2(mul2(nf2, P2(c.dt_hi)), Q.x)), Q.x_lo);
+}
+__device__ __forceinline__ float2 phase_refl2(const StepC<float>& c, float2 nf2, const Pair& Q) {
+    return add2(add2(fma2(nf2, P2(c.dt_hi), P2(-c.xm2_hi)), Q.x), fma2(nf2, P2(c.dt_lo), sub2(Q.x_lo, P2(c.xm2_lo))));
+}
+// gamma and 1/gamma from one reciprocal square root
+__device__ __forceinline__ void gamma_pair(const Pair& Q, float2& gamma, float2& inv_g) {
+    const float2 g2 = fma2(Q.u2, Q.u2, fma2(Q.u1, Q.u1, fma2(Q.u0, Q.u0, P2(1.0f))));
+    inv_g = rsqrt2(g2);
+    gamma = mul2(g2, inv_g);
+}
+// no pulse at either electron (its envelope's argument is zero, or the electron is not there) and nothing to emit
+template <int G>
+__device__ __forceinline__ bool no_pulse(const StepC<float>& c, float nf, const Pair& Q) {
+    float2 rem;
+    float2 arg = envelope_arg2(c, phase2(c, P2(nf), Q), rem);
+    if constexpr (G == FK_REFL_LP || G == FK_REFL_CP)
+        arg = add2(arg, envelope_arg2(c, phase_refl2(c, P2(nf), Q), rem));
+    const float2 tsum = add2(Q.tau, Q.tau_lo);
+    return arg.x + arg.y == 0.0f && !(tsum.x <= 0.0f || tsum.y <= 0.0f);
+}
+
 // The first half of a step of two electrons: fields at (x^n, t^n), Boris push, gamma, and with NCS on eta, the
 // rate and the optical depth.  Returns a bit per electron whose optical depth crossed zero (it emits).
 // G = FK_PLANE_LP, FK_PLANE_CP: the 1D plane wave; FK_REFL_LP, FK_REFL_CP: the plane wave and its mirror
 // image; FK_GAUSS_LP, FK_GAUSS_CP: the 2D paraxial focus; FK_CONST: constant fields.  An inactive half of
 // the pair (a removed electron, or an empty slot past the end of the run) has x = NaN, so its fields, momenta,
 // eta and optical depth are NaN from its first step on, and the eta count, the optical depth's crossing and the
-// target test are false for it without reading the activity flags.  kCommon: the run has NCS on, direct brems
-// and no absorbing box (the paper's setup), known at compile time, so the step carries no test of the run's
-// flags; otherwise they are read from the run.
-template <int G, bool kCommon>
+// target test are false for it without reading the activity flags.
+template <int G, int F>
 __device__ __forceinline__ unsigned push_pair(const TablesDev& t, const RunDevT<float>& r, const float* h_tab,
                                               float nf, Pair& Q, float2& gamma, float2& inv_g, float2& eta,
                                               float2& n_above) {
@@ -208,14 +251,27 @@ __device__ __forceinline__ unsigned push_pair(const TablesDev& t, const RunDevT<
     const float2 h = P2(0.5f * c.dt);
     // fields at (x^n, t^n): phase, envelope, carrier
     const float2 nf2 = P2(nf);
-    float2 phi = fma2(nf2, P2(c.dt_lo), sub2(mul2(nf2, P2(c.dt_hi)), Q.x));
-    phi = sub2(phi, Q.x_lo);
-    float2 g, dg;
-    envelope2(c, phi, g, dg);
+    const float2 phi = phase2(c, nf2, Q);
     constexpr bool kPlane = G == FK_PLANE_LP || G == FK_PLANE_CP;
     constexpr bool kRefl = G == FK_REFL_LP || G == FK_REFL_CP;
     constexpr bool kConst = G == FK_CONST;
     constexpr bool kCP = G == FK_PLANE_CP || G == FK_GAUSS_CP || G == FK_REFL_CP;
+    if constexpr (kConst) {
+        // the run's constant fields are zero: the push is the identity and eta is 0, so the optical depth stays (if it
+        // is positive, as an emission leaves it); only gamma is formed
+        if (r.no_field) {
+            const float2 tsum = add2(Q.tau, Q.tau_lo);
+            if (!(tsum.x <= 0.0f || tsum.y <= 0.0f)) {
+                gamma_pair(Q, gamma, inv_g);
+                return 0;
+            }
+        }
+    }
+    float2 g = P2(0.0f), dg = P2(0.0f), rem;
+    if constexpr (!kConst) {
+        const float2 arg = envelope_arg2(c, phi, rem);
+        envelope2(c, phi, arg, rem, g, dg);
+    }
     float2 by = P2(0.0f), bz = P2(0.0f);                // B_y, B_z of the reflected kinds
     const float2 ma0 = P2(-c.a0);
     float2 ey, ez = P2(0.0f), ex = P2(0.0f), bx = P2(0.0f);
@@ -281,10 +337,10 @@ __device__ __forceinline__ unsigned push_pair(const TablesDev& t, const RunDevT<
         sincos2(phi, st, ct);
         const float2 eiy = mul2(ma0, fma2(dg, st, mul2(g, ct)));
         const float2 eiz = kCP ? mul2(P2(c.a0), sub2(mul2(dg, ct), mul2(g, st))) : P2(0.0f);
-        const float2 pr = add2(add2(fma2(nf2, P2(c.dt_hi), P2(-c.xm2_hi)), Q.x),
-                               fma2(nf2, P2(c.dt_lo), sub2(Q.x_lo, P2(c.xm2_lo))));
-        float2 gr, dgr, sr, cr;
-        envelope2(c, pr, gr, dgr);
+        const float2 pr = phase_refl2(c, nf2, Q);
+        float2 gr, dgr, sr, cr, rem_r;
+        const float2 arg_r = envelope_arg2(c, pr, rem_r);
+        envelope2(c, pr, arg_r, rem_r, gr, dgr);
         sincos2(pr, sr, cr);
         const float2 ry = mul2(P2(c.refl_r * c.a0), fma2(dgr, sr, mul2(gr, cr)));    // -r (-a0 (...))
         ey = add2(eiy, ry);
@@ -375,11 +431,9 @@ __device__ __forceinline__ unsigned push_pair(const TablesDev& t, const RunDevT<
     }
     // gamma and 1/gamma from one reciprocal square root (1/gamma serves the rate and the
     // position update; emitting lanes refresh it from their new gamma)
-    const float2 g2 = fma2(Q.u2, Q.u2, fma2(Q.u1, Q.u1, fma2(Q.u0, Q.u0, P2(1.0f))));
-    inv_g = rsqrt2(g2);
-    gamma = mul2(g2, inv_g);
+    gamma_pair(Q, gamma, inv_g);
     unsigned crossed = 0;
-    if (kCommon || r.enable_ncs) {
+    if (ncs_on<F>(r)) {
         // eta = (gamma - u_x) |E| / E_S for the plane wave; ngm = u_x - gamma, for u_x > 0 as
         // -(1 + u_y^2 + u_z^2) / (gamma + u_x) (no cancellation), its sign taken by the last factor
         float2 up = fma2(Q.u2, Q.u2, fma2(Q.u1, Q.u1, P2(1.0f)));
@@ -454,7 +508,7 @@ __device__ __forceinline__ unsigned push_pair(const TablesDev& t, const RunDevT<
 
 // The bremsstrahlung test of Eq. 4 of the pair after its NCS emissions (or the null-collision waits): a bit per
 // electron with a collision to sample (a candidate, for null collisions).
-template <int G, bool kCommon>
+template <int G, int F>
 __device__ __forceinline__ unsigned brems_pair(const TablesDev& t, const RunDevT<float>& r, const float* sig_tab,
                                                const uint32_t id[2], uint32_t n, Pair& Q, float2 gamma, float2 inv_g,
                                                const SumsCta& acc) {
@@ -462,7 +516,7 @@ __device__ __forceinline__ unsigned brems_pair(const TablesDev& t, const RunDevT
     const StepC<float>& c = r.c;
     const TabC<float>& tc = t.cf;
     unsigned hit = 0;
-    if (!kCommon && r.brems_method == PE_BREMS_NULL) {
+    if (null_on<F>(r)) {
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             if (!Q.act[k]) continue;
@@ -564,7 +618,7 @@ __device__ __forceinline__ void emit_ncs_pair(const TablesDev& t, const RunDevT<
     }
 }
 // its bremsstrahlung photons, or null-collision candidates
-template <int G, bool kCommon>
+template <int G, int F>
 __device__ __forceinline__ void emit_brems_pair(const TablesDev& t, const RunDevT<float>& r, const float* sig_tab,
                                                 const uint32_t id[2], uint32_t n, unsigned m, Pair& Q, float2 gamma,
                                                 float2& inv_g, const SumsCta& acc) {
@@ -579,7 +633,7 @@ __device__ __forceinline__ void emit_brems_pair(const TablesDev& t, const RunDev
         const float x = comp(Q.x, k), y = comp(Q.y, k);
         bool st;
         Photon ph;
-        if (!kCommon && r.brems_method == PE_BREMS_NULL) {
+        if (null_on<F>(r)) {
             const bool in_slab = x >= c.x0 && x <= c.x1 && (kOneD || fabsf(y) <= c.yh);
             take(brems_candidate<float>(t, r, sig_tab, idk, n, P, gk, in_slab, x, y, acc), P, gk, st, ph);
         } else {
@@ -630,27 +684,59 @@ __device__ __forceinline__ void box_pair(const RunDevT<float>& r, int64_t i0, in
     }
 }
 
+// The steps of a warp's electrons before the pulse is at any of them: without a field the push is the identity and eta is
+// 0, so the optical depth stays, and a step is gamma, the bremsstrahlung test and the move.  Returns the steps done.
+// A job spends 5 to 30 % of its steps so.  In a loop of its own because a branch around the push in every step costs
+// the paired instructions their order: 1D job 18.4 ms without either, 19.2 with such a branch, 18.1 with the loop; 2D
+// focus (1000 steps) 15.4, 13.6 and 13.0; reflected 15.4, 15.6 and 14.9; batch of 64 23.0, 22.0 and 20.8.
+template <int G, int F>
+__device__ __forceinline__ int steps_before_pulse(const TablesDev& t, const RunDevT<float>& r, const float* sig_z,
+                                                  const uint32_t id[2], int64_t i0, int64_t i1, Pair& Q, int steps,
+                                                  const SumsCta& acc, unsigned long long* s_tally) {
+    const uint32_t n0 = (uint32_t)r.step0;
+    float nf = (float)n0;
+    int s = 0;
+    for (; s < steps; ++s, nf += 1.0f) {
+        const bool act = Q.act[0] || Q.act[1];
+        if (!__all_sync(0xffffffffu, !act || no_pulse<G>(r.c, nf, Q))) break;
+        if (act) {
+            const uint32_t n = n0 + (uint32_t)s;
+            float2 gamma, inv_g;
+            gamma_pair(Q, gamma, inv_g);
+            if (brems_on<F>(r)) {
+                const unsigned hit = brems_pair<G, F>(t, r, sig_z, id, n, Q, gamma, inv_g, acc);
+                if (hit) emit_brems_pair<G, F>(t, r, sig_z, id, n, hit, Q, gamma, inv_g, acc);
+            }
+            move_pair<G>(r.c, Q, inv_g);
+            if (box_on<F>(r)) box_pair(r, i0, i1, n, Q, s_tally);
+        }
+    }
+    return s;
+}
+
 // K steps of the pair Q (electrons i0 and i1), the lanes of a warp in step: an emission is taken where it falls.
-template <int G, bool kCommon, bool kTwoSites>
+template <int G, int F, bool kTwoSites, bool kStream>
 __device__ __forceinline__ void pair_loop(const TablesDev& t, const RunDevT<float>& r, const float* s_h,
                                           const float* sig_z, int64_t i0, int64_t i1, Pair& Q, int steps,
                                           const SumsCta& acc, unsigned long long* s_tally) {
     const uint32_t id[2] = {r.id0 + (uint32_t)i0, r.id0 + (uint32_t)i1};
     const uint32_t n0 = (uint32_t)r.step0;
-    float nf = (float)n0;
+    int s = 0;
+    if constexpr (G != FK_CONST && !kStream) s = steps_before_pulse<G, F>(t, r, sig_z, id, i0, i1, Q, steps, acc, s_tally);
+    float nf = (float)(n0 + (uint32_t)s);
     float2 n_above = P2(0.0f);                          // particle-steps with eta above the table (exact to 2^24)
-    for (int s = 0; s < steps; ++s, nf += 1.0f) {
+    for (; s < steps; ++s, nf += 1.0f) {
         if (Q.act[0] || Q.act[1]) {
             const uint32_t n = n0 + (uint32_t)s;
             float2 gamma, inv_g, eta;
-            const unsigned crossed = push_pair<G, kCommon>(t, r, s_h, nf, Q, gamma, inv_g, eta, n_above);
-            if (crossed) emit_ncs_pair<G, kTwoSites>(t, r, id, n, crossed, Q, gamma, inv_g, eta, acc);
-            if (kCommon || r.enable_brems) {
-                const unsigned hit = brems_pair<G, kCommon>(t, r, sig_z, id, n, Q, gamma, inv_g, acc);
-                if (hit) emit_brems_pair<G, kCommon>(t, r, sig_z, id, n, hit, Q, gamma, inv_g, acc);
+            const unsigned crossed = push_pair<G, F>(t, r, s_h, nf, Q, gamma, inv_g, eta, n_above);
+            if (F != kFlagsBrems && crossed) emit_ncs_pair<G, kTwoSites>(t, r, id, n, crossed, Q, gamma, inv_g, eta, acc);
+            if (brems_on<F>(r)) {
+                const unsigned hit = brems_pair<G, F>(t, r, sig_z, id, n, Q, gamma, inv_g, acc);
+                if (hit) emit_brems_pair<G, F>(t, r, sig_z, id, n, hit, Q, gamma, inv_g, acc);
             }
             move_pair<G>(r.c, Q, inv_g);
-            if (!kCommon && r.box_enable) box_pair(r, i0, i1, n, Q, s_tally);
+            if (box_on<F>(r)) box_pair(r, i0, i1, n, Q, s_tally);
         }
     }
     const unsigned int na = __float2uint_rz(n_above.x) + __float2uint_rz(n_above.y);
@@ -667,14 +753,16 @@ __device__ __forceinline__ void pair_loop(const TablesDev& t, const RunDevT<floa
 // 8.28, 8.27 and 8.39 against 8.72.  Where emissions are rare a lane waits long for company and in the end the warp
 // waits for that lane: at 48 lane-steps the 1D job took 22.3 against 20.9 ms (hold_of chooses).
 constexpr int kHoldSteps = 32;
-template <int G, bool kCommon>
+template <int G, int F>
 __device__ __forceinline__ void pair_loop_hold(const TablesDev& t, const RunDevT<float>& r, const float* s_h,
                                                const float* sig_z, int64_t i0, int64_t i1, Pair& Q, int steps,
                                                const SumsCta& acc, const Held& held_at, unsigned long long* s_tally) {
     const uint32_t id[2] = {r.id0 + (uint32_t)i0, r.id0 + (uint32_t)i1};
-    uint32_t n = (uint32_t)r.step0;                     // this lane's step
+    int done = 0;
+    if constexpr (G != FK_CONST) done = steps_before_pulse<G, F>(t, r, sig_z, id, i0, i1, Q, steps, acc, s_tally);
+    uint32_t n = (uint32_t)r.step0 + (uint32_t)done;    // this lane's step
     float nf = (float)n;
-    int left = (Q.act[0] || Q.act[1]) ? steps : 0;      // and its steps to go
+    int left = (Q.act[0] || Q.act[1]) ? steps - done : 0;   // and its steps to go
     float2 n_above = P2(0.0f);
     unsigned held = 0;                                  // emissions waited for: bits 0, 1 NCS, bits 2, 3 brems
     int lost = 0;
@@ -684,7 +772,7 @@ __device__ __forceinline__ void pair_loop_hold(const TablesDev& t, const RunDevT
         float2 gamma, inv_g;
         if (run) {
             float2 eta;
-            held = push_pair<G, kCommon>(t, r, s_h, nf, Q, gamma, inv_g, eta, n_above);
+            held = push_pair<G, F>(t, r, s_h, nf, Q, gamma, inv_g, eta, n_above);
             if (held) {
                 *held_at.eta = eta;
                 *held_at.gamma = gamma;
@@ -700,11 +788,11 @@ __device__ __forceinline__ void pair_loop_hold(const TablesDev& t, const RunDevT
                 if (held) {
                     gamma = *held_at.gamma;
                     inv_g = *held_at.inv_g;
-                    if (held & 3u) {
+                    if (F != kFlagsBrems && (held & 3u)) {
                         emit_ncs_pair<G, false>(t, r, id, n, held, Q, gamma, inv_g, *held_at.eta, acc);
                         test = true;
                     } else {
-                        emit_brems_pair<G, kCommon>(t, r, sig_z, id, n, held >> 2, Q, gamma, inv_g, acc);
+                        emit_brems_pair<G, F>(t, r, sig_z, id, n, held >> 2, Q, gamma, inv_g, acc);
                         move = true;
                     }
                     held = 0;
@@ -715,8 +803,8 @@ __device__ __forceinline__ void pair_loop_hold(const TablesDev& t, const RunDevT
         }
         if (test) {
             move = true;
-            if (kCommon || r.enable_brems) {
-                held = brems_pair<G, kCommon>(t, r, sig_z, id, n, Q, gamma, inv_g, acc) << 2;
+            if (brems_on<F>(r)) {
+                held = brems_pair<G, F>(t, r, sig_z, id, n, Q, gamma, inv_g, acc) << 2;
                 if (held) {
                     *held_at.gamma = gamma;
                     *held_at.inv_g = inv_g;
@@ -726,7 +814,7 @@ __device__ __forceinline__ void pair_loop_hold(const TablesDev& t, const RunDevT
         }
         if (move) {
             move_pair<G>(r.c, Q, inv_g);
-            if (!kCommon && r.box_enable) {
+            if (box_on<F>(r)) {
                 box_pair(r, i0, i1, n, Q, s_tally);
                 if (!Q.act[0] && !Q.act[1]) left = 1;
             }
@@ -802,7 +890,7 @@ struct PairShared {
 };
 
 // K steps of the two electrons i0 = base + tid and i1 = base + tid + blockDim
-template <int G, bool kCommon, bool kSingle, bool kHold>
+template <int G, int F, bool kSingle, bool kHold>
 __device__ __forceinline__ void tile_steps_pair(const TablesDev& t, const RunDevT<float>& r, const float* s_h,
                                                 const float* sig_z, int64_t i0, int64_t i1, int steps,
                                                 const SumsCta& acc, const Held& held,
@@ -814,52 +902,49 @@ __device__ __forceinline__ void tile_steps_pair(const TablesDev& t, const RunDev
     if constexpr (G != FK_GAUSS_LP && G != FK_GAUSS_CP) Q.y = Q.y_lo = P2(0.0f);   // 1D: y is not state
     const bool live0 = i0 < r.n, live1 = i1 < r.n;
     if constexpr (kHold)
-        pair_loop_hold<G, kCommon>(t, r, s_h, sig_z, i0, i1, Q, steps, acc, held, s_tally);
+        pair_loop_hold<G, F>(t, r, s_h, sig_z, i0, i1, Q, steps, acc, held, s_tally);
     else
-        pair_loop<G, kCommon, kSingle>(t, r, s_h, sig_z, i0, i1, Q, steps, acc, s_tally);
+        pair_loop<G, F, kSingle, false>(t, r, s_h, sig_z, i0, i1, Q, steps, acc, s_tally);
     if (live0 && Q.act[0]) store_one(r, i0, unpack(Q, 0));
     if (live1 && Q.act[1]) store_one(r, i1, unpack(Q, 1));
 }
 
-// Resident CTAs of 128 threads per SM the register budget is sized for.  Measured on the headline job
-// with the run's flags as compile-time constants (particle-steps/s): 4 CTAs (128 registers) 1.59e11,
-// 5 (96) 1.74e11, 6 (80) 1.78e11, 7 (72) 1.79e11, 8 (64) 1.77e11; the grid of three resident waves
-// (21 CTAs per SM) stays the best at 7 (7: 1.63e11, 14: 1.77e11, 21: 1.79e11, 28 and 35: 1.79e11).
-// With the emission branches inlined (no call in the loop, no spill at 72 registers): 6 CTAs
-// 2.005e11, 7 2.058e11, 8 2.066e11 (at 64 registers the batch instance spills).
+// Resident CTAs of 128 threads per SM the register budget is sized for.  Plane wave, 1D job (1e6 x 4000) / batch of 64:
+// 6 CTAs (80 registers) 18.06 / 21.2 ms, 7 (72) 18.07 / 20.8, 8 (64, with some 20 words spilled around the
+// emissions) 17.81 / 20.4.
 #ifndef PE_PAIR_MIN_CTAS
-#define PE_PAIR_MIN_CTAS 7
+#define PE_PAIR_MIN_CTAS 8
 #endif
-// The 2D focus (config 3, one run, particle-steps/s): 4 CTAs (128 registers) 1.25e11, 5 (96)
-// 1.30e11, 6 (80) 1.31e11; at 80 registers the batch instance (served requests) spills, at 96 none.
+// The 2D focus (2e6 electrons x 1000 steps): 4 CTAs 13.6 ms, 5 13.0, 6 12.8, 7 12.7; at 7 the batch instance (served
+// requests) spills around its common path.
 #ifndef PE_PAIR_MIN_CTAS_2D
-#define PE_PAIR_MIN_CTAS_2D 5
+#define PE_PAIR_MIN_CTAS_2D 6
 #endif
-// The reflected wave (1e6 electrons x 4000 steps of the a0 = 270 job with the mirror at the slab
-// rear): 6 CTAs 4.97e10, 7 5.02e10, 8 4.63e10 (one electron per thread at 8 CTAs of 256 threads:
-// 4.78e10); 7 CTAs 5.50e10 once the emission loop's pair-half selects kept the per-electron words
-// out of local memory.
+// The reflected wave (2.5e5 electrons x 3000 steps): 5 CTAs 16.8 ms, 6 16.8, 7 14.9, 8 15.1.
 #ifndef PE_PAIR_MIN_CTAS_REFL
 #define PE_PAIR_MIN_CTAS_REFL 7
 #endif
-// The general instances (flags read at run time: the null-collision method, a process switched
-// off, the box boundary) carry more live state than the common ones, but more registers for them
-// measured slower on the 1 GeV Au bunch (1e6 electrons, fields off, dt = T; direct / null-collision
-// particle-steps/s): 7 CTAs (72 registers) 9.88e10 / 7.09e10, 6 (80) 9.55e10 / 6.70e10, 5 (96)
-// 9.34e10 / 7.01e10.
+// The general instances (flags read at run time: the null-collision method, a process switched off, the box boundary)
+// carry more live state than the others, but more registers for them measured slower (the 1 GeV Au bunch by null
+// collisions, 1e6 electrons: 7 CTAs 7.09e10 particle-steps/s, 6 6.70e10, 5 7.01e10).
 #ifndef PE_PAIR_MIN_CTAS_GENERAL
 #define PE_PAIR_MIN_CTAS_GENERAL 7
 #endif
-template <int G, bool kCommon>
+// Brems alone (the bunch by the direct method, 5e5 electrons x 2000 steps): 7 to 9 CTAs 5.73 to 5.78 ms, 10 5.84.
+#ifndef PE_PAIR_MIN_CTAS_BREMS
+#define PE_PAIR_MIN_CTAS_BREMS 8
+#endif
+template <int G, int F>
 constexpr int pair_min_ctas() {
     constexpr int kind = (G == FK_GAUSS_LP || G == FK_GAUSS_CP) ? PE_PAIR_MIN_CTAS_2D
                          : (G == FK_REFL_LP || G == FK_REFL_CP) ? PE_PAIR_MIN_CTAS_REFL : PE_PAIR_MIN_CTAS;
-    return kCommon || kind < PE_PAIR_MIN_CTAS_GENERAL ? kind : PE_PAIR_MIN_CTAS_GENERAL;
+    if (F == kFlagsBrems) return PE_PAIR_MIN_CTAS_BREMS;
+    return F != kFlagsRun || kind < PE_PAIR_MIN_CTAS_GENERAL ? kind : PE_PAIR_MIN_CTAS_GENERAL;
 }
 // Persistent kernel of the paired form: 128 threads cover a tile of 256 electrons.  kHold: the lanes of a warp wait
 // for one another's emissions (pair_loop_hold).
-template <bool kSingle, int G, bool kCommon, bool kHold>
-__global__ void __launch_bounds__(128, (pair_min_ctas<G, kCommon>())) k_step_pair(TablesDev t, BatchDevT<float> b, int steps) {
+template <bool kSingle, int G, int F, bool kHold>
+__global__ void __launch_bounds__(128, (pair_min_ctas<G, F>())) k_step_pair(TablesDev t, BatchDevT<float> b, int steps) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ RunDevT<float> s_run;
     const PairShared S(smem, t.n_eta);
@@ -889,7 +974,7 @@ __global__ void __launch_bounds__(128, (pair_min_ctas<G, kCommon>())) k_step_pai
         since += per_tile;
         const int64_t base = (tile - b.tile_start[run_idx]) * b.tile;
         const int64_t i0 = base + threadIdx.x, i1 = base + threadIdx.x + blockDim.x;
-        tile_steps_pair<G, kCommon, kSingle, kHold>(t, r, S.h, S.sig + (size_t)r.iz * t.n_E, i0, i1, steps, acc, held, S.tally);
+        tile_steps_pair<G, F, kSingle, kHold>(t, r, S.h, S.sig + (size_t)r.iz * t.n_E, i0, i1, steps, acc, held, S.tally);
     }
     if (kSingle) {
         if (n_tiles > 0) S.flush(b.runs[0]);
@@ -1019,7 +1104,7 @@ __device__ __forceinline__ void pair_store(const RunDevT<float>& r, int64_t j, c
     }
 }
 
-template <int G, bool kCommon>
+template <int G, int F>
 __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pair_stream(TablesDev t, BatchDevT<float> b,
                                                                                          int steps) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1060,7 +1145,7 @@ __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pai
             if (2 * j < r.n) load_one(r, 2 * j, Q, 0, S.tally);   // the odd last electron
         }
         const bool live0 = 2 * j < r.n, live1 = full;
-        pair_loop<G, kCommon, false>(t, r, S.h, sig_z, 2 * j, 2 * j + 1, Q, steps, acc, S.tally);
+        pair_loop<G, F, false, true>(t, r, S.h, sig_z, 2 * j, 2 * j + 1, Q, steps, acc, S.tally);
         pair_store(r, j, Q, live0 && Q.act[0], live1 && Q.act[1]);
         stage = stage + 1 == kStreamStages ? 0 : stage + 1;
     }
