@@ -23,10 +23,10 @@ void launch_step_persistent_f64(const TablesDev& t, const BatchDevT<double>& b, 
     with_field_kind(b.runs[0].fk, [&](auto g) {
         constexpr int G = decltype(g)::value;
         if (b.n_runs == 1) {
-            if (smem > 48 * 1024) cudaFuncSetAttribute(kernel_f64<true, G>(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (smem > 40 * 1024) cudaFuncSetAttribute(kernel_f64<true, G>(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             k_step_persistent<double, true, G><<<grid, block, smem, s>>>(t, b, steps);
         } else {
-            if (smem > 48 * 1024) cudaFuncSetAttribute(kernel_f64<false, G>(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (smem > 40 * 1024) cudaFuncSetAttribute(kernel_f64<false, G>(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             k_step_persistent<double, false, G><<<grid, block, smem, s>>>(t, b, steps);
         }
     });
@@ -40,7 +40,7 @@ const void* persistent_kernel_f64(const BatchDevT<double>& b, int smem, int bloc
         constexpr int G = decltype(g)::value;
         f = b.n_runs == 1 ? kernel_f64<true, G>() : kernel_f64<false, G>();
     });
-    if (smem > 48 * 1024) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (smem > 40 * 1024) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     return f;
 }
 

@@ -17,11 +17,20 @@ constexpr int kStreamMaxSteps = 4;
 int pair_smem_bytes(const TablesDev& t) { return kPairFixedBytes + 4 * (t.n_eta + t.n_Z * t.n_E); }
 
 static bool plane_kind(int fk) { return fk == FK_PLANE_LP || fk == FK_PLANE_CP; }
-static bool use_stream(const BatchDevT<float>& b, int steps, int block) {
-    return b.n_runs == 1 && plane_kind(b.runs[0].fk) && steps <= kStreamMaxSteps && block == kStreamTile;
-}
 // tables, then 16-byte alignment slack and the stage buffers
 static int stream_smem_bytes(int base) { return base + 16 + kStreamStages * kStageBytes; }
+// (rate tables that leave no room for the stages and queues run on the resident form: the same results)
+static bool stream_shape(int fk, int steps, int block, int base_smem) {
+    return plane_kind(fk) && steps <= kStreamMaxSteps && block == kStreamTile &&
+           stream_smem_bytes(base_smem) + (int)sizeof(StreamQueue) * (kStreamThreads / 32) <= 227 * 1024;
+}
+static bool use_stream(const BatchDevT<float>& b, int steps, int block, int base_smem) {
+    return b.n_runs == 1 && stream_shape(b.runs[0].fk, steps, block, base_smem);
+}
+// beside the static shared memory of a kernel (below 6 KB) a launch may use 48 KB without being told so
+static void allow_smem(const void* f, int smem) {
+    if (smem > 40 * 1024) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+}
 
 // Whether the lanes of a warp wait for one another's emissions: where these are frequent, in the reflected wave (5 %
 // of the particle-steps) and in constant fields when a run's largest bremsstrahlung probability per step
@@ -59,9 +68,11 @@ static StepKernel kernel_of(const BatchDevT<float>& b, int steps, int block, int
     threads = block / 2;
     const int flags = flags_of(b);
     if constexpr (G == FK_PLANE_LP || G == FK_PLANE_CP) {
-        if (kSingle && use_stream(b, steps, block)) {
+        if (kSingle && use_stream(b, steps, block, base_smem)) {
             smem = stream_smem_bytes(base_smem);
-            return flags == kFlagsPaper ? k_step_pair_stream<G, kFlagsPaper> : k_step_pair_stream<G, kFlagsRun>;
+            if (steps == 1)
+                return flags == kFlagsPaper ? k_step_pair_stream<G, kFlagsPaper, true> : k_step_pair_stream<G, kFlagsRun, true>;
+            return flags == kFlagsPaper ? k_step_pair_stream<G, kFlagsPaper, false> : k_step_pair_stream<G, kFlagsRun, false>;
         }
     }
     constexpr bool kMayHold = G == FK_REFL_LP || G == FK_REFL_CP || G == FK_CONST;
@@ -80,8 +91,20 @@ static void launch_one(const TablesDev& t, const BatchDevT<float>& b, int steps,
                        int base_smem) {
     int threads, smem;
     const StepKernel f = kernel_of<kSingle, G>(b, steps, block, base_smem, threads, smem);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    f<<<grid, threads, smem, s>>>(t, b, steps);
+    allow_smem((const void*)f, smem);
+    // the streaming form is launched once per step or few: the next launch's CTAs start as this one's leave, clear their
+    // sums, copy the tables and wait there for its last (griddepcontrol)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = kSingle && use_stream(b, steps, block, base_smem) ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, f, t, b, steps);
 }
 
 template <typename F>
@@ -116,7 +139,7 @@ const void* persistent_kernel_f32(const BatchDevT<float>& b, int steps, int base
         f = (const void*)(b.n_runs == 1 ? kernel_of<true, decltype(g)::value>(b, steps, block, base_smem, th, smem)
                                         : kernel_of<false, decltype(g)::value>(b, steps, block, base_smem, th, smem));
     });
-    if (smem > 48 * 1024) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    allow_smem(f, smem);
     *threads = th;
     *smem_out = smem;
     return f;
@@ -129,8 +152,8 @@ const void* persistent_kernel_f32(const BatchDevT<float>& b, int steps, int base
 int default_ctas_per_sm_f32(int fk, int block, int smem, int steps_per_launch) {
     int occ = 0;
     cudaError_t e;
-    if (plane_kind(fk) && steps_per_launch <= kStreamMaxSteps && block == kStreamTile) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step_pair_stream<FK_PLANE_LP, kFlagsPaper>, block / 2,
+    if (stream_shape(fk, steps_per_launch, block, smem)) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step_pair_stream<FK_PLANE_LP, kFlagsPaper, true>, block / 2,
                                                           stream_smem_bytes(smem));
         return e == cudaSuccess && occ > 0 ? occ : 1;
     }

@@ -856,9 +856,11 @@ struct PairShared {
         sig = h + n_eta;
     }
     __device__ __forceinline__ void init(const TablesDev& t) const {
-        uint32_t* w = reinterpret_cast<uint32_t*>(sums);
-        for (int k = threadIdx.x; k < kPairFixedBytes / 4; k += blockDim.x) w[k] = 0;
+        uint4* w = reinterpret_cast<uint4*>(sums);
+        for (int k = threadIdx.x; k < kPairFixedBytes / 16; k += blockDim.x) w[k] = make_uint4(0, 0, 0, 0);
+#pragma unroll 4
         for (int k = threadIdx.x; k < t.n_eta; k += blockDim.x) h[k] = t.h32[k];
+#pragma unroll 4
         for (int k = threadIdx.x; k < t.n_Z * t.n_E; k += blockDim.x) sig[k] = t.sig32[k];
         __syncthreads();
     }
@@ -870,6 +872,7 @@ struct PairShared {
     // add everything to the run's words and clear it
     __device__ __forceinline__ void flush(const RunDevT<float>& r) const {
         __syncthreads();
+#pragma unroll 4
         for (int k = threadIdx.x; k < PE_HIST_WORDS; k += blockDim.x) {
             const uint32_t v = hist[k];
             if (v) { atomicAdd(r.hist + k, (unsigned long long)v); hist[k] = 0; }
@@ -999,16 +1002,14 @@ __global__ void __launch_bounds__(128, (pair_min_ctas<G, F>())) k_step_pair(Tabl
 // ---------------------------------------------------------------------------
 constexpr int kStreamTile = 256;                       // electrons per tile (128 threads x 2)
 constexpr int kStreamThreads = kStreamTile / 2;
-// Measured on the 3e7-electron, 4000-step one-step job (stages x CTAs per SM, TB/s at 56 B per
-// particle-step), with the emission calls of the step: 2 x 4 4.83, 3 x 3 4.77, 3 x 4 4.60, 2 x 5
-// 4.52, 4 x 4 4.12, 3 x 5 4.14, 2 x 6 3.87 (128 registers took the step without spills, and larger
-// stages shrink the L1 that holds the remaining local memory).  With the emission branches inlined
-// and photons appended in place the step needs 104 registers: 2 x 4 5.48, 2 x 5 5.80, 2 x 6 4.71.
+// Measured on 6e6 electrons, 20 calls of one step in the rising pulse (us a call, the restore of the state included): CTAs
+// x stages 3 x 3 77 (78 with the overlapped launches, which take 1e6 electrons from 24 to 21 us a call), 3 x 2 83, 4 x 3 78, 4 x 2 79, 5 x 2 87, 6 x 2 117 (spills); at the start, without the queue below, 5 x 2
+// 120.  The state's round trip is 49 us at the copy bandwidth.
 #ifndef PE_STREAM_STAGES
-#define PE_STREAM_STAGES 2    // stages per CTA: tiles in flight = stages - 1
+#define PE_STREAM_STAGES 3    // stages per CTA: tiles in flight = stages - 1
 #endif
 #ifndef PE_STREAM_MIN_CTAS
-#define PE_STREAM_MIN_CTAS 5  // resident CTAs of 128 threads per SM the registers are sized for
+#define PE_STREAM_MIN_CTAS 3  // resident CTAs of 128 threads per SM the registers are sized for
 #endif
 constexpr int kStreamStages = PE_STREAM_STAGES;
 // one stage: x pairs (float4 per thread), tau pairs (float4), ux, uy, uz (float2 each)
@@ -1089,6 +1090,23 @@ __device__ __forceinline__ void stage_take(const RunDevT<float>& r, int64_t j, c
     }
 }
 
+// electrons 2j, 2j + 1 from memory as pair_store left them (1D)
+__device__ __forceinline__ void pair_load(const RunDevT<float>& r, int64_t j, Pair& Q) {
+    const float4 x = reinterpret_cast<const float4*>(r.x)[j], tau = reinterpret_cast<const float4*>(r.tau)[j];
+    Q.x = make_float2(x.x, x.z);
+    Q.x_lo = make_float2(x.y, x.w);
+    Q.tau = make_float2(tau.x, tau.z);
+    Q.tau_lo = make_float2(tau.y, tau.w);
+    Q.u0 = reinterpret_cast<const float2*>(r.ux)[j];
+    Q.u1 = reinterpret_cast<const float2*>(r.uy)[j];
+    Q.u2 = reinterpret_cast<const float2*>(r.uz)[j];
+    Q.y = Q.y_lo = P2(0.0f);
+    Q.wait[0] = r.wait ? r.wait[2 * j] : PE_WAIT_NEVER;
+    Q.wait[1] = r.wait ? r.wait[2 * j + 1] : PE_WAIT_NEVER;
+    Q.act[0] = !isnan(Q.x.x);
+    Q.act[1] = !isnan(Q.x.y);
+}
+
 // electrons 2j, 2j + 1 back to memory (both present; removed ones were stored when removed)
 __device__ __forceinline__ void pair_store(const RunDevT<float>& r, int64_t j, const Pair& Q, bool st0, bool st1) {
     if (st0 && st1) {
@@ -1104,22 +1122,69 @@ __device__ __forceinline__ void pair_store(const RunDevT<float>& r, int64_t j, c
     }
 }
 
-template <int G, int F>
+// pairs of a warp whose emissions wait (fewer than 32 left by the last tile and at most 32 more): pair, crossings, eta
+struct StreamQueue {
+    int64_t j[64];
+    float2 eta[64];
+    uint32_t crossed[64];
+};
+
+// kOne: launches of one step.  A pair with an emission is then stored as it is after the push and queued by its warp,
+// which takes the queue 32 emissions at a time, the rest when its tiles are done, and goes through the rest of the step
+// with them, so an emission is not issued for one or two lanes of every third tile (the same job 87 us a call at its best
+// shape without the queue).
+template <int G, int F, bool kOne>
 __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pair_stream(TablesDev t, BatchDevT<float> b,
                                                                                          int steps) {
     extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ StreamQueue s_queue[kOne ? kStreamThreads / 32 : 1];
     const PairShared S(smem, t.n_eta);
     // the stages on a 16-byte boundary after the tables
     const uint32_t table_bytes = kPairFixedBytes + 4 * (t.n_eta + t.n_Z * t.n_E);
     unsigned char* stage_buf = smem + ((table_bytes + 15u) & ~15u);
     const RunDevT<float>& r = b.runs[0];
     S.init(t);
+    // what follows reads the state: the launch of this kernel may overlap the end of the one before
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const SumsCta acc = S.acc();                        // at most 2^31 / grid electrons, 4 steps: far below kSumsMax
 
     const int64_t n_tiles = b.tile_start[1];
     const int64_t n_pairs = r.n >> 1;                   // j < n_pairs: electrons 2j and 2j + 1 both present
     const int64_t stride = (int64_t)gridDim.x * kStreamThreads;
     const float* sig_z = S.sig + (size_t)r.iz * t.n_E;
+    const uint32_t n0 = (uint32_t)r.step0;
+    const int lane = threadIdx.x & 31;
+    StreamQueue& W = s_queue[kOne ? threadIdx.x >> 5 : 0];
+    int queued = 0;                                     // pairs in W (the same on every lane)
+    float2 n_above = P2(0.0f);
+    // the rest of the step after the optical depth, and the pair back to memory
+    auto finish = [&](int64_t j, Pair& Q, float2 gamma, float2 inv_g) {
+        const uint32_t id[2] = {r.id0 + (uint32_t)(2 * j), r.id0 + (uint32_t)(2 * j + 1)};
+        if (brems_on<F>(r)) {
+            const unsigned hit = brems_pair<G, F>(t, r, sig_z, id, n0, Q, gamma, inv_g, acc);
+            if (hit) emit_brems_pair<G, F>(t, r, sig_z, id, n0, hit, Q, gamma, inv_g, acc);
+        }
+        move_pair<G>(r.c, Q, inv_g);
+        if (box_on<F>(r)) box_pair(r, 2 * j, 2 * j + 1, n0, Q, S.tally);
+        pair_store(r, j, Q, Q.act[0], Q.act[1]);
+    };
+    // the last `count` queued pairs, one to a lane
+    auto drain = [&](int count) {
+        if (lane < count) {
+            const int at = queued - count + lane;
+            const int64_t j = W.j[at];
+            Pair Q;
+            pair_load(r, j, Q);
+            float2 gamma, inv_g;
+            gamma_pair(Q, gamma, inv_g);
+            const uint32_t id[2] = {r.id0 + (uint32_t)(2 * j), r.id0 + (uint32_t)(2 * j + 1)};
+            emit_ncs_pair<G, false>(t, r, id, n0, W.crossed[at], Q, gamma, inv_g, W.eta[at], acc);
+            finish(j, Q, gamma, inv_g);
+        }
+        queued -= count;
+        __syncwarp();
+    };
     // tile k of this CTA (k = 0, 1, ...) is tile blockIdx.x + k gridDim.x, staged in stage k mod S;
     // the copies of tiles k + 1 .. k + S - 1 are in flight while tile k is stepped
     const int64_t j0 = (int64_t)blockIdx.x * kStreamThreads + threadIdx.x;
@@ -1144,12 +1209,41 @@ __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pai
             pair_clear(Q);
             if (2 * j < r.n) load_one(r, 2 * j, Q, 0, S.tally);   // the odd last electron
         }
-        const bool live0 = 2 * j < r.n, live1 = full;
-        pair_loop<G, F, false, true>(t, r, S.h, sig_z, 2 * j, 2 * j + 1, Q, steps, acc, S.tally);
-        pair_store(r, j, Q, live0 && Q.act[0], live1 && Q.act[1]);
+        if constexpr (kOne) {
+            unsigned crossed = 0;
+            float2 gamma, inv_g, eta;
+            const bool act = full && (Q.act[0] || Q.act[1]);
+            if (act) crossed = push_pair<G, F>(t, r, S.h, (float)n0, Q, gamma, inv_g, eta, n_above);
+            const unsigned mask = __ballot_sync(0xffffffffu, crossed != 0);
+            if (crossed) {
+                const int at = queued + __popc(mask & ((1u << lane) - 1u));
+                W.j[at] = j;
+                W.eta[at] = eta;
+                W.crossed[at] = crossed;
+                pair_store(r, j, Q, Q.act[0], Q.act[1]);
+            } else if (act) {
+                finish(j, Q, gamma, inv_g);
+            }
+            queued += __popc(mask);
+            __syncwarp();
+            if (queued >= 32) drain(32);
+            if (!full && Q.act[0]) {                    // the odd last electron, alone
+                pair_loop<G, F, false, true>(t, r, S.h, sig_z, 2 * j, 2 * j + 1, Q, 1, acc, S.tally);
+                pair_store(r, j, Q, Q.act[0], false);
+            }
+        } else {
+            const bool live0 = 2 * j < r.n, live1 = full;
+            pair_loop<G, F, false, true>(t, r, S.h, sig_z, 2 * j, 2 * j + 1, Q, steps, acc, S.tally);
+            pair_store(r, j, Q, live0 && Q.act[0], live1 && Q.act[1]);
+        }
         stage = stage + 1 == kStreamStages ? 0 : stage + 1;
     }
     cp_async_wait<0>();
+    if constexpr (kOne) {
+        if (queued) drain(queued);
+        const unsigned int na = __float2uint_rz(n_above.x) + __float2uint_rz(n_above.y);
+        if (na) atomicAdd(S.tally + PE_T_N_ETA_ABOVE, (unsigned long long)na);
+    }
     if (n_tiles > 0) S.flush(r);
 }
 

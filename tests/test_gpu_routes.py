@@ -56,6 +56,43 @@ def test_f64_tables_beyond_shared_memory():
         pe.pe_step_ex([r.handle], 10, steps_per_launch=5)
 
 
+# --------------------------------------------------------------------------- the paired FP32 step ----
+@pytest.mark.parametrize("n", [1, 2, 63, 257, 5_000, 200_003])
+@pytest.mark.parametrize("kind", ["plane", "plane-null-box"])
+def test_one_step_launches_queue_their_emissions(n, kind):
+    """Launches of one step (an emission waits in its warp's queue) equal launches of many."""
+    lt = small_tables()
+    kw = dict(brems_method=pe.PE_BREMS_NULL, box_enable=1, box_x_m=(0.0, 0.9e-6)) if kind != "plane" else {}
+    run = W.base_run(a0=500.0, init_dist=1, seed=n, slab_x0_m=0.1e-6, slab_thick_m=0.7e-6, **kw, **W.AU)
+    outs = []
+    for cfg in (dict(steps_per_launch=1), dict(steps_per_launch=110), dict(steps_per_launch=3)):
+        r = pe.Run(lt, pe.run_params(precision=pe.PE_F32, **run), n, capacity=1 << 21, events=True)
+        pe.pe_step_ex([r.handle], 110, **cfg)
+        outs.append(outcome(r))
+    for o in outs[1:]:
+        same(o, outs[0])
+
+
+@pytest.mark.parametrize("n", [5, 3_001])
+def test_held_emissions_equal_those_taken_at_once(n):
+    """The bunch in Au at dt = T waits for company with its emissions; in a batch with a thin target, or in launches of
+    one step, it does not: the same electrons, photons and sums."""
+    lt = small_tables()
+    dense = dict(W.bunch(1000.0, "Au")["run"])
+    thin = dict(W.bunch(500.0, "Al", dt_over_T=0.1)["run"], run_id=3)
+
+    def bunch(run):
+        return pe.Run(lt, pe.run_params(precision=pe.PE_F32, **run), n, capacity=1 << 18, events=True)
+    alone, steps, mixed, other = bunch(dense), bunch(dense), bunch(dense), bunch(thin)
+    pe.pe_step([alone.handle], 900)
+    pe.pe_step_ex([steps.handle], 900, steps_per_launch=1)
+    pe.pe_step([mixed.handle, other.handle], 900)
+    ref = outcome(alone)
+    assert ref[1].any()
+    same(outcome(steps), ref)
+    same(outcome(mixed), ref)
+
+
 # ------------------------------------------------------------------- binning of the diagnostics ----
 MEC2 = 0.51099895
 
@@ -172,3 +209,38 @@ def test_pic_queue_splits(precision, n, n_cells):
     np.testing.assert_array_equal(outs[0][0], outs[1][0])
     np.testing.assert_array_equal(outs[0][1], outs[1][1])
     assert outs[0][2:] == outs[1][2:]
+
+
+# ------------------------------------------------------------------------- pair production queues ----
+@pytest.mark.parametrize("n", [1, 33, 3_000, 40_001])
+@pytest.mark.parametrize("process", ["bh-direct", "bh-free", "bw-f32", "bw-f64"])
+def test_transport_of_parts_equals_the_whole(process, n):
+    """Photons taken in one call and in two calls of uneven parts convert alike (shares, rounds and queues differ)."""
+    lt = small_tables()
+    kl = 2.0 * np.pi / W.LAMBDA
+    if process.startswith("bh"):
+        run = dict(W.bunch(1000.0, "Au", thickness_m=1e-3)["run"])
+        ph = W.synthetic_photons(n, 5, (0.0, 1500.0), (2.0, 4000.0), (0, 300), theta_max=0.3)
+    else:
+        run = W.base_run(a0=400.0, reflect_r=1.0, mirror_x_m=3e-6, seed=5, **W.AU)
+        ph = W.synthetic_photons(n, 5, (1e-6 * kl, 4e-6 * kl), (100.0, 20000.0), (0, 300), theta_max=0.6)
+    bw = pe.pe_bw_tables_create()
+    r = pe.Run(lt, pe.run_params(precision=pe.PE_F64 if process == "bw-f64" else pe.PE_F32, **run), 16)
+    pe.pe_step([r.handle], 700)
+
+    def go(p):
+        if process.startswith("bw"):
+            return r.bw_transport(bw, photons=p)
+        return r.pair_transport(photons=p, method=int(process == "bh-free"))
+    cut = n // 3
+    whole, parts = go(ph), [go(ph[:cut]), go(ph[cut:])] if cut else [go(ph)]
+    for k, p in enumerate(parts[1:]):
+        p[0]["photon"] += cut
+    got = np.concatenate([p[0] for p in parts])
+    key = lambda a: a[np.argsort(a["photon"])].tobytes()  # noqa: E731
+    assert key(got) == key(whole[0]) and sum(p[1] for p in parts) == whole[1]
+    for w in ("N_ENTERED", "N_K_ABOVE", "N_TESTS"):
+        assert sum(int(p[2][pe.PT[w]]) for p in parts) == int(whole[2][pe.PT[w]])
+    for w in ("E_PAIRS", "E_POSITRONS"):
+        val = lambda t: int(t[pe.PT[w]]) + (int(t[pe.PT[w] + 1]) << 64)  # noqa: E731
+        assert sum(val(p[2]) for p in parts) == val(whole[2])
