@@ -159,10 +159,12 @@ __device__ __forceinline__ R free_steps(R phi, R rate) {
 // pipe, and was done by the one lane that had it: 35 of 35 M FP64 warp instructions, half of the time; queued and done
 // 32 at a time it is 2.4 M.  Measured, 4e5 photons x 2000 steps in the reflected a0 = 400 pulse, two thirds of them
 // converted: 5.5 ms; 4.0 with the votes and the steps ahead of the pulse counted in one go; 2.57 with the queue.
-// What is left is issue (0.8 a cycle), a third of it for lanes that wait for the last photons of a CTA's share.
+// Records lie in order of emission, so the shares are interleaved: 9.6e6 photons of a reflected job 46.9 ms at the start,
+// 41.8 with shares in one piece, 34.1 so. What is left is issue (0.8 a cycle), a third of it at 4e5 photons for lanes
+// that wait for the last photons of a CTA's share.
 template <typename R, int G>
 __global__ void __launch_bounds__(kBwThreads, PE_BW_MIN_CTAS) k_bw_transport(BwDev bw, RunDevT<R> r, const Photon* ph,
-                                                                     int64_t n_ph, int64_t step_end, int64_t share,
+                                                                     int64_t n_ph, int64_t step_end,
                                                                      PairRec* out, int64_t cap,
                                                                      unsigned long long* tally) {
     const StepC<R>& c = r.c;
@@ -216,9 +218,6 @@ __global__ void __launch_bounds__(kBwThreads, PE_BW_MIN_CTAS) k_bw_transport(BwD
         queued -= count;
         __syncwarp();
     };
-    const int64_t j_first = (int64_t)blockIdx.x * share;
-    const int64_t j_left = n_ph - j_first;
-    const unsigned int mine = (unsigned int)(j_left < share ? (j_left > 0 ? j_left : 0) : share);
     unsigned long long n_followed = 0, n_tests = 0, n_above = 0;
     int64_t j = 0;
     bool have = false, more = true;                // a photon in hand; the share may hold another
@@ -239,11 +238,10 @@ __global__ void __launch_bounds__(kBwThreads, PE_BW_MIN_CTAS) k_bw_transport(BwD
                 // a photon to step has k > 2 m c^2, a step left before step_end, and a pulse that can raise its
                 // chi into the table; the others are only counted (no draw)
                 const unsigned int q = first + __popc(need & ((1u << lane) - 1u));
-                more = q < mine;
-                if (more) {
-                    j = j_first + q;
-                    p = ph[j];
-                }
+                // photon q of the CTA: blocks of 32, every gridDim.x-th (records are in order of emission)
+                j = ((int64_t)(q >> 5) * gridDim.x + blockIdx.x) * 32 + (q & 31u);
+                more = j < n_ph;
+                if (more) p = ph[j];
                 if (more && p.e > 2.0f) {                  // the same decision as (double) k > 2
                     ++n_followed;
                     ne = (int64_t)p.step;
@@ -384,12 +382,10 @@ void launch_kind(const BwDev& b, const RunDevT<R>& r, const void* photons, int64
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_bw_transport<R, G>, kBwThreads, 0) != cudaSuccess || occ < 1)
         occ = 1;
-    // equal shares for the resident CTAs; a few photons are spread a warp's worth to a CTA
+    // the resident CTAs share the photons by blocks of 32; a few photons are spread a block to a CTA
     const int64_t blocks = (n + 31) / 32;
-    const int64_t most = blocks < (int64_t)sms * occ ? (blocks > 0 ? blocks : 1) : (int64_t)sms * occ;
-    const int64_t share = (n + most - 1) / most;
-    const int grid = (int)((n + share - 1) / share);
-    k_bw_transport<R, G><<<grid, kBwThreads, 0, s>>>(b, r, static_cast<const Photon*>(photons), n, step_end, share,
+    const int grid = (int)(blocks < (int64_t)sms * occ ? (blocks > 0 ? blocks : 1) : (int64_t)sms * occ);
+    k_bw_transport<R, G><<<grid, kBwThreads, 0, s>>>(b, r, static_cast<const Photon*>(photons), n, step_end,
                                               static_cast<PairRec*>(pairs), cap, tally);
 }
 

@@ -153,8 +153,9 @@ int default_ctas_per_sm_f32(int fk, int block, int smem, int steps_per_launch) {
     int occ = 0;
     cudaError_t e;
     if (stream_shape(fk, steps_per_launch, block, smem)) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step_pair_stream<FK_PLANE_LP, kFlagsPaper, true>, block / 2,
-                                                          stream_smem_bytes(smem));
+        const auto f = k_step_pair_stream<FK_PLANE_LP, kFlagsPaper, true>;
+        allow_smem((const void*)f, stream_smem_bytes(smem));
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, block / 2, stream_smem_bytes(smem));
         return e == cudaSuccess && occ > 0 ? occ : 1;
     }
     with_paired_kind(fk, [&](auto g) {

@@ -1002,14 +1002,14 @@ __global__ void __launch_bounds__(128, (pair_min_ctas<G, F>())) k_step_pair(Tabl
 // ---------------------------------------------------------------------------
 constexpr int kStreamTile = 256;                       // electrons per tile (128 threads x 2)
 constexpr int kStreamThreads = kStreamTile / 2;
-// Measured on 6e6 electrons, 20 calls of one step in the rising pulse (us a call, the restore of the state included): CTAs
-// x stages 3 x 3 77 (78 with the overlapped launches, which take 1e6 electrons from 24 to 21 us a call), 3 x 2 83, 4 x 3 78, 4 x 2 79, 5 x 2 87, 6 x 2 117 (spills); at the start, without the queue below, 5 x 2
-// 120.  The state's round trip is 49 us at the copy bandwidth.
+// Measured on 6e6 / 1e6 electrons, 20 calls of one step in the rising pulse (us a call, the restore of the state included):
+// CTAs x stages 4 x 2 75 / 20.7, 4 x 3 75 / 20.9, 3 x 3 78 / 21.7, 5 x 2 84 / 20.9; at the start, without the queue below
+// and the overlapped launches, 5 x 2 120 / 30. The state's round trip is 49 us at the copy bandwidth.
 #ifndef PE_STREAM_STAGES
-#define PE_STREAM_STAGES 3    // stages per CTA: tiles in flight = stages - 1
+#define PE_STREAM_STAGES 2    // stages per CTA: tiles in flight = stages - 1
 #endif
 #ifndef PE_STREAM_MIN_CTAS
-#define PE_STREAM_MIN_CTAS 3  // resident CTAs of 128 threads per SM the registers are sized for
+#define PE_STREAM_MIN_CTAS 4  // resident CTAs of 128 threads per SM the registers are sized for
 #endif
 constexpr int kStreamStages = PE_STREAM_STAGES;
 // one stage: x pairs (float4 per thread), tau pairs (float4), ux, uy, uz (float2 each)
@@ -1131,8 +1131,7 @@ struct StreamQueue {
 
 // kOne: launches of one step.  A pair with an emission is then stored as it is after the push and queued by its warp,
 // which takes the queue 32 emissions at a time, the rest when its tiles are done, and goes through the rest of the step
-// with them, so an emission is not issued for one or two lanes of every third tile (the same job 87 us a call at its best
-// shape without the queue).
+// with them, so an emission is not issued for one or two lanes of every third tile (the same job 87 us a call at 5 x 2 without the queue).
 template <int G, int F, bool kOne>
 __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pair_stream(TablesDev t, BatchDevT<float> b,
                                                                                          int steps) {
