@@ -51,3 +51,35 @@ def test_nonfinite_momenta_removed_and_counted(precision, launch):
     clean.close()
     bad.close()
     pe.pe_destroy_tables(tables)
+
+
+@pytest.mark.parametrize("precision,launch", [(pe.PE_F32, dict(steps_per_launch=1)), (pe.PE_F32, dict(steps_per_launch=3)),
+                                              (pe.PE_F32, {}), (pe.PE_F64, {})])
+def test_removed_electron_keeps_its_event_word(precision, launch):
+    """An electron whose momentum turns non-finite after some emissions is removed with the event word it has (both
+    electrons of a pair, either of them, and the odd last one), whatever the launch shape."""
+    import torch
+    run = W.base_run(a0=500.0, init_dist=1, seed=3, slab_x0_m=0.1e-6, slab_thick_m=0.7e-6, **W.AU)
+    tables = pe.pe_create_tables(TP, (13.0, 79.0))
+    n = 2001
+    clean = pe.Run(tables, pe.run_params(precision=precision, **run), n, events=True)
+    bad = pe.Run(tables, pe.run_params(precision=precision, **run), n, events=True)
+    for r in (clean, bad):
+        pe.pe_step_ex([r.handle], 110, **launch)
+    words = bad.event_words()
+    np.testing.assert_array_equal(words, clean.event_words())
+    emitted = np.flatnonzero(words)
+    assert len(emitted) > 20
+    ids = np.unique(np.concatenate([emitted[::2], emitted[:6] ^ 1, [n - 1]]))
+    ids = ids[ids < n]
+    bad.uy[torch.from_numpy(ids).to(bad.uy.device)] = float("nan")
+    for r in (clean, bad):
+        pe.pe_step_ex([r.handle], 8, **launch)
+    np.testing.assert_array_equal(bad.event_words()[ids], words[ids])
+    keep = np.setdiff1d(np.arange(n), ids)
+    np.testing.assert_array_equal(bad.event_words()[keep], clean.event_words()[keep])
+    np.testing.assert_array_equal(bad.state()[keep], clean.state()[keep])
+    assert bad.tally_out().tally[pe.T["N_NONFINITE"]] == len(ids)
+    clean.close()
+    bad.close()
+    pe.pe_destroy_tables(tables)
