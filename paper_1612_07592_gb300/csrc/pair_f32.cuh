@@ -194,6 +194,14 @@ __device__ __forceinline__ void repack(Pair& Q, int k, const Particle<float>& P)
     set_comp(Q.tau, k, P.tau); set_comp(Q.tau_lo, k, P.tau_lo);
     if (k) Q.wait[1] = P.wait; else Q.wait[0] = P.wait;
 }
+// The inactive halves of a pair take no further part (see push_pair); in registers only, after what is stored of them.
+template <int G>
+__device__ __forceinline__ void retire(Pair& Q) {
+    if constexpr (G == FK_CONST) {
+        if (!Q.act[0]) Q.u0.x = __int_as_float(0x7fc00000);
+        if (!Q.act[1]) Q.u0.y = __int_as_float(0x7fc00000);
+    }
+}
 // an emission's fingerprint into electron id's word (its thread alone has the electron)
 __device__ __forceinline__ void add_events(const RunDevT<float>& r, uint32_t id, const Particle<float>& P) {
     if (!r.events) return;
@@ -239,9 +247,10 @@ __device__ __forceinline__ bool no_pulse(const StepC<float>& c, float nf, const 
 // rate and the optical depth.  Returns a bit per electron whose optical depth crossed zero (it emits).
 // G = FK_PLANE_LP, FK_PLANE_CP: the 1D plane wave; FK_REFL_LP, FK_REFL_CP: the plane wave and its mirror
 // image; FK_GAUSS_LP, FK_GAUSS_CP: the 2D paraxial focus; FK_CONST: constant fields.  An inactive half of
-// the pair (a removed electron, or an empty slot past the end of the run) has x = NaN, so its fields, momenta,
-// eta and optical depth are NaN from its first step on, and the eta count, the optical depth's crossing and the
-// target test are false for it without reading the activity flags.
+// the pair (a removed electron, or an empty slot past the end of the run) has x = NaN -- and u_x = NaN (retire) in
+// constant fields, which do not depend on x -- so its momenta, gamma and optical depth are NaN from its first step on
+// and its eta NaN or (where a maximum with 0 is taken) 0: the eta count, the optical depth's crossing and the target
+// test are false for it without reading the activity flags.  Nothing of an inactive half is stored.
 template <int G, int F>
 __device__ __forceinline__ unsigned push_pair(const TablesDev& t, const RunDevT<float>& r, const float* h_tab,
                                               float nf, Pair& Q, float2& gamma, float2& inv_g, float2& eta,
@@ -669,6 +678,7 @@ __device__ __forceinline__ void load_one(const RunDevT<float>& r, int64_t i, Pai
 }
 
 // absorbing box (Sec. 3) after a step: a removed electron is stored at once
+template <int G>
 __device__ __forceinline__ void box_pair(const RunDevT<float>& r, int64_t i0, int64_t i1, uint32_t n, Pair& Q,
                                          unsigned long long* s_tally) {
 #pragma unroll
@@ -682,6 +692,7 @@ __device__ __forceinline__ void box_pair(const RunDevT<float>& r, int64_t i0, in
             store_one(r, k ? i1 : i0, P);
         }
     }
+    retire<G>(Q);
 }
 
 // The steps of a warp's electrons before the pulse is at any of them: without a field the push is the identity and eta is
@@ -708,7 +719,7 @@ __device__ __forceinline__ int steps_before_pulse(const TablesDev& t, const RunD
                 if (hit) emit_brems_pair<G, F>(t, r, sig_z, id, n, hit, Q, gamma, inv_g, acc);
             }
             move_pair<G>(r.c, Q, inv_g);
-            if (box_on<F>(r)) box_pair(r, i0, i1, n, Q, s_tally);
+            if (box_on<F>(r)) box_pair<G>(r, i0, i1, n, Q, s_tally);
         }
     }
     return s;
@@ -736,7 +747,7 @@ __device__ __forceinline__ void pair_loop(const TablesDev& t, const RunDevT<floa
                 if (hit) emit_brems_pair<G, F>(t, r, sig_z, id, n, hit, Q, gamma, inv_g, acc);
             }
             move_pair<G>(r.c, Q, inv_g);
-            if (box_on<F>(r)) box_pair(r, i0, i1, n, Q, s_tally);
+            if (box_on<F>(r)) box_pair<G>(r, i0, i1, n, Q, s_tally);
         }
     }
     const unsigned int na = __float2uint_rz(n_above.x) + __float2uint_rz(n_above.y);
@@ -815,7 +826,7 @@ __device__ __forceinline__ void pair_loop_hold(const TablesDev& t, const RunDevT
         if (move) {
             move_pair<G>(r.c, Q, inv_g);
             if (box_on<F>(r)) {
-                box_pair(r, i0, i1, n, Q, s_tally);
+                box_pair<G>(r, i0, i1, n, Q, s_tally);
                 if (!Q.act[0] && !Q.act[1]) left = 1;
             }
             ++n;
@@ -903,6 +914,7 @@ __device__ __forceinline__ void tile_steps_pair(const TablesDev& t, const RunDev
     if (i0 < r.n) load_one(r, i0, Q, 0, s_tally);
     if (i1 < r.n) load_one(r, i1, Q, 1, s_tally);
     if constexpr (G != FK_GAUSS_LP && G != FK_GAUSS_CP) Q.y = Q.y_lo = P2(0.0f);   // 1D: y is not state
+    retire<G>(Q);
     const bool live0 = i0 < r.n, live1 = i1 < r.n;
     if constexpr (kHold)
         pair_loop_hold<G, F>(t, r, s_h, sig_z, i0, i1, Q, steps, acc, held, s_tally);
@@ -1161,7 +1173,7 @@ __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pai
             if (hit) emit_brems_pair<G, F>(t, r, sig_z, id, n0, hit, Q, gamma, inv_g, acc);
         }
         move_pair<G>(r.c, Q, inv_g);
-        if (box_on<F>(r)) box_pair(r, 2 * j, 2 * j + 1, n0, Q, S.tally);
+        if (box_on<F>(r)) box_pair<G>(r, 2 * j, 2 * j + 1, n0, Q, S.tally);
         pair_store(r, j, Q, Q.act[0], Q.act[1]);
     };
     // the last `count` queued pairs, one to a lane

@@ -83,3 +83,34 @@ def test_removed_electron_keeps_its_event_word(precision, launch):
     clean.close()
     bad.close()
     pe.pe_destroy_tables(tables)
+
+
+@pytest.mark.parametrize("method", [pe.PE_BREMS_DIRECT, pe.PE_BREMS_NULL])
+@pytest.mark.parametrize("precision,dense,launch", [(pe.PE_F32, False, {}), (pe.PE_F32, False, dict(steps_per_launch=20)),
+                                                    (pe.PE_F32, True, {}), (pe.PE_F64, False, {})])
+def test_removed_electron_takes_no_part_in_constant_fields(precision, dense, launch, method):
+    """Electrons leave the box at different times while their partners in a pair go on: the removed ones emit nothing,
+    keep their event words and are not counted (the fields of PE_CONST do not depend on the position).  dense: a target in
+    which the lanes wait for one another's emissions.  The field lies along x (electrons leave along it) and every eta,
+    u_perp B / E_S, is above the table, so N_ETA_ABOVE counts the steps of the live electrons."""
+    tables = pe.pe_create_tables(dict(TP, eta_min=1e-6, eta_max=1e-5), (13.0, 79.0))
+    target = dict(Z=79.0, charge_state=79.0, ne_over_nc=4177.0 * (50.0 if dense else 0.02))
+    run = W.base_run(geometry=pe.PE_CONST, B_const=(2000.0, 0.0, 0.0), init_dist=1, seed=5, slab_x0_m=0.1e-6,
+                     slab_thick_m=0.7e-6, box_enable=1, box_x_m=(0.0, 0.9e-6), brems_method=method, **target)
+    n, steps = 3001, 60
+    r = pe.Run(tables, pe.run_params(precision=precision, **run), n, events=True)
+    x, words, emissions = np.zeros(n), np.zeros(n, np.uint64), 0
+    for _ in range(4):
+        pe.pe_step_ex([r.handle], steps, **launch)
+        gone = np.isnan(x)
+        w = r.event_words()
+        np.testing.assert_array_equal(w[gone], words[gone])
+        x, words = r.state()[:, 0], w
+        t = r.tally_out()
+        assert t.tally[pe.T["N_ETA_ABOVE"]] == t.live_particle_steps
+        emissions = sum(int(t.tally[pe.T[k]]) for k in ("N_NCS_STORED", "N_NCS_BELOW", "N_BR_STORED", "N_BR_BELOW"))
+        assert emissions == int((words & np.uint64(0xFFFF)).sum() + ((words >> np.uint64(16)) & np.uint64(0xFFFF)).sum())
+        assert np.isfinite(r.photon_records()["x"]).all()
+    assert emissions > 500 and 0 < np.isnan(x).sum()
+    r.close()
+    pe.pe_destroy_tables(tables)
