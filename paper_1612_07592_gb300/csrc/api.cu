@@ -624,9 +624,10 @@ static void set_step0(PlanLaunch& L, pe_run* const* runs, int64_t base_extra) {
 }
 
 // persistent launches (grouped by field kind, chunked by steps_per_launch)
-// (any_tables: FP64 rate tables that do not fit shared memory stay in global memory; otherwise they are refused)
+// (lone_f64: one FP64 run without a number of steps per launch; its rate tables may be larger than shared memory, and
+// non-finite momenta are removed at the step they appear before, whatever the launches)
 static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, const pe_launch_config* cfg,
-                            bool any_tables, Plan& plan) {
+                            bool lone_f64, Plan& plan) {
     const pe_tables* t = runs[0]->tables;
     int prec = runs[0]->params.precision;
     int block = (cfg && cfg->block > 0) ? cfg->block : 256;          // electrons per tile
@@ -644,7 +645,7 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
     }
     int smem = persistent_smem_bytes(t->dev, prec);
     const bool staged = smem <= 200 * 1024;
-    if (!staged && any_tables)
+    if (!staged && lone_f64)
         smem = kSumsBytesF64;
     else if (!staged)
         return fail(PE_ERR_ARG, "pe_step: rate tables (n_eta + n_Z * n_E) too large for shared memory");
@@ -689,6 +690,7 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
                 std::memset(L.bd.get(), 0, sizeof(BatchDevT<double>));
                 L.bd->n_runs = m;
                 L.bd->staged = staged;
+                L.bd->each_step = lone_f64;
                 L.bd->tile = block;
                 for (int k = 0; k <= m; ++k) L.bd->tile_start[k] = tile_start[k];
                 for (int k = 0; k < m; ++k) L.bd->runs[k] = runs[idx[k]]->dev;

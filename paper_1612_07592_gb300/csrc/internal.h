@@ -126,6 +126,7 @@ struct BatchDevT {
     int n_runs;
     int tile;                           // particles per tile
     int staged;                         // FP64: the rate tables are copied to shared memory
+    int each_step;                      // FP64: non-finite momenta are looked for before every step, not every launch
     int64_t tile_start[PE_MAX_BATCH + 1];
     RunDevT<R> runs[PE_MAX_BATCH];
 };

@@ -114,3 +114,28 @@ def test_removed_electron_takes_no_part_in_constant_fields(precision, dense, lau
     assert emissions > 500 and 0 < np.isnan(x).sum()
     r.close()
     pe.pe_destroy_tables(tables)
+
+
+@pytest.mark.parametrize("n,calls", [(70, (400,)), (70, (100, 300)), (70, (1,) * 400)])
+def test_momenta_that_overflow_within_a_call(n, calls):
+    """An FP64 run alone looks for non-finite momenta before every step, however many steps a call does: electrons that a
+    huge constant field drives beyond the largest double are removed at that step and counted in that call."""
+    E, dt = 1e307, 0.01 * 2 * np.pi
+    tables = pe.pe_create_tables(TP, (13.0, 79.0))
+    run = W.base_run(geometry=pe.PE_CONST, E_const=(E, 0.0, 0.0), enable_ncs=0, enable_brems=0, **W.AU)
+    r = pe.Run(tables, pe.run_params(precision=pe.PE_F64, **run), n, events=True)
+    for k in calls:
+        pe.pe_step([r.handle], k)
+    u, alive = 0.0, 0
+    with np.errstate(over="ignore"):
+        while np.isfinite(u):                       # two half kicks a step; the first steps to end beyond the range
+            u = (u - 0.5 * dt * E) - 0.5 * dt * E
+            alive += 1
+    assert 10 < alive < 390
+    t = r.tally_out()
+    assert t.tally[pe.T["N_NONFINITE"]] == t.tally[pe.T["N_KILLED"]] == n
+    assert t.tally[pe.T["KILLED_STEPS"]] == n * alive
+    s = r.state()
+    assert np.isnan(s[:, 0]).all() and (s[:, 2:5] == 0).all()
+    r.close()
+    pe.pe_destroy_tables(tables)
