@@ -628,15 +628,23 @@ __device__ __forceinline__ void store_particle(const RunDevT<R>& r, int64_t i, c
 // overflowed) is removed here: x = NaN, momenta zeroed so it is counted once, stored back,
 // and counted in N_NONFINITE and N_KILLED with its n steps alive.
 template <typename R>
-__device__ __forceinline__ bool live_or_kill(const RunDevT<R>& r, int64_t i, Particle<R>& P, uint32_t n,
-                                             unsigned long long* tally) {
-    if (isfinite(P.u[0]) && isfinite(P.u[1]) && isfinite(P.u[2])) return !isnan(P.x);
+__device__ __forceinline__ bool finite_momenta(const Particle<R>& P) {
+    return isfinite(P.u[0]) && isfinite(P.u[1]) && isfinite(P.u[2]);
+}
+template <typename R>
+__device__ __forceinline__ void kill_nonfinite(Particle<R>& P, uint32_t n, unsigned long long* tally) {
     P.x = (R)NAN;
     P.u[0] = P.u[1] = P.u[2] = (R)0;
-    store_particle<R>(r, i, P);
     atomicAdd(tally + PE_T_N_NONFINITE, 1ull);
     atomicAdd(tally + PE_T_N_KILLED, 1ull);
     atomicAdd(tally + PE_T_KILLED_STEPS, (unsigned long long)n);
+}
+template <typename R>
+__device__ __forceinline__ bool live_or_kill(const RunDevT<R>& r, int64_t i, Particle<R>& P, uint32_t n,
+                                             unsigned long long* tally) {
+    if (finite_momenta(P)) return !isnan(P.x);
+    kill_nonfinite(P, n, tally);
+    store_particle<R>(r, i, P);
     return false;
 }
 

@@ -1094,7 +1094,14 @@ __device__ __forceinline__ void stage_take(const RunDevT<float>& r, int64_t j, c
     Q.act[1] = !isnan(Q.x.y);
     if (!finite3(Q.u0.x, Q.u1.x, Q.u2.x) || !finite3(Q.u0.y, Q.u1.y, Q.u2.y)) {
 #pragma unroll
-        for (int k = 0; k < 2; ++k) load_one(r, 2 * j + k, Q, k, tally);   // rare: remove and count; with the event word
+        for (int k = 0; k < 2; ++k) {             // rare: remove and count (as live_or_kill; the event word stays)
+            Particle<float> P = unpack(Q, k);
+            if (finite_momenta(P)) continue;
+            kill_nonfinite(P, (uint32_t)r.step0, tally);
+            store_one(r, 2 * j + k, P);
+            Q.act[k] = false;
+            repack(Q, k, P);
+        }
     }
 }
 
