@@ -109,12 +109,13 @@ __device__ __forceinline__ int log_bin(double v, double ln_lo, double inv_dln, i
 struct FastBin {
     float ln_lo, inv_dln, eps;     // position = (ln v - ln_lo) inv_dln, off by at most eps + 3e-7 |position|
 };
-// bin of e (in units of m c^2; scale = ln of m c^2 in MeV) or kUnsure.  Errors of ln v - ln_lo: e itself 6e-7 relative,
-// lg2.approx 2^-22 and half an ulp of a result below 64 (1.9e-6 ln 2), the FMA's and the difference's rounding (1.9e-6
-// each): below 5.9e-6, taken as 8e-6 in eps.
+// bin of e (in units of m c^2; scale = ln of m c^2 in MeV) or kUnsure.  Errors of ln v - ln_lo for e < 2^25 (17 TeV):
+// e itself 6e-7 relative, lg2.approx 2^-22 of its result (4.2e-6) and the result's rounding to float (0.7e-6), the FMA's
+// rounding (1e-6): below 6.5e-6, taken as 8e-6 in eps; the difference's and ln_lo's own rounding are in eps's other terms.
+// Further up the logarithm's documented error grows with its result, beyond eps: those bins are the FP64 form's.
 constexpr int kUnsure = INT_MIN;
 __device__ __forceinline__ int fast_log_bin(const FastBin& f, float e, float scale) {
-    if (!(e > 1e-6f && e < 1e18f)) return kUnsure;
+    if (!(e > 1e-6f && e < 0x1p25f)) return kUnsure;
     const float pos = (fmaf(__log2f(e), 0.693147180559945309f, scale) - f.ln_lo) * f.inv_dln;
     const float fl = floorf(pos), w = pos - fl, eps = f.eps + 3e-7f * fabsf(pos);
     return w > eps && w < 1.0f - eps && fabsf(pos) < 1e6f ? (int)fl : kUnsure;

@@ -588,3 +588,44 @@ def test_phase_beyond_8192_steps_within_stated_rounding():
 @pytest.mark.parametrize("mistake", ["x_lo dropped", "dt_lo dropped", "mirror low part sign"])
 def test_phase_bound_catches_mistakes(mistake):
     assert phase_errors([1, 1234, 4000, 8191], mistake) > 1.0
+
+
+# ------------------------------------------------- bins of the diagnostics from a float position ----
+def fast_log_bin_source():
+    """The range in which the float position may name the bin, from the source."""
+    import os
+    import re
+    path = os.path.join(os.path.dirname(__file__), "..", "paper_1612_07592_gb300", "csrc", "kernels.cu")
+    lo, hi = re.search(r"if \(!\(e > (\S+)f && e < (\S+)f\)\) return kUnsure;", open(path).read()).groups()
+    return float(lo), float.fromhex(hi) if "x" in hi else float(hi)
+
+
+def float_position(e, ln_lo, inv_dln, sign):
+    """pos of fast_log_bin (physics: e in m c^2, ln_lo in MeV) with lg2.approx at its documented bound, 2^-22 absolute in
+    [1/2, 2] and 2^-22 relative outside, and e itself 6e-7 off, all errors to one side."""
+    l2 = np.log2(e.astype(np.float64) * (1.0 + sign * 6e-7))
+    l2 = (l2 + sign * 2.0 ** -22 * np.maximum(np.abs(l2), 1.0)).astype(F)
+    v = (l2.astype(np.float64) * F(0.693147180559945309) + np.float64(F(-0.671387683))).astype(F)
+    return (v - F(ln_lo)) * F(inv_dln)
+
+
+@pytest.mark.parametrize("sign", [-1.0, 1.0])
+@pytest.mark.parametrize("span", [1.05, 10.0, 1e6])
+def test_float_bin_positions_are_within_their_error(sign, span):
+    """Where the float position is taken to name the bin, it is the bin of the exact logarithm, over the whole range in
+    which it is taken, for energy ranges that begin anywhere in it."""
+    e_min, e_max = fast_log_bin_source()
+    rng = np.random.default_rng(int(span))
+    mev = 0.51099895
+    for lo in np.exp(np.linspace(np.log(e_min), np.log(e_max / 1.01), 60)) * mev:
+        bins = 64
+        ln_lo, inv_dln = np.log(lo), bins / np.log(span)
+        # values within 3e-5 of the edges (the float form's error in ln e is of that order)
+        e = (lo / mev * np.exp(rng.integers(0, bins, 4000) / inv_dln + rng.uniform(-3e-5, 3e-5, 4000))).astype(F)
+        e = e[(e > F(e_min)) & (e < F(e_max))]
+        pos = float_position(e, ln_lo, inv_dln, sign)
+        eps = F(F(inv_dln * (8e-6 + 1.2e-7 * abs(ln_lo))) + F(3e-7) * np.abs(pos))
+        w = pos - np.floor(pos)
+        sure = (w > eps) & (w < F(1.0) - eps)
+        exact = (np.log(e.astype(np.float64) * mev) - ln_lo) * inv_dln
+        np.testing.assert_array_equal(np.floor(pos[sure]), np.floor(exact[sure]))
