@@ -624,8 +624,8 @@ static void set_step0(PlanLaunch& L, pe_run* const* runs, int64_t base_extra) {
 }
 
 // persistent launches (grouped by field kind, chunked by steps_per_launch)
-// (lone_f64: one FP64 run without a number of steps per launch; its rate tables may be larger than shared memory, and
-// non-finite momenta are removed at the step they appear before, whatever the launches)
+// (lone_f64: one FP64 run without a number of steps per launch; its rate tables may have any size, and non-finite
+// momenta are removed at the step they appear before, whatever the launches)
 static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, const pe_launch_config* cfg,
                             bool lone_f64, Plan& plan) {
     const pe_tables* t = runs[0]->tables;
@@ -643,13 +643,9 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
         for (int k = 0; k < n_runs; ++k) n_all += runs[k]->dev.n;
         block = default_tile_f64(n_all, sms);
     }
-    int smem = persistent_smem_bytes(t->dev, prec);
-    const bool staged = smem <= 200 * 1024;
-    if (!staged && lone_f64)
-        smem = kSumsBytesF64;
-    else if (!staged)
+    if (rate_table_bytes(t->dev, prec) > 200 * 1024 - 8 * (PE_HIST_WORDS + PE_TALLY_WORDS) && !lone_f64)
         return fail(PE_ERR_ARG, "pe_step: rate tables (n_eta + n_Z * n_E) too large for shared memory");
-    if (prec == PE_F32) smem = pair_smem_bytes(t->dev);
+    const int smem = prec == PE_F32 ? pair_smem_bytes(t->dev) : 0;
     for (int fk = 0; fk < kFieldKinds; ++fk) {
         std::vector<int> idx;
         for (int k = 0; k < n_runs; ++k)
@@ -665,7 +661,7 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
         // resident CTAs of the one-electron kernel, so the block scheduler evens out tiles of unequal cost
         int per_sm = (cfg && cfg->ctas_per_sm > 0) ? cfg->ctas_per_sm
                                                   : (prec == PE_F32 ? default_ctas_per_sm_f32(fk, block, smem, K)
-                                                                    : 2 * persistent_occupancy_f64(block, smem));
+                                                                    : 2 * persistent_occupancy_f64(block));
         if (per_sm < 1) per_sm = 1;
         int grid = (int)std::min<int64_t>(n_tiles, (int64_t)sms * per_sm);
         for (int64_t done = 0; done < n_steps; done += K) {
@@ -681,7 +677,6 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
                 L.bf.reset(new BatchDevT<float>());
                 std::memset(L.bf.get(), 0, sizeof(BatchDevT<float>));
                 L.bf->n_runs = m;
-                L.bf->staged = staged;
                 L.bf->tile = block;
                 for (int k = 0; k <= m; ++k) L.bf->tile_start[k] = tile_start[k];
                 for (int k = 0; k < m; ++k) L.bf->runs[k] = to_float(runs[idx[k]]->dev);
@@ -689,7 +684,6 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
                 L.bd.reset(new BatchDevT<double>());
                 std::memset(L.bd.get(), 0, sizeof(BatchDevT<double>));
                 L.bd->n_runs = m;
-                L.bd->staged = staged;
                 L.bd->each_step = lone_f64;
                 L.bd->tile = block;
                 for (int k = 0; k <= m; ++k) L.bd->tile_start[k] = tile_start[k];
@@ -758,7 +752,7 @@ extern "C" pe_status pe_step_ex(pe_run* const* runs, int n_runs, int64_t n_steps
         if (L.prec == PE_F32)
             launch_step_persistent_f32(t->dev, *L.bf, L.steps, L.grid, L.block, s);
         else
-            launch_step_persistent_f64(t->dev, *L.bd, L.steps, L.grid, L.block, L.smem, s);
+            launch_step_persistent_f64(t->dev, *L.bd, L.steps, L.grid, L.block, s);
         g_launches++;
     }
     cudaError_t e = cudaGetLastError();
@@ -992,7 +986,7 @@ extern "C" pe_status pe_graph_create(pe_run* const* runs, int n_runs, int64_t st
         int smem = L.smem;
         p.func = const_cast<void*>(L.prec == PE_F32 ? persistent_kernel_f32(*L.bf, L.steps, L.smem, L.block, &threads,
                                                                             &smem)
-                                                    : persistent_kernel_f64(*L.bd, L.smem, L.block, &threads));
+                                                    : persistent_kernel_f64(*L.bd));
         p.gridDim = dim3(L.grid);
         p.blockDim = dim3(threads);
         p.sharedMemBytes = smem;

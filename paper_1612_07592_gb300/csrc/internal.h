@@ -125,7 +125,6 @@ template <typename R>
 struct BatchDevT {
     int n_runs;
     int tile;                           // particles per tile
-    int staged;                         // FP64: the rate tables are copied to shared memory
     int each_step;                      // FP64: non-finite momenta are looked for before every step, not every launch
     int64_t tile_start[PE_MAX_BATCH + 1];
     RunDevT<R> runs[PE_MAX_BATCH];
@@ -207,15 +206,14 @@ void launch_init(const RunDev& r, int precision, int init_dist, double theta, do
 void launch_step_persistent_f32(const TablesDev& t, const BatchDevT<float>& b, int steps, int grid, int block,
                                 cudaStream_t s);
 void launch_step_persistent_f64(const TablesDev& t, const BatchDevT<double>& b, int steps, int grid, int block,
-                                int smem, cudaStream_t s);
-constexpr int kSumsBytesF64 = 8 * (PE_HIST_WORDS + PE_TALLY_WORDS);
-int persistent_smem_bytes(const TablesDev& t, int precision);   // the FP64 kernels
+                                cudaStream_t s);
+size_t rate_table_bytes(const TablesDev& t, int precision);       // h(eta) and sigma_Z(gamma)
 int pair_smem_bytes(const TablesDev& t);                          // the paired FP32 kernels
 int default_ctas_per_sm_f32(int fk, int block, int smem, int steps_per_launch);
 const void* persistent_kernel_f32(const BatchDevT<float>& b, int steps, int smem, int block, int* threads,
                                   int* smem_out);
-const void* persistent_kernel_f64(const BatchDevT<double>& b, int smem, int block, int* threads);
-int persistent_occupancy_f64(int block, int smem);
+const void* persistent_kernel_f64(const BatchDevT<double>& b);
+int persistent_occupancy_f64(int block);
 int default_tile_f64(int64_t n, int sms);
 
 }  // namespace pe

@@ -80,9 +80,8 @@ void launch_init(const RunDev& r, int precision, int init_dist, double theta, do
         k_init<double><<<grid, 256, 0, s>>>(r, init_dist, theta, beam_u);
 }
 
-int persistent_smem_bytes(const TablesDev& t, int precision) {
-    size_t rs = precision == PE_F32 ? 4 : 8;
-    return (int)(kSumsBytesF64 + rs * (t.n_eta + (size_t)t.n_Z * t.n_E));
+size_t rate_table_bytes(const TablesDev& t, int precision) {
+    return (precision == PE_F32 ? 4 : 8) * (t.n_eta + (size_t)t.n_Z * t.n_E);
 }
 
 }  // namespace pe

@@ -3,14 +3,12 @@
 //  k_init            one thread per particle: initial position, momentum and
 //                    optical depth from the particle's Philox stream.
 //  k_step_persistent FP64: grid-stride over tiles of one or many runs, K steps per
-//                    launch with the particle state in registers, the rate
-//                    tables (h(eta), sigma_Z(gamma)) staged in shared memory,
-//                    photons appended inside the emission branch (one atomic per
+//                    launch with the particle state in registers, photons
+//                    appended inside the emission branch (one atomic per
 //                    group of lanes there together), histograms and tallies
 //                    accumulated in shared memory and flushed once per run per
-//                    CTA.  The FP32 step runs on the
-//                    paired kernels (pair_f32.cuh), and the FP32 PIC kernel
-//                    uses step_one below.
+//                    CTA.  The FP32 step runs on the paired kernels (pair_f32.cuh),
+//                    the PIC kernel on the two halves of step_one.
 //
 // Step order per particle (Sec. 2.2): fields at (x^n, t^n) -> Boris push ->
 // eta -> NCS optical depth (emission at tau <= 0) -> brems test (Eq. 4) ->
@@ -707,23 +705,17 @@ __device__ __forceinline__ void tile_steps(const TablesDev& t, const RunDevT<R>&
 #endif
 template <typename R, bool kSingle, int G, bool kCommon = false>
 __global__ void __launch_bounds__(256, PE_MIN_CTAS) k_step_persistent(TablesDev t, BatchDevT<R> b, int steps) {
-    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ unsigned long long s_hist[PE_HIST_WORDS];
+    __shared__ unsigned long long s_tally[PE_TALLY_WORDS];
     __shared__ RunDevT<R> s_run;
-    unsigned long long* s_hist = reinterpret_cast<unsigned long long*>(smem);
-    unsigned long long* s_tally = s_hist + PE_HIST_WORDS;
-    R* s_h = reinterpret_cast<R*>(s_tally + PE_TALLY_WORDS);
-    R* s_sig = s_h + t.n_eta;
-    const R* g_h = (sizeof(R) == 4) ? (const R*)t.h32 : (const R*)t.h64;
-    const R* g_sig = (sizeof(R) == 4) ? (const R*)t.sig32 : (const R*)t.sig64;
-
-    for (int k = threadIdx.x; k < PE_HIST_WORDS + PE_TALLY_WORDS; k += blockDim.x) s_hist[k] = 0;
-    if (b.staged) {
-        for (int k = threadIdx.x; k < t.n_eta; k += blockDim.x) s_h[k] = g_h[k];
-        for (int k = threadIdx.x; k < t.n_Z * t.n_E; k += blockDim.x) s_sig[k] = g_sig[k];
-    }
+    for (int k = threadIdx.x; k < PE_HIST_WORDS; k += blockDim.x) s_hist[k] = 0;
+    for (int k = threadIdx.x; k < PE_TALLY_WORDS; k += blockDim.x) s_tally[k] = 0;
     __syncthreads();
-    const R* h_tab = b.staged ? s_h : g_h;                     // tables too large for shared memory are read where they are
-    const R* sig_tab = b.staged ? s_sig : g_sig;
+    // The rate tables are read where they are: a step takes two of their values beside some 13000 clocks of FP64
+    // operations, and a copy in shared memory costs resident CTAs: 7e4 electrons, 40 steps, tables of 12 / 24 / 40 / 192 KB
+    // 1.18 / 1.23 / 4.23 / 4.31 ms with the copy, 1.14 without whatever their size (1e4 electrons 0.37 to 0.97 and 0.36).
+    const R* h_tab = t.h64;
+    const R* sig_tab = t.sig64;
 
     const int64_t n_tiles = b.tile_start[b.n_runs];
     int cur = -1;

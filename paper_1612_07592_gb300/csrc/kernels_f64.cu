@@ -12,35 +12,23 @@ namespace pe {
 // ---------------------------------------------------------------------------
 // persistent kernel for double
 // ---------------------------------------------------------------------------
-template <bool kSingle, int G>
-static const void* kernel_f64() {
-    return (const void*)k_step_persistent<double, kSingle, G>;
-}
-
 void launch_step_persistent_f64(const TablesDev& t, const BatchDevT<double>& b, int steps, int grid, int block,
-                                int smem, cudaStream_t s) {
+                                cudaStream_t s) {
     // all runs of b share one field kind (the caller groups a batch by kind)
     with_field_kind(b.runs[0].fk, [&](auto g) {
         constexpr int G = decltype(g)::value;
-        if (b.n_runs == 1) {
-            if (smem > 40 * 1024) cudaFuncSetAttribute(kernel_f64<true, G>(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            k_step_persistent<double, true, G><<<grid, block, smem, s>>>(t, b, steps);
-        } else {
-            if (smem > 40 * 1024) cudaFuncSetAttribute(kernel_f64<false, G>(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            k_step_persistent<double, false, G><<<grid, block, smem, s>>>(t, b, steps);
-        }
+        if (b.n_runs == 1) k_step_persistent<double, true, G><<<grid, block, 0, s>>>(t, b, steps);
+        else k_step_persistent<double, false, G><<<grid, block, 0, s>>>(t, b, steps);
     });
 }
 
-// the kernel a launch of these runs uses (for graph nodes); sets the shared-memory attribute
-const void* persistent_kernel_f64(const BatchDevT<double>& b, int smem, int block, int* threads) {
-    *threads = block;
+// the kernel a launch of these runs uses (for graph nodes)
+const void* persistent_kernel_f64(const BatchDevT<double>& b) {
     const void* f = nullptr;
     with_field_kind(b.runs[0].fk, [&](auto g) {
         constexpr int G = decltype(g)::value;
-        f = b.n_runs == 1 ? kernel_f64<true, G>() : kernel_f64<false, G>();
+        f = b.n_runs == 1 ? (const void*)k_step_persistent<double, true, G> : (const void*)k_step_persistent<double, false, G>;
     });
-    if (smem > 40 * 1024) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     return f;
 }
 
@@ -52,9 +40,9 @@ const void* persistent_kernel_f64(const BatchDevT<double>& b, int smem, int bloc
 // formed for every brems test took 23 us a step on 1e4 electrons (the 2000-step job 46.5 ms, now 12.9).
 int default_tile_f64(int64_t n, int sms) { return n <= (int64_t)sms * 512 ? 32 : 256; }
 
-int persistent_occupancy_f64(int block, int smem) {
+int persistent_occupancy_f64(int block) {
     int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step_persistent<double, false, FK_PLANE_LP>, block, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step_persistent<double, false, FK_PLANE_LP>, block, 0);
     return e == cudaSuccess ? occ : 1;
 }
 

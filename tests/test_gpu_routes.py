@@ -56,6 +56,34 @@ def test_f64_tables_beyond_shared_memory():
         pe.pe_step_ex([r.handle], 10, steps_per_launch=5)
 
 
+@pytest.mark.parametrize("n_E,n_z", [(512, 1), (2048, 2), (3500, 4), (3840, 6)])
+def test_f64_rate_tables_of_every_size(n_E, n_z):
+    """FP64 runs read the rate tables where they are: alone, in launches of 7 steps, in a batch and replayed from a graph they
+    give the same results with tables of 12 to 192 KB."""
+    lt = pe.pe_create_tables(dict(W.tables_small(), n_eta=1024, n_y=16, n_E=n_E, n_s=16), tuple(79.0 - k for k in range(n_z)))
+    run = W.base_run(a0=270.0, init_dist=1, seed=5, slab_x0_m=0.1e-6, slab_thick_m=0.7e-6, **W.AU)
+    n, steps, outs = 700, 126, []
+    for how in ("alone", "launches", "batch", "graph"):
+        r = pe.Run(lt, pe.run_params(precision=pe.PE_F64, **run), n, events=True)
+        if how == "alone":
+            pe.pe_step([r.handle], steps)
+        elif how == "launches":
+            pe.pe_step_ex([r.handle], steps, steps_per_launch=7)
+        elif how == "batch":
+            other = pe.Run(lt, pe.run_params(precision=pe.PE_F64, **dict(run, run_id=1)), 50)
+            pe.pe_step([r.handle, other.handle], steps)
+        else:
+            g = pe.pe_graph_create([r.handle], steps // 2)
+            pe.pe_graph_launch(g)
+            pe.pe_graph_launch(g)
+        outs.append(outcome(r))
+        if how == "graph":
+            pe.pe_graph_destroy(g)
+    assert outs[0][1].any()
+    for o in outs[1:]:
+        same(o, outs[0])
+
+
 # --------------------------------------------------------------------------- the paired FP32 step ----
 @pytest.mark.parametrize("n", [1, 2, 63, 257, 5_000, 200_003])
 @pytest.mark.parametrize("kind", ["plane", "plane-null-box"])
