@@ -14,18 +14,16 @@ namespace pe {
 // of a plane-wave kind use the streaming form of the paired kernel.
 constexpr int kStreamMaxSteps = 4;
 
-int pair_smem_bytes(const TablesDev& t) { return kPairFixedBytes + 4 * (t.n_eta + t.n_Z * t.n_E); }
+int pair_smem_bytes(const TablesDev& t) { return kPairFixedBytes + 4 * (t.n_eta + t.n_E); }   // 54 KB at most (4096 rows)
 
 static bool plane_kind(int fk) { return fk == FK_PLANE_LP || fk == FK_PLANE_CP; }
 // tables, then 16-byte alignment slack and the stage buffers
 static int stream_smem_bytes(int base) { return base + 16 + kStreamStages * kStageBytes; }
-// (rate tables that leave no room for the stages and queues run on the resident form: the same results)
-static bool stream_shape(int fk, int steps, int block, int base_smem) {
-    return plane_kind(fk) && steps <= kStreamMaxSteps && block == kStreamTile &&
-           stream_smem_bytes(base_smem) + (int)sizeof(StreamQueue) * (kStreamThreads / 32) <= 227 * 1024;
+static bool stream_shape(int fk, int steps, int block) {
+    return plane_kind(fk) && steps <= kStreamMaxSteps && block == kStreamTile;
 }
-static bool use_stream(const BatchDevT<float>& b, int steps, int block, int base_smem) {
-    return b.n_runs == 1 && stream_shape(b.runs[0].fk, steps, block, base_smem);
+static bool use_stream(const BatchDevT<float>& b, int steps, int block) {
+    return b.n_runs == 1 && stream_shape(b.runs[0].fk, steps, block);
 }
 // beside the static shared memory of a kernel (below 6 KB) a launch may use 48 KB without being told so
 static void allow_smem(const void* f, int smem) {
@@ -68,7 +66,7 @@ static StepKernel kernel_of(const BatchDevT<float>& b, int steps, int block, int
     threads = block / 2;
     const int flags = flags_of(b);
     if constexpr (G == FK_PLANE_LP || G == FK_PLANE_CP) {
-        if (kSingle && use_stream(b, steps, block, base_smem)) {
+        if (kSingle && use_stream(b, steps, block)) {
             smem = stream_smem_bytes(base_smem);
             if (steps == 1)
                 return flags == kFlagsPaper ? k_step_pair_stream<G, kFlagsPaper, true> : k_step_pair_stream<G, kFlagsRun, true>;
@@ -103,7 +101,7 @@ static void launch_one(const TablesDev& t, const BatchDevT<float>& b, int steps,
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = kSingle && use_stream(b, steps, block, base_smem) ? 1 : 0;
+    cfg.numAttrs = kSingle && use_stream(b, steps, block) ? 1 : 0;
     cudaLaunchKernelEx(&cfg, f, t, b, steps);
 }
 
@@ -152,7 +150,7 @@ const void* persistent_kernel_f32(const BatchDevT<float>& b, int steps, int base
 int default_ctas_per_sm_f32(int fk, int block, int smem, int steps_per_launch) {
     int occ = 0;
     cudaError_t e;
-    if (stream_shape(fk, steps_per_launch, block, smem)) {
+    if (stream_shape(fk, steps_per_launch, block)) {
         const auto f = k_step_pair_stream<FK_PLANE_LP, kFlagsPaper, true>;
         allow_smem((const void*)f, stream_smem_bytes(smem));
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, block / 2, stream_smem_bytes(smem));
@@ -160,8 +158,9 @@ int default_ctas_per_sm_f32(int fk, int block, int smem, int steps_per_launch) {
     }
     with_paired_kind(fk, [&](auto g) {
         constexpr int G = decltype(g)::value;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &occ, k_step_pair<true, G, kFlagsPaper, G == FK_REFL_LP || G == FK_REFL_CP>, block / 2, smem);
+        const auto f = k_step_pair<true, G, kFlagsPaper, G == FK_REFL_LP || G == FK_REFL_CP>;
+        allow_smem((const void*)f, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, block / 2, smem);
     });
     return 3 * (e == cudaSuccess && occ > 0 ? occ : 1);
 }

@@ -845,8 +845,10 @@ __device__ __forceinline__ void pair_clear(Pair& Q) {
     Q.act[0] = Q.act[1] = false;
 }
 
-// Shared memory of the paired kernels: the CTA's sums, the held lanes' slots, the rate tables (kPairFixedBytes,
-// then h(eta) and sigma_Z(gamma)); a multiple of 16 bytes up to the tables.
+// Shared memory of the paired kernels: the CTA's sums and the held lanes' slots (kPairFixedBytes, a multiple of 16
+// bytes), then h(eta) and sigma_Z(gamma) of the run's Z alone (a batch copies the row again when it comes to another run).
+// Rate tables of 2 / 20 / 36 / 100 KB (n_E = 256 / 2048 / 4000 / 4000 rows of 2 / 2 / 2 / 6 Z), 2e5 electrons x 300 steps:
+// 0.54 / 0.65 / 0.67 / 1.54 ms with every row copied, 0.54 / 0.55 / 0.65 / 0.65 so.
 constexpr int kPairFixedBytes = kSumsThreads * (16 * kEnergySums + 3 * 8) + 8 * PE_TALLY_WORDS + 4 * PE_HIST_WORDS +
                                 4 * PE_T_E_NCS_STORED;
 static_assert(kPairFixedBytes % 16 == 0, "tables after a 16-byte boundary");
@@ -871,9 +873,11 @@ struct PairShared {
         for (int k = threadIdx.x; k < kPairFixedBytes / 16; k += blockDim.x) w[k] = make_uint4(0, 0, 0, 0);
 #pragma unroll 4
         for (int k = threadIdx.x; k < t.n_eta; k += blockDim.x) h[k] = t.h32[k];
+    }
+    __device__ __forceinline__ void load_sigma(const TablesDev& t, int iz) const {
+        const float* row = t.sig32 + (size_t)iz * t.n_E;
 #pragma unroll 4
-        for (int k = threadIdx.x; k < t.n_Z * t.n_E; k += blockDim.x) sig[k] = t.sig32[k];
-        __syncthreads();
+        for (int k = threadIdx.x; k < t.n_E; k += blockDim.x) sig[k] = row[k];
     }
     __device__ __forceinline__ SumsCta acc() const { return SumsCta{hist, cnt, sums + threadIdx.x}; }
     __device__ __forceinline__ Held slots() const {
@@ -964,6 +968,8 @@ __global__ void __launch_bounds__(128, (pair_min_ctas<G, F>())) k_step_pair(Tabl
     __shared__ RunDevT<float> s_run;
     const PairShared S(smem, t.n_eta);
     S.init(t);
+    if (kSingle) S.load_sigma(t, b.runs[0].iz);
+    __syncthreads();
     const SumsCta acc = S.acc();
     const Held held = S.slots();
 
@@ -980,6 +986,7 @@ __global__ void __launch_bounds__(128, (pair_min_ctas<G, F>())) k_step_pair(Tabl
                 constexpr int kWords = sizeof(RunDevT<float>) / 4;
                 for (int w = threadIdx.x; w < kWords; w += blockDim.x)
                     reinterpret_cast<uint32_t*>(&s_run)[w] = reinterpret_cast<const uint32_t*>(&b.runs[run_idx])[w];
+                S.load_sigma(t, b.runs[run_idx].iz);
                 __syncthreads();
                 cur = run_idx;
             }
@@ -989,7 +996,7 @@ __global__ void __launch_bounds__(128, (pair_min_ctas<G, F>())) k_step_pair(Tabl
         since += per_tile;
         const int64_t base = (tile - b.tile_start[run_idx]) * b.tile;
         const int64_t i0 = base + threadIdx.x, i1 = base + threadIdx.x + blockDim.x;
-        tile_steps_pair<G, F, kSingle, kHold>(t, r, S.h, S.sig + (size_t)r.iz * t.n_E, i0, i1, steps, acc, held, S.tally);
+        tile_steps_pair<G, F, kSingle, kHold>(t, r, S.h, S.sig, i0, i1, steps, acc, held, S.tally);
     }
     if (kSingle) {
         if (n_tiles > 0) S.flush(b.runs[0]);
@@ -1154,10 +1161,12 @@ __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pai
     __shared__ StreamQueue s_queue[kOne ? kStreamThreads / 32 : 1];
     const PairShared S(smem, t.n_eta);
     // the stages on a 16-byte boundary after the tables
-    const uint32_t table_bytes = kPairFixedBytes + 4 * (t.n_eta + t.n_Z * t.n_E);
+    const uint32_t table_bytes = kPairFixedBytes + 4 * (t.n_eta + t.n_E);
     unsigned char* stage_buf = smem + ((table_bytes + 15u) & ~15u);
     const RunDevT<float>& r = b.runs[0];
     S.init(t);
+    S.load_sigma(t, r.iz);
+    __syncthreads();
     // what follows reads the state: the launch of this kernel may overlap the end of the one before
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1166,7 +1175,7 @@ __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pai
     const int64_t n_tiles = b.tile_start[1];
     const int64_t n_pairs = r.n >> 1;                   // j < n_pairs: electrons 2j and 2j + 1 both present
     const int64_t stride = (int64_t)gridDim.x * kStreamThreads;
-    const float* sig_z = S.sig + (size_t)r.iz * t.n_E;
+    const float* sig_z = S.sig;
     const uint32_t n0 = (uint32_t)r.step0;
     const int lane = threadIdx.x & 31;
     StreamQueue& W = s_queue[kOne ? threadIdx.x >> 5 : 0];

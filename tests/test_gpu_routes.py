@@ -85,6 +85,29 @@ def test_f64_rate_tables_of_every_size(n_E, n_z):
 
 
 # --------------------------------------------------------------------------- the paired FP32 step ----
+@pytest.mark.parametrize("n_eta,n_E,n_z", [(48, 48, 2), (1024, 2048, 3), (4096, 4096, 7)])
+def test_f32_rate_tables_of_every_size(n_eta, n_E, n_z):
+    """The paired kernels copy h(eta) and the run's own row of sigma_Z: runs of several Z give the same results alone, in
+    launches of one step and in a batch in which a CTA goes from one row to another."""
+    Zs = (13.0, 79.0, 29.0, 47.0, 6.0, 22.0, 73.0)[:n_z]
+    lt = pe.pe_create_tables(dict(W.tables_small(), n_eta=n_eta, n_y=16, n_E=n_E, n_s=16), Zs)
+    kw = dict(a0=400.0, init_dist=1, slab_x0_m=0.1e-6, slab_thick_m=0.7e-6, dt_over_T=0.02, charge_state=6.0, ne_over_nc=4000.0)
+
+    def runs():
+        return [pe.Run(lt, pe.run_params(precision=pe.PE_F32, **W.base_run(**dict(kw, Z=Zs[k % n_z], seed=k, run_id=k))),
+                       3_001, events=True) for k in range(5)]
+    alone, one, batch = runs(), runs(), runs()
+    for r in alone:
+        pe.pe_step([r.handle], 90)
+    for r in one:
+        pe.pe_step_ex([r.handle], 90, steps_per_launch=1)
+    pe.pe_step_ex([r.handle for r in batch], 90, ctas_per_sm=1, block=64)
+    assert sum(int(r.tally_out().tally[pe.T["N_BR_STORED"]]) for r in alone) > 0
+    for a, b, c in zip(alone, one, batch):
+        same(outcome(b), outcome(a))
+        same(outcome(c), outcome(a))
+
+
 @pytest.mark.parametrize("n", [1, 2, 63, 257, 5_000, 200_003])
 @pytest.mark.parametrize("kind", ["plane", "plane-null-box"])
 def test_one_step_launches_queue_their_emissions(n, kind):
