@@ -657,17 +657,13 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
         for (int k = 0; k < m; ++k) tile_start[k + 1] = tile_start[k] + (runs[idx[k]]->dev.n + block - 1) / block;
         int64_t n_tiles = tile_start[m];
         if (n_tiles == 0) continue;
-        // default grid: three resident waves of the paired kernel (plane wave, 2D focus), twice the
-        // resident CTAs of the one-electron kernel, so the block scheduler evens out tiles of unequal cost
-        int per_sm = (cfg && cfg->ctas_per_sm > 0) ? cfg->ctas_per_sm
-                                                  : (prec == PE_F32 ? default_ctas_per_sm_f32(fk, block, smem, K)
-                                                                    : 2 * persistent_occupancy_f64(block));
-        if (per_sm < 1) per_sm = 1;
-        int grid = (int)std::min<int64_t>(n_tiles, (int64_t)sms * per_sm);
+        // default grid: resident waves of the kernel launched (default_ctas_per_sm_f32), twice the resident CTAs of
+        // the one-electron kernel, so the block scheduler evens out tiles of unequal cost
+        const int per_sm_set = cfg && cfg->ctas_per_sm > 0 ? cfg->ctas_per_sm : 0;
+        int grid = 0;
         for (int64_t done = 0; done < n_steps; done += K) {
             PlanLaunch L;
             L.prec = prec;
-            L.grid = grid;
             L.block = block;
             L.smem = smem;
             L.steps = (int)std::min<int64_t>(K, n_steps - done);
@@ -689,6 +685,13 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
                 for (int k = 0; k <= m; ++k) L.bd->tile_start[k] = tile_start[k];
                 for (int k = 0; k < m; ++k) L.bd->runs[k] = runs[idx[k]]->dev;
             }
+            if (done == 0 || L.steps != K) {             // the launches of one length have one kernel
+                const int per_sm = per_sm_set ? per_sm_set
+                                   : prec == PE_F32 ? default_ctas_per_sm_f32(*L.bf, L.steps, block, smem)
+                                                    : 2 * persistent_occupancy_f64(block);
+                grid = (int)std::min<int64_t>(n_tiles, (int64_t)sms * std::max(per_sm, 1));
+            }
+            L.grid = grid;
             plan.launches.push_back(std::move(L));
         }
     }

@@ -209,7 +209,7 @@ void launch_step_persistent_f64(const TablesDev& t, const BatchDevT<double>& b, 
                                 cudaStream_t s);
 size_t rate_table_bytes(const TablesDev& t, int precision);       // h(eta) and sigma_Z(gamma)
 int pair_smem_bytes(const TablesDev& t);                          // the paired FP32 kernels
-int default_ctas_per_sm_f32(int fk, int block, int smem, int steps_per_launch);
+int default_ctas_per_sm_f32(const BatchDevT<float>& b, int steps, int block, int base_smem);
 const void* persistent_kernel_f32(const BatchDevT<float>& b, int steps, int smem, int block, int* threads,
                                   int* smem_out);
 const void* persistent_kernel_f64(const BatchDevT<double>& b);

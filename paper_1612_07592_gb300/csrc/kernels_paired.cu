@@ -18,7 +18,8 @@ int pair_smem_bytes(const TablesDev& t) { return kPairFixedBytes + 4 * (t.n_eta 
 
 static bool plane_kind(int fk) { return fk == FK_PLANE_LP || fk == FK_PLANE_CP; }
 // tables, then 16-byte alignment slack and the stage buffers
-static int stream_smem_bytes(int base) { return base + 16 + kStreamStages * kStageBytes; }
+template <int F>
+static int stream_smem_bytes(int base) { return base + 16 + kStreamStages * kStageBytes<F>; }
 static bool stream_shape(int fk, int steps, int block) {
     return plane_kind(fk) && steps <= kStreamMaxSteps && block == kStreamTile;
 }
@@ -67,10 +68,9 @@ static StepKernel kernel_of(const BatchDevT<float>& b, int steps, int block, int
     const int flags = flags_of(b);
     if constexpr (G == FK_PLANE_LP || G == FK_PLANE_CP) {
         if (kSingle && use_stream(b, steps, block)) {
-            smem = stream_smem_bytes(base_smem);
-            if (steps == 1)
-                return flags == kFlagsPaper ? k_step_pair_stream<G, kFlagsPaper, true> : k_step_pair_stream<G, kFlagsRun, true>;
-            return flags == kFlagsPaper ? k_step_pair_stream<G, kFlagsPaper, false> : k_step_pair_stream<G, kFlagsRun, false>;
+            smem = flags == kFlagsPaper ? stream_smem_bytes<kFlagsPaper>(base_smem) : stream_smem_bytes<kFlagsRun>(base_smem);
+            if (flags != kFlagsPaper) return k_step_pair_stream<G, kFlagsRun, false>;
+            return steps == 1 ? k_step_pair_stream<G, kFlagsPaper, true> : k_step_pair_stream<G, kFlagsPaper, false>;
         }
     }
     constexpr bool kMayHold = G == FK_REFL_LP || G == FK_REFL_CP || G == FK_CONST;
@@ -147,22 +147,11 @@ const void* persistent_kernel_f32(const BatchDevT<float>& b, int steps, int base
 // cost with their emission histories, and a CTA per one or two tiles lets the block scheduler balance
 // them: measured +6 % over one wave, +2.5 % over two, on 1e6 electrons); one wave for the streaming
 // form (each CTA streams many tiles of equal cost).
-int default_ctas_per_sm_f32(int fk, int block, int smem, int steps_per_launch) {
-    int occ = 0;
-    cudaError_t e;
-    if (stream_shape(fk, steps_per_launch, block)) {
-        const auto f = k_step_pair_stream<FK_PLANE_LP, kFlagsPaper, true>;
-        allow_smem((const void*)f, stream_smem_bytes(smem));
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, block / 2, stream_smem_bytes(smem));
-        return e == cudaSuccess && occ > 0 ? occ : 1;
-    }
-    with_paired_kind(fk, [&](auto g) {
-        constexpr int G = decltype(g)::value;
-        const auto f = k_step_pair<true, G, kFlagsPaper, G == FK_REFL_LP || G == FK_REFL_CP>;
-        allow_smem((const void*)f, smem);
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, block / 2, smem);
-    });
-    return 3 * (e == cudaSuccess && occ > 0 ? occ : 1);
+int default_ctas_per_sm_f32(const BatchDevT<float>& b, int steps, int block, int base_smem) {
+    int threads, smem, occ = 0;
+    const void* f = persistent_kernel_f32(b, steps, base_smem, block, &threads, &smem);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, threads, smem);
+    return (use_stream(b, steps, block) ? 1 : 3) * (e == cudaSuccess && occ > 0 ? occ : 1);
 }
 
 }  // namespace pe

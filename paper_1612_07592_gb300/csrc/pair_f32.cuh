@@ -1016,8 +1016,8 @@ __global__ void __launch_bounds__(128, (pair_min_ctas<G, F>())) k_step_pair(Tabl
 // tile, and waits only for its own copies (cp.async.wait_group): no barrier, no spin-wait.
 // Results go back with streaming vector stores.  The arithmetic is that of the resident
 // kernel (the paired step is elementwise in its two electrons), so the results are the
-// same bit for bit.  Single run; the ragged end (an odd last electron) and the optional
-// event / wait words use plain loads.
+// same bit for bit.  Single run; the ragged end (an odd last electron) and the event words
+// use plain loads.
 // ---------------------------------------------------------------------------
 constexpr int kStreamTile = 256;                       // electrons per tile (128 threads x 2)
 constexpr int kStreamThreads = kStreamTile / 2;
@@ -1031,8 +1031,10 @@ constexpr int kStreamThreads = kStreamTile / 2;
 #define PE_STREAM_MIN_CTAS 4  // resident CTAs of 128 threads per SM the registers are sized for
 #endif
 constexpr int kStreamStages = PE_STREAM_STAGES;
-// one stage: x pairs (float4 per thread), tau pairs (float4), ux, uy, uz (float2 each)
-constexpr int kStageBytes = kStreamThreads * (16 + 16 + 8 + 8 + 8);
+// one stage: x pairs (float4 per thread), tau pairs (float4), ux, uy, uz (float2 each), and in the instances that may have
+// null collisions the waits (uint2)
+template <int F>
+constexpr int kStageBytes = kStreamThreads * (16 + 16 + 8 + 8 + 8 + (F == kFlagsRun ? 8 : 0));
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -1050,10 +1052,11 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 
 // this thread's slots of a stage
 struct StageSlots {
-    uint32_t x, tau, ux, uy, uz;       // shared addresses (for the copies)
+    uint32_t x, tau, ux, uy, uz, wait; // shared addresses (for the copies)
     const float4* px;                  // generic pointers (for the reads)
     const float4* ptau;
     const float2 *pux, *puy, *puz;
+    const uint2* pwait;
 };
 __device__ __forceinline__ StageSlots stage_slots(unsigned char* stage, int t) {
     StageSlots q;
@@ -1063,22 +1066,27 @@ __device__ __forceinline__ StageSlots stage_slots(unsigned char* stage, int t) {
     q.pux = reinterpret_cast<const float2*>(b + kStreamThreads * 32) + t;
     q.puy = reinterpret_cast<const float2*>(b + kStreamThreads * 40) + t;
     q.puz = reinterpret_cast<const float2*>(b + kStreamThreads * 48) + t;
+    q.pwait = reinterpret_cast<const uint2*>(b + kStreamThreads * 56) + t;
+    q.wait = smem_addr(q.pwait);
     q.x = smem_addr(q.px); q.tau = smem_addr(q.ptau);
     q.ux = smem_addr(q.pux); q.uy = smem_addr(q.puy); q.uz = smem_addr(q.puz);
     return q;
 }
 // copies of electrons 2j, 2j + 1 (both present) into the slots
+template <int F>
 __device__ __forceinline__ void stage_issue(const RunDevT<float>& r, int64_t j, const StageSlots& q) {
     cp_async16(q.x, reinterpret_cast<const float4*>(r.x) + j);
     cp_async16(q.tau, reinterpret_cast<const float4*>(r.tau) + j);
     cp_async8(q.ux, reinterpret_cast<const float2*>(r.ux) + j);
     cp_async8(q.uy, reinterpret_cast<const float2*>(r.uy) + j);
     cp_async8(q.uz, reinterpret_cast<const float2*>(r.uz) + j);
+    if (F == kFlagsRun && r.wait) cp_async8(q.wait, reinterpret_cast<const uint2*>(r.wait) + j);
 }
 // a particle is removed (x NaN, finite momenta), live, or has a non-finite momentum
 __device__ __forceinline__ bool finite3(float a, float b, float c) { return isfinite(a) && isfinite(b) && isfinite(c); }
 
-// electrons 2j, 2j + 1 from the slots (the optional words from global memory)
+// electrons 2j, 2j + 1 from the slots
+template <int F>
 __device__ __forceinline__ void stage_take(const RunDevT<float>& r, int64_t j, const StageSlots& q, Pair& Q,
                                            unsigned long long* tally) {
     const float4 x = *q.px, tau = *q.ptau;
@@ -1090,8 +1098,8 @@ __device__ __forceinline__ void stage_take(const RunDevT<float>& r, int64_t j, c
     Q.u1 = *q.puy;
     Q.u2 = *q.puz;
     Q.y = Q.y_lo = P2(0.0f);
-    if (r.wait) {
-        const uint2 w = reinterpret_cast<const uint2*>(r.wait)[j];
+    if (F == kFlagsRun && r.wait) {
+        const uint2 w = *q.pwait;
         Q.wait[0] = w.x;
         Q.wait[1] = w.y;
     } else {
@@ -1214,20 +1222,20 @@ __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pai
 #pragma unroll
     for (int k = 0; k < kStreamStages - 1; ++k) {
         const int64_t jk = j0 + k * stride;
-        if (jk < n_pairs) stage_issue(r, jk, stage_slots(stage_buf + k * kStageBytes, threadIdx.x));
+        if (jk < n_pairs) stage_issue<F>(r, jk, stage_slots(stage_buf + k * kStageBytes<F>, threadIdx.x));
         cp_async_commit();
     }
     int stage = 0;
     for (int64_t j = j0; j - threadIdx.x < n_tiles * kStreamThreads; j += stride) {
         const int64_t jn = j + (kStreamStages - 1) * stride;
         const int sn = stage == 0 ? kStreamStages - 1 : stage - 1;       // (stage + S - 1) mod S
-        if (jn < n_pairs) stage_issue(r, jn, stage_slots(stage_buf + sn * kStageBytes, threadIdx.x));
+        if (jn < n_pairs) stage_issue<F>(r, jn, stage_slots(stage_buf + sn * kStageBytes<F>, threadIdx.x));
         cp_async_commit();
         cp_async_wait<kStreamStages - 1>();             // this thread's copies of the current tile
         Pair Q;
         const bool full = j < n_pairs;
         if (full) {
-            stage_take(r, j, stage_slots(stage_buf + stage * kStageBytes, threadIdx.x), Q, S.tally);
+            stage_take<F>(r, j, stage_slots(stage_buf + stage * kStageBytes<F>, threadIdx.x), Q, S.tally);
         } else {
             pair_clear(Q);
             if (2 * j < r.n) load_one(r, 2 * j, Q, 0, S.tally);   // the odd last electron
