@@ -944,10 +944,11 @@ __device__ __forceinline__ void tile_steps_pair(const TablesDev& t, const RunDev
 #define PE_PAIR_MIN_CTAS_REFL 7
 #endif
 // The general instances (flags read at run time: the null-collision method, a process switched off, the box boundary)
-// carry more live state than the others, but more registers for them measured slower (the 1 GeV Au bunch by null
-// collisions, 1e6 electrons: 7 CTAs 7.09e10 particle-steps/s, 6 6.70e10, 5 7.01e10).
+// carry more live state than the others.  2e5 electrons x 400 steps, plane wave without brems / by null collisions /
+// reflected wave by null collisions, and the 1 GeV Au bunch by null collisions (1500 steps at dt = T): 5 CTAs 652 / 785 /
+// 2360 us, 6 587 / 677 / 1844 / 2008, 7 616 / 702 / 1901 / 2240, 8 632 / 742 / 1894 / 2554.
 #ifndef PE_PAIR_MIN_CTAS_GENERAL
-#define PE_PAIR_MIN_CTAS_GENERAL 7
+#define PE_PAIR_MIN_CTAS_GENERAL 6
 #endif
 // Brems alone (the bunch by the direct method, 5e5 electrons x 2000 steps): 7 to 9 CTAs 5.73 to 5.78 ms, 10 5.84.
 #ifndef PE_PAIR_MIN_CTAS_BREMS
