@@ -160,9 +160,16 @@ __device__ void pic_fields_block(const RunDevT<R>& r) {
     }
 }
 
+// Resident CTAs of 256 threads per SM the registers are sized for.  FP32, 1e6 electrons, 500 steps: 4 24.6 ms, 2 26.8, 3
+// 26.3, 5 27.6 (each CTA adds one flush of its current sums).  FP64 (us a step, 1000 cells): 4 (64 registers, spilled) 451
+// at 5e5 electrons and 760 at 1e6, 3 434 / 794, 2 409 / 755.  FP64 with at most a tile a warp takes the emissions in
+// place (a queue would send the few electrons of a warp through the rest of the step a second time, at the FP64 price of
+// a full warp) and fits 3 CTAs: 1e5 electrons 117, with the queue 173 at 4 CTAs and 147 at 2; 1e3 electrons 44 and 51.
 #ifndef PE_PIC_MIN_CTAS
 #define PE_PIC_MIN_CTAS 4
 #endif
+template <typename R, bool kInPlace>
+constexpr int pic_ctas() { return sizeof(R) == 4 ? PE_PIC_MIN_CTAS : kInPlace ? 3 : 2; }
 constexpr int kPicThreads = 256;
 // emissions of a warp that wait (fewer than 32 left by the last round and at most 32 more): electron, eta, gamma
 template <typename R>
@@ -176,15 +183,16 @@ struct PicQueue {
 //
 // An emission is several times as long as the rest of the step and falls to a few per cent of the electrons, so more
 // than half of the warps would issue all of it for one or two lanes.  An electron whose optical depth crosses is
-// stored as it is after the push and queued by its warp; the warp takes the queue 32 emissions at a time, or what there
-// is when its electrons of the round are done, and goes through the rest of the step with them.  1e6 electrons, 1000
-// cells, steps 0 to 500 (us per step): 59 with the emissions where they fell, 64-bit shared sums and a kernel that waits
+// (unless kInPlace) stored as it is after the push and queued by its warp; the warp takes the queue 32 emissions at a
+// time, or what there is when its electrons of the round are done, and goes through the rest of the step with them.  1e6
+// electrons, 1000 cells, steps 0 to 500 (us per step): 59 with the emissions where they fell, 64-bit shared sums and a kernel that waits
 // for the one before; 58.6 with the currents' 64-bit conversions off the FP64 pipe; 49 with the queue, native sums and
 // overlapped launches; 48 with the test of Eq. 4 from the draw's high word; 45 with the field update below.  5000
 // electrons: 19, now 14, the length of the chain from one step's loads to the next's.  What is left is issue (0.6 a
 // cycle, some 900 instructions for 32 electrons, a quarter of them the deposit).
-template <typename R, bool kCommon>
-__global__ void __launch_bounds__(kPicThreads, PE_PIC_MIN_CTAS) k_pic_particles(TablesDev t, RunDevT<R> r, int staged) {
+template <typename R, bool kCommon, bool kInPlace>
+__global__ void __launch_bounds__(kPicThreads, (pic_ctas<R, kInPlace>()))
+    k_pic_particles(TablesDev t, RunDevT<R> r, int staged) {
     extern __shared__ __align__(16) unsigned char smem[];
     PicQueue<R>* s_queue = reinterpret_cast<PicQueue<R>*>(smem);
     int* s_j = reinterpret_cast<int*>(s_queue + kPicThreads / 32);              // 3 n_cells current sums (split)
@@ -250,16 +258,22 @@ __global__ void __launch_bounds__(kPicThreads, PE_PIC_MIN_CTAS) k_pic_particles(
                 if (active) {
                     x_old = P.x + P.x_lo;
                     crossed = push_one<R, FK_PIC, kCommon>(t, r, h_tab, nf, P, gamma, inv_g, eta, acc);
+                    if (kInPlace && crossed) {
+                        emit_one<R>(t, r, r.id0 + (uint32_t)i, step, P, gamma, inv_g, eta, acc);
+                        crossed = false;
+                    }
                 }
-                const unsigned mask = __ballot_sync(0xffffffffu, crossed);
-                if (crossed) {
-                    const int at = queued + __popc(mask & ((1u << lane) - 1u));
-                    Q.i[at] = (uint32_t)i;
-                    Q.eta[at] = eta;
-                    Q.gamma[at] = gamma;
-                    store_particle<R>(r, i, P);
+                if constexpr (!kInPlace) {
+                    const unsigned mask = __ballot_sync(0xffffffffu, crossed);
+                    if (crossed) {
+                        const int at = queued + __popc(mask & ((1u << lane) - 1u));
+                        Q.i[at] = (uint32_t)i;
+                        Q.eta[at] = eta;
+                        Q.gamma[at] = gamma;
+                        store_particle<R>(r, i, P);
+                    }
+                    queued += __popc(mask);
                 }
-                queued += __popc(mask);
                 on = active && !crossed;
                 base += stride;
                 ++tiles;
@@ -349,12 +363,14 @@ static void pic_step(const TablesDev& t, const RunDevT<R>& r, int sms, cudaStrea
     int staged = 1;
     const size_t smem = pic_smem_bytes(t, r.n_cells, sizeof(R) == 4 ? PE_F32 : PE_F64, staged);
     const bool common = r.enable_ncs && r.enable_brems && r.brems_method == PE_BREMS_DIRECT;
-    auto* f = common ? k_pic_particles<R, true> : k_pic_particles<R, false>;
-    cudaFuncSetAttribute((const void*)f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    // four resident CTAs of 256 threads per SM (64 registers): on 1e6 electrons, 500 steps, 24.6 ms against 26.8 at
-    // two, 26.3 at three and 27.6 at five (each CTA adds one flush of its current sums)
     const int64_t blocks = (r.n + kPicThreads - 1) / kPicThreads;
-    const int grid = (int)(blocks < PE_PIC_MIN_CTAS * (int64_t)sms ? (blocks > 0 ? blocks : 1) : PE_PIC_MIN_CTAS * (int64_t)sms);
+    const bool in_place = sizeof(R) == 8 && blocks <= (int64_t)pic_ctas<R, true>() * sms;
+    auto* f = common ? k_pic_particles<R, true, false> : k_pic_particles<R, false, false>;
+    if constexpr (sizeof(R) == 8)
+        if (in_place) f = common ? k_pic_particles<R, true, true> : k_pic_particles<R, false, true>;
+    cudaFuncSetAttribute((const void*)f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int64_t most = (int64_t)(in_place ? pic_ctas<R, true>() : pic_ctas<R, false>()) * sms;
+    const int grid = (int)(blocks < most ? (blocks > 0 ? blocks : 1) : most);
     // the next step's CTAs start as this step's leave, clear their sums and wait there for its last (griddepcontrol)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);

@@ -262,6 +262,28 @@ def test_pic_queue_splits(precision, n, n_cells):
     assert outs[0][2:] == outs[1][2:]
 
 
+@pytest.mark.parametrize("precision,n_eta,n_z,n_E", [(pe.PE_F64, 1200, 7, 3550), (pe.PE_F32, 2800, 13, 3846)])
+def test_pic_rate_tables_read_in_place(precision, n_eta, n_z, n_E):
+    """Rate tables that leave no room for the warps' queues beside a grid of 400 cells are read in global memory: the same
+    steps as on a grid of 300 cells, where they fit (nothing reaches the 300th), for a few electrons and for many tiles
+    a warp."""
+    lt = pe.pe_create_tables(dict(W.tables_small(), n_eta=n_eta, n_y=16, n_E=n_E, n_s=16), (79.0,) + tuple(range(60, 59 + n_z)))
+    for n in (500, 130_001):
+        outs = []
+        for n_cells in (400, 300):
+            run = W.base_run(a0=600.0, init_dist=1, seed=n, geometry=pe.PE_PIC_1D, n_cells=n_cells, slab_x0_m=0.3e-6, **W.AU)
+            r = pe.Run(lt, pe.run_params(precision=precision, **run), n, events=True)
+            pe.pe_step([r.handle], 120)
+            outs.append(outcome(r))
+        assert outs[0][1].any()
+        same(outs[0], outs[1])
+        t, ph, w = r.tally_out(), r.photon_records(), outs[0][1]
+        stored, below = (t.tally[pe.T["N_NCS_" + k]] + t.tally[pe.T["N_BR_" + k]] for k in ("STORED", "BELOW"))
+        assert len(ph) == stored == sum(t.hist[:2 * pe.HIST_E_BINS])
+        assert int((w & np.uint64(0xFFFF)).sum() + ((w >> np.uint64(16)) & np.uint64(0xFFFF)).sum()) == stored + below
+        np.testing.assert_allclose(ph["energy"].astype(np.float64).sum(), t.e_ncs_stored + t.e_br_stored, rtol=1e-6)
+
+
 # ------------------------------------------------------------------------- pair production queues ----
 @pytest.mark.parametrize("n", [1, 33, 3_000, 40_001])
 @pytest.mark.parametrize("process", ["bh-direct", "bh-free", "bw-f32", "bw-f64"])
