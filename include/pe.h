@@ -208,7 +208,7 @@ typedef struct {
  * tile with block/2 threads, two electrons each, the FP64 kernel with block
  * threads; ctas_per_sm: CTAs per SM in the grid; steps_per_launch: steps done
  * per launch with the state held in registers (1 = state round-trips memory
- * every step; at most 2^20).  Zeros pick defaults: 256 electrons per tile (32 for FP64
+ * every step; at most 2^20, longer calls take several launches).  Zeros pick defaults: 256 electrons per tile (32 for FP64
  * runs of up to 512 electrons per SM); three times the
  * CTAs that fit on an SM for the FP32 kernel (once for the one-step form of a
  * single plane-wave run, launches of at most 4 steps), twice for the FP64
@@ -274,9 +274,15 @@ pe_status pe_resume_particles(const pe_tables* tables, const pe_run_params* para
                               const pe_buffers* buffers, int64_t step0, void* cuda_stream, pe_run** out);
 
 /* Advance runs by n_steps in launches of at most steps_per_launch steps.  n_runs > 1
- * (<= PE_MAX_BATCH): all runs must be PE_F32 and share the first run's
+ * (<= PE_MAX_BATCH): all runs must share precision, tables and the first run's
  * stream; they advance together, one persistent launch per field kind present
  * per steps_per_launch steps.  Asynchronous.  cfg may be NULL.
+ * One PE_F64 run with steps_per_launch 0 takes the default shape (block and
+ * ctas_per_sm of cfg are not read), rate tables of any size, and looks for
+ * non-finite momenta before every step; other calls look at the start of each
+ * launch (a PE_PIC_1D run takes a launch per step) and refuse (PE_ERR_ARG; for
+ * PE_PIC_1D the launch fails, with the grid counted in) rate tables n_eta +
+ * n_Z * n_E of more than 193472 bytes in the run's precision.
  * Precision: the FP32 kernels form the laser phase t^n - x with t^n = n dt_hi +
  * n dt_lo, dt_hi holding 11 significant bits, so n dt_hi is exact up to step
  * 8192 (the paper's runs take 4000); later steps add one rounding of about

@@ -168,7 +168,7 @@ __device__ __forceinline__ void hist_bins(float e, float kx, float ky, float inv
 }
 
 // Where an emission's counts, energies and histogram bins go.
-// Sums64: 64-bit words in global or shared memory, every add an atomic (the FP64 kernels and the PIC).
+// Sums64: 64-bit words in global or shared memory, every add an atomic (the FP64 kernels).
 struct Sums64 {
     unsigned long long* hist;
     unsigned long long* tally;
@@ -536,15 +536,16 @@ __device__ __forceinline__ void rest_one(const TablesDev& t, const RunDevT<R>& r
     advance(P.x, P.x_lo, over_gamma(c.dt * P.u[0], gamma, inv_g));
     if (G == FK_GAUSS_LP || G == FK_GAUSS_CP) advance(P.y, P.y_lo, over_gamma(c.dt * P.u[1], gamma, inv_g));
 }
-template <typename R, int G, bool kCommon = false>
+// both halves and the absorbing boundary; returns the particle's Lorentz factor
+template <typename R, int G>
 __device__ __forceinline__ R step_one(const TablesDev& t, const RunDevT<R>& r, const R* h_tab, const R* sig_tab,
                                       uint32_t id, uint32_t n, R nf, Particle<R>& P,
                                       unsigned long long* hist, unsigned long long* tally) {
     const Sums64 acc{hist, tally};
     R gamma, inv_g, eta;
-    if (push_one<R, G, kCommon>(t, r, h_tab, nf, P, gamma, inv_g, eta, acc)) emit_one<R>(t, r, id, n, P, gamma, inv_g, eta, acc);
-    rest_one<R, G, kCommon>(t, r, sig_tab, id, n, P, gamma, inv_g, acc);
-    if (!kCommon) box_check<R>(r, P, n, tally);
+    if (push_one<R, G, false>(t, r, h_tab, nf, P, gamma, inv_g, eta, acc)) emit_one<R>(t, r, id, n, P, gamma, inv_g, eta, acc);
+    rest_one<R, G, false>(t, r, sig_tab, id, n, P, gamma, inv_g, acc);
+    box_check<R>(r, P, n, tally);
     return gamma;
 }
 
@@ -673,7 +674,7 @@ __device__ void flush_shared(unsigned long long* s_hist, unsigned long long* s_t
 // looked at before every step (live_or_kill), not only at the start of the launch.  Momenta that are not finite show
 // in gamma, so the loop of the steps only tests its exponent, and leaves for the look (the 1e4-electron job 12.8 ms;
 // 13.1 with the look in that loop, 12.9 with no test, and with a particle that is not active kept in the loop).
-template <typename R, int G, bool kCommon>
+template <typename R, int G>
 __device__ __forceinline__ void tile_steps(const TablesDev& t, const RunDevT<R>& r, const R* s_h, const R* sig_z,
                                            int64_t i, Particle<R>& P, int steps, bool each_step,
                                            unsigned long long* s_hist, unsigned long long* s_tally) {
@@ -683,8 +684,8 @@ __device__ __forceinline__ void tile_steps(const TablesDev& t, const RunDevT<R>&
     while (true) {
         bool look = false;
         while (n != end && !look) {
-            const R gamma = step_one<R, G, kCommon>(t, r, s_h, sig_z, r.id0 + (uint32_t)i, n, nf, P, s_hist, s_tally);
-            if (!kCommon && r.box_enable && isnan(P.x)) { store_particle<R>(r, i, P); return; }
+            const R gamma = step_one<R, G>(t, r, s_h, sig_z, r.id0 + (uint32_t)i, n, nf, P, s_hist, s_tally);
+            if (r.box_enable && isnan(P.x)) { store_particle<R>(r, i, P); return; }
             look = (__double2hiint(gamma) & 0x7FF00000) == 0x7FF00000;
             ++n;
             nf += (R)1;
@@ -703,7 +704,7 @@ __device__ __forceinline__ void tile_steps(const TablesDev& t, const RunDevT<R>&
 #ifndef PE_MIN_CTAS
 #define PE_MIN_CTAS 2
 #endif
-template <typename R, bool kSingle, int G, bool kCommon = false>
+template <typename R, bool kSingle, int G>
 __global__ void __launch_bounds__(256, PE_MIN_CTAS) k_step_persistent(TablesDev t, BatchDevT<R> b, int steps) {
     __shared__ unsigned long long s_hist[PE_HIST_WORDS];
     __shared__ unsigned long long s_tally[PE_TALLY_WORDS];
@@ -741,7 +742,7 @@ __global__ void __launch_bounds__(256, PE_MIN_CTAS) k_step_persistent(TablesDev 
             active = live_or_kill<R>(r, i, P, (uint32_t)r.step0, s_tally);
         }
         const R* sig_z = sig_tab + (size_t)r.iz * t.n_E;
-        if (active) tile_steps<R, G, kCommon>(t, r, h_tab, sig_z, i, P, steps, b.each_step, s_hist, s_tally);
+        if (active) tile_steps<R, G>(t, r, h_tab, sig_z, i, P, steps, b.each_step, s_hist, s_tally);
         cur = kSingle ? 0 : cur;
     }
     if (kSingle) {

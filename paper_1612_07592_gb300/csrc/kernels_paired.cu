@@ -20,11 +20,8 @@ static bool plane_kind(int fk) { return fk == FK_PLANE_LP || fk == FK_PLANE_CP; 
 // tables, then 16-byte alignment slack and the stage buffers
 template <int F>
 static int stream_smem_bytes(int base) { return base + 16 + kStreamStages * kStageBytes<F>; }
-static bool stream_shape(int fk, int steps, int block) {
-    return plane_kind(fk) && steps <= kStreamMaxSteps && block == kStreamTile;
-}
 static bool use_stream(const BatchDevT<float>& b, int steps, int block) {
-    return b.n_runs == 1 && stream_shape(b.runs[0].fk, steps, block);
+    return b.n_runs == 1 && plane_kind(b.runs[0].fk) && steps <= kStreamMaxSteps && block == kStreamTile;
 }
 // beside the static shared memory of a kernel (below 6 KB) a launch may use 48 KB without being told so
 static void allow_smem(const void* f, int smem) {
@@ -32,9 +29,12 @@ static void allow_smem(const void* f, int smem) {
 }
 
 // Whether the lanes of a warp wait for one another's emissions: where these are frequent, in the reflected wave (5 %
-// of the particle-steps) and in constant fields when a run's largest bremsstrahlung probability per step
-// reaches 1e-3 (the bunch in Au at dt = T 2.6e-3: 8.2 against 8.7 ms; in Al at dt = T / 10, 1e-5: 0.96 against
-// 0.84 ms); not in the plane wave and the 2D focus (below 1e-3).
+// of the particle-steps) and in constant fields when a run's largest bremsstrahlung probability per step P reaches 1e-3;
+// not in the plane wave and the 2D focus (below 1e-3).  1 GeV bunch, 2e5 electrons x 1500 steps, us waiting / not: in Au
+// at P = 5e-4 1558 / 1395, 1.1e-3 1679 / 1528, 1.6e-3 1765 / 1659, 2.7e-3 1889 / 1876, 5.4e-3 2166 / 2390; by null
+// collisions (one candidate in P of the steps) 5e-4 1156 / 1024, 1.1e-3 1284 / 1483, 5.4e-3 2001 / 4424; in Al at 2e-4 1469 /
+// 1312 and 1016 / 798.  The direct method alone breaks even at 3e-3 and loses a tenth at most below that; null collisions
+// gain from 1e-3 on, and so do runs that emit by NCS as well (a field of 10, P = 1.1e-3: 2075 / 4443 for 1e5 electrons x 800).
 template <int G>
 static bool hold_of(const BatchDevT<float>& b) {
     if constexpr (G == FK_CONST) {

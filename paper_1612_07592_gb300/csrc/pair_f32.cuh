@@ -1,5 +1,5 @@
-// pair_f32.cuh -- the FP32 step for the 1D plane-wave field kinds with two
-// electrons per thread.  Blackwell issues paired single-precision arithmetic
+// pair_f32.cuh -- the FP32 step of every prescribed-field kind (the 1D plane wave, its
+// reflection, the 2D focus, constant fields) with two electrons per thread.  Blackwell issues paired single-precision arithmetic
 // (FFMA2/FADD2/FMUL2: two FP32 results per instruction), so the common path of
 // the step -- fields, Boris push, eta, rate lookup, optical depth, the
 // bremsstrahlung probability of Eq. 4, position -- runs on float2 values holding
