@@ -18,8 +18,8 @@ int pair_smem_bytes(const TablesDev& t) { return kPairFixedBytes + 4 * (t.n_eta 
 
 static bool plane_kind(int fk) { return fk == FK_PLANE_LP || fk == FK_PLANE_CP; }
 // tables, then 16-byte alignment slack and the stage buffers
-template <int F>
-static int stream_smem_bytes(int base) { return base + 16 + kStreamStages * kStageBytes<F>; }
+template <int F, bool kOne>
+static int stream_smem_bytes(int base) { return base + 16 + StreamShape<F, kOne>::kStages * kStageBytes<F>; }
 static bool use_stream(const BatchDevT<float>& b, int steps, int block) {
     return b.n_runs == 1 && plane_kind(b.runs[0].fk) && steps <= kStreamMaxSteps && block == kStreamTile;
 }
@@ -68,9 +68,14 @@ static StepKernel kernel_of(const BatchDevT<float>& b, int steps, int block, int
     const int flags = flags_of(b);
     if constexpr (G == FK_PLANE_LP || G == FK_PLANE_CP) {
         if (kSingle && use_stream(b, steps, block)) {
-            smem = flags == kFlagsPaper ? stream_smem_bytes<kFlagsPaper>(base_smem) : stream_smem_bytes<kFlagsRun>(base_smem);
-            if (flags != kFlagsPaper) return k_step_pair_stream<G, kFlagsRun, false>;
-            return steps == 1 ? k_step_pair_stream<G, kFlagsPaper, true> : k_step_pair_stream<G, kFlagsPaper, false>;
+            auto shape = [&](auto f, auto one) -> StepKernel {
+                smem = stream_smem_bytes<decltype(f)::value, decltype(one)::value>(base_smem);
+                return k_step_pair_stream<G, decltype(f)::value, decltype(one)::value>;
+            };
+            using Paper = std::integral_constant<int, kFlagsPaper>;
+            using Run = std::integral_constant<int, kFlagsRun>;
+            if (flags == kFlagsPaper) return steps == 1 ? shape(Paper{}, std::true_type{}) : shape(Paper{}, std::false_type{});
+            return steps == 1 ? shape(Run{}, std::true_type{}) : shape(Run{}, std::false_type{});
         }
     }
     constexpr bool kMayHold = G == FK_REFL_LP || G == FK_REFL_CP || G == FK_CONST;

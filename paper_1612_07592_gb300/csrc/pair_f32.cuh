@@ -1031,7 +1031,18 @@ constexpr int kStreamThreads = kStreamTile / 2;
 #ifndef PE_STREAM_MIN_CTAS
 #define PE_STREAM_MIN_CTAS 4  // resident CTAs of 128 threads per SM the registers are sized for
 #endif
-constexpr int kStreamStages = PE_STREAM_STAGES;
+// What a launch of one step does and an instance's stages and resident CTAs.  The instances that read the flags at run time
+// need more registers than 4 CTAs leave them: 6e6 electrons, us a step, with a box / by null collisions / without brems /
+// neither process: 4 CTAs x 2 stages 83.8 / 86.2 / 79.1 / 68.3, 3 x 3 83.8 / 82.8 / 75.4 / 56.0, 4 x 3 88 / 90 / 82 / 73, 5 x 2
+// 91 / 92 / 82 / 71, and with the queue below (spilled) 104 / 105 / 92 / 74; on 1e6 electrons 21.0 / 21.1 / 19.4 / 12.3 and
+// 21.9 / 21.5 / 20.1 / 10.9.  In launches of 2 to 4 steps they keep 4 x 2 (1e6 electrons 11.3 / 10.7 / 9.5 / 5.1, 3 x 3 12.7 /
+// 12.0 / 10.7 / 5.2).
+template <int F, bool kOne>
+struct StreamShape {
+    static constexpr bool kQueue = kOne && F == kFlagsPaper;
+    static constexpr int kStages = kOne && F != kFlagsPaper ? 3 : PE_STREAM_STAGES;
+    static constexpr int kCtas = kOne && F != kFlagsPaper ? 3 : PE_STREAM_MIN_CTAS;
+};
 // one stage: x pairs (float4 per thread), tau pairs (float4), ux, uy, uz (float2 each), and in the instances that may have
 // null collisions the waits (uint2)
 template <int F>
@@ -1160,14 +1171,16 @@ struct StreamQueue {
     uint32_t crossed[64];
 };
 
-// kOne: launches of one step.  A pair with an emission is then stored as it is after the push and queued by its warp,
+// kOne: launches of one step.  With kQueue a pair with an emission is then stored as it is after the push and queued by its warp,
 // which takes the queue 32 emissions at a time, the rest when its tiles are done, and goes through the rest of the step
 // with them, so an emission is not issued for one or two lanes of every third tile (the same job 87 us a call at 5 x 2 without the queue).
 template <int G, int F, bool kOne>
-__global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pair_stream(TablesDev t, BatchDevT<float> b,
+__global__ void __launch_bounds__(kStreamThreads, (StreamShape<F, kOne>::kCtas)) k_step_pair_stream(TablesDev t, BatchDevT<float> b,
                                                                                          int steps) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ StreamQueue s_queue[kOne ? kStreamThreads / 32 : 1];
+    constexpr bool kQueue = StreamShape<F, kOne>::kQueue;
+    constexpr int kStages = StreamShape<F, kOne>::kStages;
+    __shared__ StreamQueue s_queue[kQueue ? kStreamThreads / 32 : 1];
     const PairShared S(smem, t.n_eta);
     // the stages on a 16-byte boundary after the tables
     const uint32_t table_bytes = kPairFixedBytes + 4 * (t.n_eta + t.n_E);
@@ -1187,7 +1200,7 @@ __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pai
     const float* sig_z = S.sig;
     const uint32_t n0 = (uint32_t)r.step0;
     const int lane = threadIdx.x & 31;
-    StreamQueue& W = s_queue[kOne ? threadIdx.x >> 5 : 0];
+    StreamQueue& W = s_queue[kQueue ? threadIdx.x >> 5 : 0];
     int queued = 0;                                     // pairs in W (the same on every lane)
     float2 n_above = P2(0.0f);
     // the rest of the step after the optical depth, and the pair back to memory
@@ -1221,18 +1234,18 @@ __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pai
     // the copies of tiles k + 1 .. k + S - 1 are in flight while tile k is stepped
     const int64_t j0 = (int64_t)blockIdx.x * kStreamThreads + threadIdx.x;
 #pragma unroll
-    for (int k = 0; k < kStreamStages - 1; ++k) {
+    for (int k = 0; k < kStages - 1; ++k) {
         const int64_t jk = j0 + k * stride;
         if (jk < n_pairs) stage_issue<F>(r, jk, stage_slots(stage_buf + k * kStageBytes<F>, threadIdx.x));
         cp_async_commit();
     }
     int stage = 0;
     for (int64_t j = j0; j - threadIdx.x < n_tiles * kStreamThreads; j += stride) {
-        const int64_t jn = j + (kStreamStages - 1) * stride;
-        const int sn = stage == 0 ? kStreamStages - 1 : stage - 1;       // (stage + S - 1) mod S
+        const int64_t jn = j + (kStages - 1) * stride;
+        const int sn = stage == 0 ? kStages - 1 : stage - 1;       // (stage + S - 1) mod S
         if (jn < n_pairs) stage_issue<F>(r, jn, stage_slots(stage_buf + sn * kStageBytes<F>, threadIdx.x));
         cp_async_commit();
-        cp_async_wait<kStreamStages - 1>();             // this thread's copies of the current tile
+        cp_async_wait<kStages - 1>();             // this thread's copies of the current tile
         Pair Q;
         const bool full = j < n_pairs;
         if (full) {
@@ -1241,7 +1254,7 @@ __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pai
             pair_clear(Q);
             if (2 * j < r.n) load_one(r, 2 * j, Q, 0, S.tally);   // the odd last electron
         }
-        if constexpr (kOne) {
+        if constexpr (kQueue) {
             unsigned crossed = 0;
             float2 gamma, inv_g, eta;
             const bool act = full && (Q.act[0] || Q.act[1]);
@@ -1268,10 +1281,10 @@ __global__ void __launch_bounds__(kStreamThreads, PE_STREAM_MIN_CTAS) k_step_pai
             pair_loop<G, F, false, true>(t, r, S.h, sig_z, 2 * j, 2 * j + 1, Q, steps, acc, S.tally);
             pair_store(r, j, Q, live0 && Q.act[0], live1 && Q.act[1]);
         }
-        stage = stage + 1 == kStreamStages ? 0 : stage + 1;
+        stage = stage + 1 == kStages ? 0 : stage + 1;
     }
     cp_async_wait<0>();
-    if constexpr (kOne) {
+    if constexpr (kQueue) {
         if (queued) drain(queued);
         const unsigned int na = __float2uint_rz(n_above.x) + __float2uint_rz(n_above.y);
         if (na) atomicAdd(S.tally + PE_T_N_ETA_ABOVE, (unsigned long long)na);
