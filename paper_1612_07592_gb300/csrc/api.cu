@@ -673,6 +673,7 @@ static pe_status build_plan(pe_run* const* runs, int n_runs, int64_t n_steps, co
                 L.bf.reset(new BatchDevT<float>());
                 std::memset(L.bf.get(), 0, sizeof(BatchDevT<float>));
                 L.bf->n_runs = m;
+                L.bf->sig_stride = pair_sig_stride(t->dev);
                 L.bf->tile = block;
                 for (int k = 0; k <= m; ++k) L.bf->tile_start[k] = tile_start[k];
                 for (int k = 0; k < m; ++k) L.bf->runs[k] = to_float(runs[idx[k]]->dev);

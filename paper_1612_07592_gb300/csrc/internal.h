@@ -125,6 +125,7 @@ template <typename R>
 struct BatchDevT {
     int n_runs;
     int tile;                           // particles per tile
+    int sig_stride;                     // FP32: n_E if every row of sigma_Z is in shared memory, 0 if the run's alone
     int each_step;                      // FP64: non-finite momenta are looked for before every step, not every launch
     int64_t tile_start[PE_MAX_BATCH + 1];
     RunDevT<R> runs[PE_MAX_BATCH];
@@ -209,6 +210,7 @@ void launch_step_persistent_f64(const TablesDev& t, const BatchDevT<double>& b, 
                                 cudaStream_t s);
 size_t rate_table_bytes(const TablesDev& t, int precision);       // h(eta) and sigma_Z(gamma)
 int pair_smem_bytes(const TablesDev& t);                          // the paired FP32 kernels
+int pair_sig_stride(const TablesDev& t);
 int default_ctas_per_sm_f32(const BatchDevT<float>& b, int steps, int block, int base_smem);
 const void* persistent_kernel_f32(const BatchDevT<float>& b, int steps, int smem, int block, int* threads,
                                   int* smem_out);

@@ -14,7 +14,11 @@ namespace pe {
 // of a plane-wave kind use the streaming form of the paired kernel.
 constexpr int kStreamMaxSteps = 4;
 
-int pair_smem_bytes(const TablesDev& t) { return kPairFixedBytes + 4 * (t.n_eta + t.n_E); }   // 54 KB at most (4096 rows)
+// The rows of sigma_Z in shared memory: all of them up to 8 KB, where they cost no resident CTA; above that the run's own.
+int pair_sig_stride(const TablesDev& t) { return t.n_Z * t.n_E <= 2048 ? t.n_E : 0; }
+int pair_smem_bytes(const TablesDev& t) {                            // 54 KB at most (tables of up to 4096 rows)
+    return kPairFixedBytes + 4 * (t.n_eta + (pair_sig_stride(t) ? t.n_Z * t.n_E : t.n_E));
+}
 
 static bool plane_kind(int fk) { return fk == FK_PLANE_LP || fk == FK_PLANE_CP; }
 // tables, then 16-byte alignment slack and the stage buffers

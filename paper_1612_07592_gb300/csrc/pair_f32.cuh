@@ -846,9 +846,9 @@ __device__ __forceinline__ void pair_clear(Pair& Q) {
 }
 
 // Shared memory of the paired kernels: the CTA's sums and the held lanes' slots (kPairFixedBytes, a multiple of 16
-// bytes), then h(eta) and sigma_Z(gamma) of the run's Z alone (a batch copies the row again when it comes to another run).
-// Rate tables of 2 / 20 / 36 / 100 KB (n_E = 256 / 2048 / 4000 / 4000 rows of 2 / 2 / 2 / 6 Z), 2e5 electrons x 300 steps:
-// 0.54 / 0.65 / 0.67 / 1.54 ms with every row copied, 0.54 / 0.55 / 0.65 / 0.65 so.
+// bytes), then h(eta) and sigma_Z(gamma): every row of a small set, otherwise that of the run's Z alone (a batch copies the
+// row again when it comes to another run).  Rate tables of 2 / 20 / 36 / 100 KB (n_E = 256 / 2048 / 4000 / 4000 rows of
+// 2 / 2 / 2 / 6 Z), 2e5 electrons x 300 steps: 0.54 / 0.65 / 0.67 / 1.54 ms with every row copied, 0.54 / 0.55 / 0.65 / 0.65 so.
 constexpr int kPairFixedBytes = kSumsThreads * (16 * kEnergySums + 3 * 8) + 8 * PE_TALLY_WORDS + 4 * PE_HIST_WORDS +
                                 4 * PE_T_E_NCS_STORED;
 static_assert(kPairFixedBytes % 16 == 0, "tables after a 16-byte boundary");
@@ -874,10 +874,12 @@ struct PairShared {
 #pragma unroll 4
         for (int k = threadIdx.x; k < t.n_eta; k += blockDim.x) h[k] = t.h32[k];
     }
-    __device__ __forceinline__ void load_sigma(const TablesDev& t, int iz) const {
-        const float* row = t.sig32 + (size_t)iz * t.n_E;
+    // row iz alone (stride 0) or all rows
+    __device__ __forceinline__ void load_sigma(const TablesDev& t, int stride, int iz) const {
+        const float* rows = t.sig32 + (stride ? 0 : (size_t)iz * t.n_E);
+        const int n = stride ? t.n_Z * t.n_E : t.n_E;
 #pragma unroll 4
-        for (int k = threadIdx.x; k < t.n_E; k += blockDim.x) sig[k] = row[k];
+        for (int k = threadIdx.x; k < n; k += blockDim.x) sig[k] = rows[k];
     }
     __device__ __forceinline__ SumsCta acc() const { return SumsCta{hist, cnt, sums + threadIdx.x}; }
     __device__ __forceinline__ Held slots() const {
@@ -944,11 +946,11 @@ __device__ __forceinline__ void tile_steps_pair(const TablesDev& t, const RunDev
 #define PE_PAIR_MIN_CTAS_REFL 7
 #endif
 // The general instances (flags read at run time: the null-collision method, a process switched off, the box boundary)
-// carry more live state than the others.  2e5 electrons x 400 steps, plane wave without brems / by null collisions /
-// reflected wave by null collisions, and the 1 GeV Au bunch by null collisions (1500 steps at dt = T): 5 CTAs 652 / 785 /
-// 2360 us, 6 587 / 677 / 1844 / 2008, 7 616 / 702 / 1901 / 2240, 8 632 / 742 / 1894 / 2554.
+// carry more live state than the others and spill 250 to 370 bytes at 7 CTAs.  At 6 small runs gain (3e5 electrons, plane
+// wave with a box / by null collisions, 700 steps, the Au bunch by null collisions at dt = T / 10, 2500 steps: 1.99 / 1.60 /
+// 2.86 ms, at 7 2.03 / 1.71 / 2.95), larger ones lose more (1e6 electrons 5.80 / 4.49 / 7.33, at 7 5.44 / 4.41 / 6.64).
 #ifndef PE_PAIR_MIN_CTAS_GENERAL
-#define PE_PAIR_MIN_CTAS_GENERAL 6
+#define PE_PAIR_MIN_CTAS_GENERAL 7
 #endif
 // Brems alone (the bunch by the direct method, 5e5 electrons x 2000 steps): 7 to 9 CTAs 5.73 to 5.78 ms, 10 5.84.
 #ifndef PE_PAIR_MIN_CTAS_BREMS
@@ -969,7 +971,7 @@ __global__ void __launch_bounds__(128, (pair_min_ctas<G, F>())) k_step_pair(Tabl
     __shared__ RunDevT<float> s_run;
     const PairShared S(smem, t.n_eta);
     S.init(t);
-    if (kSingle) S.load_sigma(t, b.runs[0].iz);
+    S.load_sigma(t, b.sig_stride, b.runs[0].iz);
     __syncthreads();
     const SumsCta acc = S.acc();
     const Held held = S.slots();
@@ -987,7 +989,7 @@ __global__ void __launch_bounds__(128, (pair_min_ctas<G, F>())) k_step_pair(Tabl
                 constexpr int kWords = sizeof(RunDevT<float>) / 4;
                 for (int w = threadIdx.x; w < kWords; w += blockDim.x)
                     reinterpret_cast<uint32_t*>(&s_run)[w] = reinterpret_cast<const uint32_t*>(&b.runs[run_idx])[w];
-                S.load_sigma(t, b.runs[run_idx].iz);
+                if (!b.sig_stride) S.load_sigma(t, 0, b.runs[run_idx].iz);
                 __syncthreads();
                 cur = run_idx;
             }
@@ -997,7 +999,7 @@ __global__ void __launch_bounds__(128, (pair_min_ctas<G, F>())) k_step_pair(Tabl
         since += per_tile;
         const int64_t base = (tile - b.tile_start[run_idx]) * b.tile;
         const int64_t i0 = base + threadIdx.x, i1 = base + threadIdx.x + blockDim.x;
-        tile_steps_pair<G, F, kSingle, kHold>(t, r, S.h, S.sig, i0, i1, steps, acc, held, S.tally);
+        tile_steps_pair<G, F, kSingle, kHold>(t, r, S.h, S.sig + (size_t)r.iz * b.sig_stride, i0, i1, steps, acc, held, S.tally);
     }
     if (kSingle) {
         if (n_tiles > 0) S.flush(b.runs[0]);
@@ -1183,11 +1185,11 @@ __global__ void __launch_bounds__(kStreamThreads, (StreamShape<F, kOne>::kCtas))
     __shared__ StreamQueue s_queue[kQueue ? kStreamThreads / 32 : 1];
     const PairShared S(smem, t.n_eta);
     // the stages on a 16-byte boundary after the tables
-    const uint32_t table_bytes = kPairFixedBytes + 4 * (t.n_eta + t.n_E);
+    const uint32_t table_bytes = kPairFixedBytes + 4 * (t.n_eta + (b.sig_stride ? t.n_Z * t.n_E : t.n_E));
     unsigned char* stage_buf = smem + ((table_bytes + 15u) & ~15u);
     const RunDevT<float>& r = b.runs[0];
     S.init(t);
-    S.load_sigma(t, r.iz);
+    S.load_sigma(t, b.sig_stride, r.iz);
     __syncthreads();
     // what follows reads the state: the launch of this kernel may overlap the end of the one before
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1197,7 +1199,7 @@ __global__ void __launch_bounds__(kStreamThreads, (StreamShape<F, kOne>::kCtas))
     const int64_t n_tiles = b.tile_start[1];
     const int64_t n_pairs = r.n >> 1;                   // j < n_pairs: electrons 2j and 2j + 1 both present
     const int64_t stride = (int64_t)gridDim.x * kStreamThreads;
-    const float* sig_z = S.sig;
+    const float* sig_z = S.sig + (size_t)r.iz * b.sig_stride;
     const uint32_t n0 = (uint32_t)r.step0;
     const int lane = threadIdx.x & 31;
     StreamQueue& W = s_queue[kQueue ? threadIdx.x >> 5 : 0];
