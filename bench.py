@@ -8,7 +8,7 @@ One benchmark step = that whole job: all 1e6 electrons advanced through all
 kernel, state in registers across the steps of a launch).
 
 Lines printed (rank 0): one JSON object with the contract keys plus
-  roofline      the dominant kernel (k_step_persistent<float>) against the FP32 pipe
+  roofline      the dominant kernel (k_step_pair) against the FP32 pipe
   roofline_hbm  the one-step-per-launch form on a state larger than L2 against HBM
   fp64_plain    the FP64 path on the same job
   cpu_baseline  the FP64 oracle on the host cores on a bounded sample
@@ -34,10 +34,11 @@ sys.path.insert(0, ROOT)
 METRIC = "emitting particle-steps/s at 1 GB300 (FP32/batched vs FP64 plain); % HBM roofline; p99"
 UNIT = "particle-steps/s"
 # FP32 operations of one particle-step of the headline job, counted by ncu's SASS counters on one
-# launch of the whole job (1e6 electrons x 4000 steps): 2 per FFMA, 4 per FFMA2, 1 per FADD/FMUL,
-# 2 per FADD2/FMUL2, over the 4e9 particle-steps (profiles/k_step_pair__1d-au-a270-mj-1e6x4000__flops.md)
-FLOP_PER_PSTEP_1D = 123.9
-FLOP_COUNT_SOURCE = "ncu SASS counters on the headline launch (FFMA 2, FFMA2 4, FADD/FMUL 1, FADD2/FMUL2 2)"
+# launch of the job with 1e5 of its electrons (x 4000 steps): 2 per FFMA, 4 per FFMA2, 1 per FADD/FMUL,
+# 2 per FADD2/FMUL2, over the 4e8 particle-steps (profiles/k_step_pair__1d-au-a270-mj-1e5x4000__flops.md)
+FLOP_PER_PSTEP_1D = 117.4
+FLOP_COUNT_SOURCE = ("ncu SASS counters on a launch of the headline job with 1e5 electrons "
+                     "(FFMA 2, FFMA2 4, FADD/FMUL 1, FADD2/FMUL2 2)")
 # Algorithmic bytes of one particle-step when the state round-trips memory every step:
 # read + write of x (float pair, 8 B), ux, uy, uz (f32) and tau (float pair, 8 B) in 1D;
 # + y (float pair) in 2D.
@@ -48,24 +49,14 @@ BYTES_PER_PSTEP_2D = 72
 BYTES_PER_PSTEP_1D_PLAIN_X = 48
 FP32_LANES_PER_SM = 128
 # warp instructions per 64 electron-steps of the dominant kernel (one warp steps 64 electrons), from
-# the same ncu capture of the headline launch; the kernel is bound by instruction issue (one warp
-# instruction per scheduler per clock), which the roofline's `issue` entry reports beside the FP32 pipe.
-# Counted before the optical-depth draw's renormalisation below U = 2^-10 entered the emission
-# branch: a compare per emission (2.9e6 per job) and the rare renormalisation, about 2e-3
-# instructions per particle-step, within the count's last digit.
-NCU_WARP_INST_PER_64_ESTEPS = 279.1
+# the same ncu capture; the kernel is bound by instruction issue (one warp instruction per scheduler
+# per clock), which the roofline's `issue` entry reports beside the FP32 pipe.
+NCU_WARP_INST_PER_64_ESTEPS = 250.0
 SCHEDULERS_PER_SM = 4
-# DRAM bytes (read + write) per electron and launch of the dominant kernel, from the same ncu
-# capture of the headline launch (29.1 MB for 1e6 electrons: the state read once, the final state
-# still in L2 at the end, the cold emission tables; profiles/k_step_pair__1d-au-a270-mj-1e6x4000__flops.md:
-# 29.13 B); None once the kernel changes, as it has since (the optical-depth draw of the inlined
-# emission branch), until the next capture.
+# DRAM bytes (read + write) per electron and launch of the dominant kernel, from an ncu capture of the
+# headline launch with 1e6 electrons; None until one is taken of the present kernel.
 NCU_TRAFFIC_BYTES_PER_ELECTRON = None
-# DRAM bytes (read + write) per electron of one launch of the one-step form, from an ncu capture of
-# one launch on 8e6 electrons (386.7 MB: 28 B read, 20.3 B written -- the rest of the 28 B still
-# dirty in L2 when the kernel ends), scaled by the electron count of the measured workload
-# (profiles/k_step_pair_stream__1d-au-a270-mj-8e6-K1__full.md: 48.34 B); None once the kernel
-# changes, as it has since (the same emission branch), until the next capture.
+# The same of one launch of the one-step form, on a state larger than L2.
 NCU_STREAM_TRAFFIC_BYTES_PER_ELECTRON = None
 
 
